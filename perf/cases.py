@@ -83,15 +83,15 @@ def draw(rng):
         c["sx"] = max(2 if kind == "sweep" else 1, min(4, round(n / rng.uniform(5, 9))))
     else:
         # whole solves are small: with the Eq. 7 preconditioner their iteration counts make them long
-        full = c["order"] == 2 and kind in ("sweep", "solve", "grad") and rng.random() < 0.4
+        full = c["order"] == 2 and kind in ("solve", "grad") and rng.random() < 0.4
         lo, hi = {"apply": (12, 256), "sweep": (12, 160), "setup": (12, 256), "solve": (8, 20), "grad": (6, 12)}[kind]
-        if full and kind != "sweep":
+        if full:
             hi *= 4
         c["nx"] = _log_int(rng, lo, hi)
         c["ny"] = max(lo, c["nx"] - rng.randint(0, 9))
         c["sx"] = max(2 if kind == "sweep" else 1, min(8, round(c["nx"] / rng.uniform(14, 34))))
         if full:
-            c.update(precond="full", relax=1 if kind != "sweep" else 0)
+            c.update(precond="full", relax=1)
         elif kind == "sweep" and rng.random() < 0.3:
             c.update(order=1, sx=0, nx=rng.randint(24, 96), ny=0, problems=rng.randint(5, 24))
     # phase per cell: from coarse lowest-order (6 cells per wavelength) to well resolved
