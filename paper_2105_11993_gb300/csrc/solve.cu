@@ -1563,8 +1563,7 @@ void apply_local(thm_sys* s, int op, int mode, const double2* x, double2* y) {
 int sweep_diag(thm_sys* s, const thm_solve_opts* opts, int with_sources, const double2* g_in, double2* g_out,
                double2* uloc, thm_stats* stats) {
     SolveCfg c = make_cfg(opts);
-    ensure_factor(s, c.fp32);
-    ensure_work(s, c.fp32, c.m_in, c.m_out);
+    prepare(s, c);
     RunStats rs;
     sweep(s, c, with_sources ? s->f_loc.p : nullptr, g_in, g_out, uloc, rs, with_sources ? s->uD.p : nullptr);
     THM_CUDA(cudaStreamSynchronize(s->st));
