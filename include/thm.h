@@ -72,9 +72,9 @@ typedef struct thm_sys thm_sys;     /* opaque: assembled operators + preconditio
  *  bfaces       host int64  [n_bface][2 | 4]: boundary faces (2-D: the edge's two
  *               vertices; 3-D: the quad's four vertices in tensor order).
  *  btag         host uint8  [n_bface]: THM_TAG_*.
- *  max_block    largest block of the level-block-tridiagonal factorisation of
- *               P_i (<= 0: library default); 0 < max_block sets the trade-off
- *               between sequential depth and bytes of the preconditioner.
+ *  max_block    largest level block of the local order (edge DOFs of a subdomain
+ *               by merged BFS levels; <= 0: library default).  The factorisation
+ *               of P_i has an order of its own and does not depend on it.
  *
  *  Numbering (bit-exact contract): edges are the distinct vertex pairs of the
  *  cells' local edges, numbered in lexicographic order of (min id, max id);
@@ -375,11 +375,11 @@ int thm_dirichlet_values(thm_sys* s, double* u_d);
  * overhead and not counted):
  *   THM_K_SPMV: nnz(P_i) values + 2 diagonal face terms per row
  *               + x read + y written (complex vectors)
- *   THM_K_PINV: the inverse blocks W_l of the forward sweeps and the middle
- *               level (sum_l m_l^2 per subdomain), the backward-sweep blocks
- *               H_l = W_l F_l resp. W_l E_l (sum_{l != k} m_l m_{l+-1}), the
- *               level coupling values of the forward and middle steps, the
- *               order-2 condensation tables, x read + y written
+ *   THM_K_PINV: the factor values a solve multiplies by, sum over the nodes of
+ *               the subdomains' elimination trees of s^2 + 2 s b (s unknowns
+ *               eliminated at the node, b unknowns of its ancestors that it
+ *               couples to: the inverse block once, the coupling block on the
+ *               way up and on the way down), x read + y written
  * Other classes: THM_EINVAL. */
 int thm_alg_bytes(const thm_sys* s, int mode, int cls, double* bytes);
 
@@ -428,12 +428,10 @@ int thm_work_bytes(const thm_sys* s, int mode, int cls, double* bytes);
  * ------------------------------------------------------------------------ */
 int thm_residual_noalloc(const thm_sys* s, const double* u, double* out);
 
-/* Bytes of the stored preconditioner factors (the dense inverse blocks W_l of
- * the twisted block factorisation and the backward-sweep blocks H_l^T =
- * (W_l F_l)^T resp. (W_l E_l)^T of every level but the middle one, row strides
- * padded to 4 entries) for precond THM_PRECOND_* in mode
- * THM_MODE_*: real values for Eq. 7, complex ones for the full 2x2 block
- * operator.  From the sizes alone (nothing is factorised by this call). */
+/* Bytes of the stored preconditioner factors (the dense blocks of every node of
+ * the subdomains' elimination trees, in slices of 32 rows padded to the widest
+ * of their rows) for precond THM_PRECOND_* in mode THM_MODE_*: real values for
+ * Eq. 7, complex ones for the full 2x2 block operator.  From the sizes alone (nothing is factorised by this call). */
 int thm_factor_bytes(const thm_sys* s, int precond, int mode, double* bytes);
 
 /* Kernel launches issued by this library since the process started. */

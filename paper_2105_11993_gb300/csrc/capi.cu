@@ -417,14 +417,10 @@ int thm_alg_bytes(const thm_sys* s, int mode, int cls, double* bytes) {
             for (uint8_t p : m->sell_pad) nnz += !p;
             *bytes = nnz * bv + 2.0 * m->n_loc * bv + 2.0 * m->n_loc * bx;
         } else if (cls == THM_K_PINV) {
-            double w = 0, ne = 0, nb = 0;
-            for (const auto& S : m->subs) {
-                w += (double)bt_stream_values(S, m->levels.data());
-                ne += (double)S.ne;
-                nb += (double)(S.n - S.ne);
-            }
-            double tab = m->order == 2 ? (8 * ne + 12 * nb) : 0;
-            *bytes = (w + tab) * bv + 2.0 * m->n_loc * bx;
+            require_nd(m);
+            double w = 0;
+            for (int64_t v : m->nd.welem) w += (double)v;
+            *bytes = w * bv + 2.0 * m->n_loc * bx;
         } else {
             fail(THM_EINVAL, "no byte model for this kernel class");
         }
@@ -469,7 +465,8 @@ int thm_factor_bytes(const thm_sys* s, int precond, int mode, double* bytes) {
         THM_REQUIRE(s && bytes, "NULL argument");
         THM_REQUIRE(precond == THM_PRECOND_BLOCKDIAG || precond == THM_PRECOND_FULL, "unknown preconditioner");
         const double bv = mode == THM_MODE_MIXED ? 4.0 : 8.0;
-        *bytes = (double)s->m->fac_elems * bv * (precond == THM_PRECOND_FULL ? 2.0 : 1.0);
+        require_nd(s->m);
+        *bytes = (double)s->m->nd.fac_elems * bv * (precond == THM_PRECOND_FULL ? 2.0 : 1.0);
         return THM_OK;
     });
 }

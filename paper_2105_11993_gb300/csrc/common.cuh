@@ -7,6 +7,7 @@
 #include <string>
 #include <vector>
 
+#include "nd.cuh"
 #include "thm.h"
 
 namespace thm {
@@ -84,49 +85,11 @@ void prof_read(int cls, int64_t* launches, double* ms);
 constexpr int SELL_C = 32;       // rows per SELL slice (one warp)
 constexpr int CHUNK = 1024;      // elements per reduction chunk of a segment
 
-// One block of the level-block-tridiagonal factorisation of P_i.
-struct Level {
-    int32_t start;    // first local row (absolute index into local vectors)
-    int32_t size;     // m_l
-    int32_t prev;     // m_{l-1} (0 for the first level of a subdomain)
-    int32_t next;     // m_{l+1} (0 for the last)
-    int64_t offW;     // W_l = S_l^{-1}: m_l rows of stride r4(m_l) (16-byte aligned)
-    int64_t offH;     // H_l^T, the backward-sweep product (l != kmid): H_l = W_l F_l above the
-                      // middle level, W_l E_l below it; m_{l+1} resp. m_{l-1} rows of stride
-                      // r4(m_l), or -1 (16-byte aligned)
-    // coupling blocks of S to level l-1 (E) and l+1 (F): m_l+1 row pointers
-    // (0-based, at cpl_ptr[eptr..]) and nz (column local to the neighbour
-    // level, value) entries at cpl_col/cpl_val[eoff..]; offsets 16-byte aligned
-    int64_t eptr, eoff, fptr, foff;
-    int32_t enz, fnz;
-};
-
 struct Sub {
     int64_t off;      // first local row
     int64_t n;        // free DOFs
     int64_t ne;       // free edge DOFs (rows off .. off+ne-1); cell bubbles follow
-    int32_t lev0;     // first level
-    int32_t nlev;
-    int32_t kmid;     // middle level of the twisted factorisation (0 <= kmid < nlev)
-    int32_t cell0;    // order 2: slot of the first bubble cell (rows off+ne.. in groups of 4) in thm_sys::tab_e8
 };
-
-// Values one block solve streams for subdomain S (the byte model of the
-// block-solve kernel, in values): W_l once for every level (forward steps and
-// the middle level), H_l for every level but the middle (backward steps),
-// and the coupling lists of the forward and middle steps (E_1..E_k of the top
-// chain, F_k..F_{L-2} of the bottom one).
-inline int64_t bt_stream_values(const Sub& S, const Level* lv) {
-    int64_t w = 0;
-    for (int l = 0; l < S.nlev; ++l) {
-        const Level& L = lv[S.lev0 + l];
-        w += (int64_t)L.size * L.size;
-        if (l != S.kmid) w += (int64_t)L.size * (l < S.kmid ? L.next : L.prev);
-        if (l >= 1 && l <= S.kmid) w += L.enz;
-        if (l >= S.kmid && l + 1 < S.nlev) w += L.fnz;
-    }
-    return w;
-}
 
 // A contiguous piece of one segment, used for deterministic segmented reductions.
 struct Chunk {
@@ -157,7 +120,6 @@ struct thm_mesh {
 
     // local (per-subdomain, free DOFs) structure
     int64_t n_loc = 0;
-    int64_t n_bcell = 0;                            // order 2: cells (bubble groups) over all subdomains
     std::vector<thm::Sub> subs;
     std::vector<int64_t> loc_gdof;                  // [n_loc]
     std::vector<int32_t> loc_sub;                   // [n_loc]
@@ -188,25 +150,19 @@ struct thm_mesh {
     std::vector<int32_t> face_loc;                  // [n_face][2][fd] local rows per side (-1: Dirichlet)
     std::vector<int32_t> row_face;                  // [n_loc][RF] face ids (-1: none)
     std::vector<int8_t> row_face_a, row_face_side;  // [n_loc][RF]
-    // levels of the block-tridiagonal factorisation
-    std::vector<thm::Level> levels;
-    int max_m = 0;
-    int max_lev = 0;                                // most levels of a subdomain
-    int64_t bt_nvec = 0;                            // longest half-chain vector of the twisted solve
-    std::vector<int64_t> bt_welem;                  // [n_sub] values one block solve reads (W, couplings, tables)
-    thm::DArr<int64_t> d_bt_welem;
-    int64_t fac_elems = 0;
-    // W-tile size of the block-solve kernel picked by its autotuner ([0] FP64
-    // factors, [1] FP32), 0 until the first apply of a system on this mesh.
-    // The factor layout (levels, block sizes) is the mesh's, so every system
-    // assembled on the mesh reuses the choice.
-    mutable size_t bt_tile[4] = {0, 0, 0, 0};    // [2], [3]: complex factors (full-block preconditioner)
-    // level couplings of S as compact CSR lists (columns local to the
-    // neighbouring level; slot = position of the value in the SELL arrays)
-    std::vector<int32_t> cpl_ptr, cpl_col;
-    std::vector<int64_t> cpl_slot;                  // -1 for alignment padding
-    int max_cnz = 0;                                // largest coupling block
-    int64_t max_ne = 0;                             // largest number of edge DOFs of a subdomain
+    // elimination trees of the subdomains (the block preconditioner's factorisation)
+    thm::NdHost nd;
+    bool nd_ok = false;                             // false: a subdomain outgrows the solve kernel
+    struct {
+        thm::DArr<thm::NdPart> parts;
+        thm::DArr<thm::NdLev> levs;
+        thm::DArr<int2> slt;
+        thm::DArr<uint32_t> rowd, rowm, ymap, rmap;
+        thm::DArr<uint16_t> idx;
+        thm::DArr<int32_t> perm, rows, cmap, childs;
+        thm::DArr<int64_t> welem;
+        thm::DArr<thm::NdNode> nodes;
+    } ndd;
     // reduction chunks over subdomains
     std::vector<thm::Chunk> chunks;
     // interface entries (directed pairs i <- j, one per free DOF on Sigma_ij)
@@ -232,7 +188,6 @@ struct thm_mesh {
     std::vector<int64_t> copy_ptr;                  // [n_dof+1]
     std::vector<int32_t> copy_idx;
     std::vector<uint8_t> loc_is_owner;              // [n_loc]
-    std::vector<uint8_t> loc_is_bub;                // [n_loc] order-2 cell bubble
 
     // device mirrors
     thm::DArr<double> d_coords;
@@ -241,13 +196,10 @@ struct thm_mesh {
     thm::DArr<int64_t> d_edge_lo, d_edge_hi, d_slice_ptr, d_dir_edges, d_loc_gdof, d_rowg_ptr,
         d_copy_ptr;
     thm::DArr<int8_t> d_cell_signs, d_face_sgn, d_face_kind, d_row_face_a, d_row_face_side, d_if_ta, d_if_tb;
-    thm::DArr<uint8_t> d_sell_pad, d_loc_is_owner, d_loc_is_bub;
+    thm::DArr<uint8_t> d_sell_pad, d_loc_is_owner;
     thm::DArr<int32_t> d_if_rowi, d_if_partner, d_rowg_idx, d_owner_loc, d_copy_idx, d_loc_sub, d_face_v,
         d_face_dof, d_face_loc, d_row_face, d_if_tf, d_if_tcol;
     thm::DArr<int64_t> d_if_ptr;
-    thm::DArr<thm::Level> d_levels;
-    thm::DArr<int32_t> d_cpl_ptr, d_cpl_col;
-    thm::DArr<int64_t> d_cpl_slot;
     thm::DArr<thm::Sub> d_subs;
     thm::DArr<thm::Chunk> d_chunks;
     thm::DArr<thm::Chunk> d_dof_chunks;
@@ -292,7 +244,7 @@ struct thm_sys {
     thm::DArr<double2> dir_vals;
     thm::DArr<double2> f_loc;          // [n_loc] subdomain sources: -(T_i)_{F,D} u_D (Eq. 5)
     thm::DArr<double2> f_res;          // [n_loc] split of the global right-hand side: -(K_i^loc)_{F,D} u_D
-    // block-tridiagonal factors of P_i (lazily built per precision)
+    // factors of P_i over the elimination trees (lazily built per precision)
     bool fac64_ok = false, fac32_ok = false;
     thm::DArr<double> fac64;
     thm::DArr<float> fac32;
@@ -301,25 +253,9 @@ struct thm_sys {
     bool facc64_ok = false, facc32_ok = false;
     thm::DArr<double2> facc64;
     thm::DArr<float2> facc32;
-    // static condensation of order-2 cell bubbles: S = P_EE - P_EI D^{-1} P_IE
-    thm::DArr<double> sval64;          // SELL values of S on edge rows/columns (P elsewhere 0)
-    thm::DArr<float> sval32;
-    thm::DArr<double> cinv64, cg64;    // per cell: D_II^{-1} (4x4), G = P_EI D_II^{-1} (8x4)
-    thm::DArr<float> cinv32, cg32;
     thm::DArr<int> dev_err;            // set by a device-side bounded wait that gave up
-    thm::DArr<double> cpl64;           // values of the level coupling lists
-    thm::DArr<float> cpl32;
-    // order-2 gather tables (structure of arrays, [8][n_loc]): for an edge row
-    // the <= 8 (bubble, G entry) pairs of r_E - G r_I; for a bubble row the 4
-    // (bubble, D^{-1} entry) and 8 (edge, -G entry) pairs of D^{-1} r_I - G^T x_E.
-    // The bubbles of a cell are 4 consecutive local rows, so the indices are
-    // not stored per entry: tab_ab [2][n_loc] holds an edge row's (<= 2) cells'
-    // first bubble rows (-1: none; entry u*4+k of av belongs to bubble ab[u]+k),
-    // tab_e8 [bubble cells][8] a cell's 8 edge rows (-1: Dirichlet), the cell of
-    // bubble row b being slot subs.cell0 + (b - off - ne) / 4
-    thm::DArr<int32_t> tab_ab, tab_e8;
-    thm::DArr<double> tab_av64, tab_cv64, tab_ev64;
-    thm::DArr<float> tab_av32, tab_cv32, tab_ev32;
+    // workspace of the solve kernel for subdomains whose vectors outgrow shared memory
+    mutable thm::DArr<double2> nd_glob;
     // block-solve work actually done, per factor precision ([0..1] FP64, [2..3]
     // FP32): values read and local rows processed, summed by the kernel over
     // the subdomains it did not skip
@@ -334,6 +270,9 @@ struct thm_sys {
 
 namespace thm {
 void build_mesh(thm_mesh* m);
+void build_nd(thm_mesh* m);
+void require_nd(const thm_mesh* m);
+NdTables nd_tables(const thm_mesh* m);
 void assemble(thm_sys* s);
 void ensure_factor(thm_sys* s, bool fp32);
 void ensure_factor_full(thm_sys* s, bool fp32);

@@ -411,8 +411,6 @@ void build_mesh(thm_mesh* m) {
     m->subs.resize(ns);
     m->loc_gdof.clear();
     m->loc_sub.clear();
-    m->levels.clear();
-    m->n_bcell = 0;
     std::vector<std::vector<int32_t>> row_cols_all;   // per local row: sorted local columns
     m->maxc = d == 2 ? 2 : 4;
     std::vector<int32_t> row_cell_v, row_k_v;
@@ -454,8 +452,7 @@ void build_mesh(thm_mesh* m) {
             std::sort(v.begin(), v.end());
             v.erase(std::unique(v.begin(), v.end()), v.end());
         }
-        // Order-2 cell bubbles are condensed cell by cell and ordered last;
-        // the block-tridiagonal levels cover the edge DOFs only.
+        // local order: order-2 cell bubbles last, the edge DOFs by BFS levels
         std::vector<uint8_t> bub(n, 0);
         int64_t nbub = 0;
         if (m->order == 2)
@@ -514,18 +511,6 @@ void build_mesh(thm_mesh* m) {
         m->subs[s].n = n;
         m->subs[s].ne = n - nbub;
         THM_REQUIRE(nbub % 4 == 0, "internal: order-2 bubbles not in groups of 4");
-        m->subs[s].cell0 = (int32_t)m->n_bcell;
-        m->n_bcell += nbub / 4;
-        m->subs[s].lev0 = (int32_t)m->levels.size();
-        m->subs[s].nlev = (int32_t)bsize.size();
-        int32_t st = (int32_t)off;
-        for (size_t b = 0; b < bsize.size(); ++b) {
-            Level L{};
-            L.start = st;
-            L.size = (int32_t)bsize[b];
-            st += L.size;
-            m->levels.push_back(L);
-        }
         for (int64_t i = 0; i < n; ++i) {
             int64_t o = order[i];
             m->loc_gdof.push_back(gd[o]);
@@ -552,62 +537,6 @@ void build_mesh(thm_mesh* m) {
     m->n_loc = off;
     m->row_cell.swap(row_cell_v);
     m->row_k.swap(row_k_v);
-
-    // ---- level offsets into the factor storage (rows padded to a multiple
-    //      of 4 entries, so every row and every block is 16-byte aligned) and
-    //      the middle level of the twisted factorisation: the level that
-    //      balances the factor bytes (plus a per-level latency allowance) of
-    //      the two chains
-    m->max_m = 0;
-    m->max_lev = 0;
-    m->bt_nvec = 0;
-    int64_t fo = 0;
-    for (int s = 0; s < ns; ++s) {
-        auto& S = m->subs[s];
-        m->max_lev = std::max(m->max_lev, S.nlev);
-        std::vector<double> cost(S.nlev);
-        for (int l = 0; l < S.nlev; ++l) {
-            Level& L = m->levels[S.lev0 + l];
-            L.prev = l > 0 ? m->levels[S.lev0 + l - 1].size : 0;
-            L.next = l + 1 < S.nlev ? m->levels[S.lev0 + l + 1].size : 0;
-            m->max_m = std::max(m->max_m, L.size);
-            L.offW = fo;
-            fo += (int64_t)L.size * (((int64_t)L.size + 3) / 4 * 4);
-            cost[l] = (double)L.size * L.size + 16384.0;
-        }
-        S.kmid = 0;
-        if (S.nlev > 0) {
-            double tot = 0, below = 0, best = 1e300;
-            for (double c : cost) tot += c;
-            for (int k = 0; k < S.nlev; ++k) {
-                const double above = tot - below - cost[k];
-                const double w = std::max(below, above);
-                if (w < best) { best = w; S.kmid = k; }
-                below += cost[k];
-            }
-            const Level& Lk = m->levels[S.lev0 + S.kmid];
-            const Level& L0 = m->levels[S.lev0];
-            const Level& Le = m->levels[S.lev0 + S.nlev - 1];
-            m->bt_nvec = std::max<int64_t>(m->bt_nvec, (int64_t)Lk.start + Lk.size - L0.start);
-            m->bt_nvec = std::max<int64_t>(m->bt_nvec, (int64_t)Le.start + Le.size - Lk.start);
-        }
-    }
-    // H_l^T after all W blocks: rows of the level the backward sweep comes
-    // from (l + 1 above the middle, l - 1 below it), stride r4(m_l)
-    for (int s = 0; s < ns; ++s) {
-        const auto& S = m->subs[s];
-        for (int l = 0; l < S.nlev; ++l) {
-            Level& L = m->levels[S.lev0 + l];
-            if (l == S.kmid) {
-                L.offH = -1;
-                continue;
-            }
-            const int nb = l < S.kmid ? L.next : L.prev;
-            L.offH = fo;
-            fo += (int64_t)nb * (((int64_t)L.size + 3) / 4 * 4);
-        }
-    }
-    m->fac_elems = fo + 4;
 
     // ---- SELL-32 pattern
     m->n_slices = (m->n_loc + SELL_C - 1) / SELL_C;
@@ -655,61 +584,6 @@ void build_mesh(thm_mesh* m) {
             }
         }
     }
-    // ---- level coupling lists: for every level row, its S entries in the
-    //      previous level (E_l) and in the next level (F_l), one 16-byte
-    //      aligned block per (level, side)
-    m->cpl_ptr.clear(); m->cpl_col.clear(); m->cpl_slot.clear();
-    m->max_cnz = 0;
-    m->max_ne = 0;
-    auto pad4i = [](std::vector<int32_t>& v) { while (v.size() % 4) v.push_back(0); };
-    for (int s = 0; s < ns; ++s) {
-        const auto& S = m->subs[s];
-        m->max_ne = std::max<int64_t>(m->max_ne, S.ne);
-        for (int l = 0; l < S.nlev; ++l) {
-            Level& L = m->levels[S.lev0 + l];
-            for (int side = 0; side < 2; ++side) {
-                int64_t c0 = side == 0 ? (int64_t)L.start - L.prev : (int64_t)L.start + L.size;
-                int64_t c1 = side == 0 ? (int64_t)L.start : c0 + L.next;
-                pad4i(m->cpl_ptr);
-                while (m->cpl_col.size() % 4) { m->cpl_col.push_back(0); m->cpl_slot.push_back(-1); }
-                int64_t p0 = (int64_t)m->cpl_ptr.size(), q0 = (int64_t)m->cpl_col.size();
-                for (int i = 0; i <= L.size; ++i) {
-                    m->cpl_ptr.push_back((int32_t)(m->cpl_col.size() - q0));
-                    if (i == L.size) break;
-                    int64_t r = L.start + i;
-                    int64_t sl = r / SELL_C;
-                    int lane = (int)(r % SELL_C);
-                    int64_t w = (m->slice_ptr[sl + 1] - m->slice_ptr[sl]) / SELL_C;
-                    for (int64_t t = 0; t < w; ++t) {
-                        int64_t idx = m->slice_ptr[sl] + t * SELL_C + lane;
-                        if (m->sell_pad[idx]) continue;
-                        int64_t c = m->sell_col[idx];
-                        if (c >= c0 && c < c1) {
-                            m->cpl_col.push_back((int32_t)(c - c0));
-                            m->cpl_slot.push_back(idx);
-                        }
-                    }
-                }
-                int32_t nz = (int32_t)(m->cpl_col.size() - q0);
-                m->max_cnz = std::max(m->max_cnz, nz);
-                if (side == 0) { L.eptr = p0; L.eoff = q0; L.enz = nz; }
-                else { L.fptr = p0; L.foff = q0; L.fnz = nz; }
-            }
-        }
-    }
-    pad4i(m->cpl_ptr);
-    for (int k = 0; k < 8; ++k) { m->cpl_ptr.push_back(0); m->cpl_col.push_back(0); m->cpl_slot.push_back(-1); }
-    // values one block solve reads per subdomain (the byte model of the
-    // block-solve kernel): the factor blocks and coupling lists it streams,
-    // and the order-2 condensation tables
-    m->bt_welem.assign(ns, 0);
-    for (int s = 0; s < ns; ++s) {
-        const auto& S = m->subs[s];
-        int64_t w = bt_stream_values(S, m->levels.data());
-        if (m->order == 2) w += 8 * S.ne + 12 * (S.n - S.ne);
-        m->bt_welem[s] = w;
-    }
-    THM_REQUIRE(m->cpl_col.size() < (size_t)INT32_MAX, "coupling lists too large");
     row_cols_all.clear();
 
     // ---- reduction chunks
@@ -941,12 +815,7 @@ void build_mesh(thm_mesh* m) {
     m->d_if_ta.upload(m->if_ta);
     m->d_if_tb.upload(m->if_tb);
     m->d_if_tcol.upload(m->if_tcol);
-    m->d_levels.upload(m->levels);
-    m->d_cpl_ptr.upload(m->cpl_ptr);
-    m->d_cpl_col.upload(m->cpl_col);
-    m->d_cpl_slot.upload(m->cpl_slot);
     m->d_subs.upload(m->subs);
-    m->d_bt_welem.upload(m->bt_welem);
     m->d_chunks.upload(m->chunks);
     m->d_dir_edges.upload(m->dir_edges);
     m->dir_dofs.clear();
@@ -963,10 +832,7 @@ void build_mesh(thm_mesh* m) {
     m->d_copy_ptr.upload(m->copy_ptr);
     m->d_copy_idx.upload(m->copy_idx);
     m->d_loc_is_owner.upload(m->loc_is_owner);
-    m->loc_is_bub.assign(m->n_loc, 0);
-    if (m->order == 2)
-        for (int64_t r = 0; r < m->n_loc; ++r) m->loc_is_bub[r] = m->loc_gdof[r] >= 2 * m->n_edge;
-    m->d_loc_is_bub.upload(m->loc_is_bub);
+    build_nd(m);
     THM_CUDA(cudaDeviceSynchronize());
 }
 

@@ -7,10 +7,11 @@
 #include <cstdio>
 #include <cstdlib>
 #include <functional>
+#include <mutex>
 #include <string>
 
-#include "btsolve.cuh"
 #include "kernels.cuh"
+#include "ndsolve.cuh"
 #include "solver.cuh"
 
 namespace thm {
@@ -1103,142 +1104,69 @@ static void apply_T(const thm_sys* s, const F* val, const F* bg, const F* bs, in
                        m->d_loc_sub.p, act, work)));
 }
 
-// Twisted block-tridiagonal solve, one 2-CTA cluster per subdomain.  The
-// coupling blocks get a small ring of their own; the W ring takes what the
-// rest of the layout leaves: tiles of about `target` bytes (fewer, larger bulk
-// copies stream faster per SM, more slots reach further ahead), 2..16 slots.
-struct BtCfg {
-    int rows = 0, ns = 0, cglob = 0, nvec = 0;
-    size_t slot = 0, cslot = 0, smem = 0;
-};
-
-template <class V, class F, class FW = F>
-static BtCfg bt_config(const thm_mesh* m, size_t target) {
-    BtCfg c;
-    const size_t cap = 227 * 1024 - 256;
-    const size_t row_bytes = (size_t)bt_r4(m->max_m) * sizeof(FW);
-    const size_t cfull = bt_r16((size_t)(m->max_m + 1) * 4) + bt_r16((size_t)m->max_cnz * 4) +
-                         bt_r16((size_t)m->max_cnz * sizeof(F));
-    // coupling blocks larger than 12 KB are read from global memory in place
-    // (THM_BT_CPL_GLOBAL=1 forces that path, for tests)
-    const char* force = getenv("THM_BT_CPL_GLOBAL");
-    c.cglob = (cfull > 12 * 1024 || (force && atoi(force) != 0)) ? 1 : 0;
-    c.cslot = c.cglob ? 16 : cfull;
-    THM_REQUIRE(m->bt_nvec < INT32_MAX, "block-solve data too large");
-    c.nvec = (int)m->bt_nvec;
-    auto layout = [&](int ns, size_t slot) {
-        return bt_layout<V>(ns, (int)slot, (int)c.cslot, m->max_lev, c.nvec, m->max_m).total;
-    };
-    // the largest tile height (<= the target) that leaves room for at least 3 slots
-    c.rows = (int)std::max<size_t>(1, target / row_bytes);
-    while (c.rows > 1 && layout(3, bt_r16((size_t)c.rows * row_bytes)) > cap) --c.rows;
-    c.slot = bt_r16((size_t)c.rows * row_bytes);
-    THM_REQUIRE(c.slot < (size_t)INT32_MAX, "block-solve tile too large");
-    for (int q = 16; q >= 2 && c.ns == 0; --q)
-        if (layout(q, c.slot) <= cap) c.ns = q;
-    THM_REQUIRE(c.ns >= 2, "subdomain too large for the shared-memory block solve (" +
-                               std::to_string(layout(0, 0)) + " bytes of vectors and level data, " +
-                               std::to_string(c.slot) + "-byte tiles)");
-    c.smem = layout(c.ns, c.slot);
-    return c;
-}
-
-template <class V, class F, class FW = F>
-static void bt_launch(const thm_sys* s, const BtCfg& c, const FW* fac, const F* cval, const int32_t* ab, const F* av,
-                      const F* cv, const int32_t* e8, const F* ev, const V* x, V* y,
-                      const int* act = nullptr) {
+// The block preconditioner of every subdomain: one cluster of nd.C CTAs each.
+// Two CTAs to an SM where their vectors fit (each hides the other's barriers
+// and L2 latency); vectors that outgrow shared memory leave the u buffers,
+// then the staged y, in a workspace of the system.
+template <class V, class FW>
+static void nd_apply(const thm_sys* s, const FW* fac, const V* x, V* y, const int* act) {
     const thm_mesh* m = s->m;
-    static size_t attr = 0;
-    if (c.smem > 48 * 1024 && c.smem > attr) {
-        THM_CUDA(cudaFuncSetAttribute(k_bt_solve<V, F, FW>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)c.smem));
-        attr = c.smem;
-    }
-    // the work counter follows the Eq. 7 (real-factor) applies only
-    unsigned long long* work =
-        (s->bt_work.p && !BtCplx<FW>::value) ? s->bt_work.p + (sizeof(F) == 4 ? 2 : 0) : nullptr;
-    // every device wait gives up after THM_BT_WAIT_LIMIT_MS (default 1000 ms);
-    // THM_TEST_STALL_TMA=1 makes the tile stream never arrive, so that a test
-    // can see the bounded waits expire and THM_ETIMEOUT come back
-    const char* lim = getenv("THM_BT_WAIT_LIMIT_MS");
-    const unsigned long long wait_ns = 1000000ull * (unsigned long long)(lim ? std::max(1, atoi(lim)) : 1000);
-    const char* stall = getenv("THM_TEST_STALL_TMA");
-    const int stall_w = stall && atoi(stall) != 0 ? 1 : 0;
-    THM_LAUNCH(THM_K_PINV, s->st,
-               (k_bt_solve<V, F, FW><<<dim3(2, m->n_sub), BT_THREADS, c.smem, s->st>>>(
-                   m->d_subs.p, m->d_levels.p, fac, m->d_cpl_ptr.p, m->d_cpl_col.p, cval, m->n_loc,
-                   m->order == 2 ? 1 : 0, ab, av, cv, e8, ev, c.rows, c.ns, (int)c.slot, (int)c.cslot, c.cglob,
-                   m->max_lev, c.nvec, m->max_m, wait_ns, stall_w, s->dev_err.p, act, m->d_bt_welem.p, work, x,
-                   y)));
-}
-
-// The tile size is tuned once per mesh and factor precision: on the first
-// apply of a system every candidate runs on the caller's vectors (the result
-// is the same each time) and the fastest of two timed launches wins; later
-// systems on the same mesh reuse it.  THM_BT_TILE_BYTES fixes it instead.
-template <class V, class F, class FW = F>
-static void apply_Pinv(const thm_sys* s, const FW* fac, const F* cval, const int32_t* ab, const F* av,
-                       const F* cv, const int32_t* e8, const F* ev, const V* x, V* y,
-                       const int* act = nullptr) {
-    const thm_mesh* m = s->m;
-    THM_REQUIRE(m->max_m <= BT_MAX_M, "level block larger than the block-solve kernel supports (" +
-                                          std::to_string(m->max_m) + " > " + std::to_string(BT_MAX_M) + ")");
-    size_t& tile = m->bt_tile[(sizeof(F) == 4 ? 1 : 0) + (BtCplx<FW>::value ? 2 : 0)];
+    require_nd(m);
+    const NdSizes& z = m->nd.z;
     if (!s->bt_work.p) {
         s->bt_work.alloc(4);
         s->bt_work.zero(s->st);
     }
-    if (tile == 0) {
-        if (const char* e = getenv("THM_BT_TILE_BYTES")) {
-            tile = (size_t)std::max(1024, atoi(e));
-        } else {
-            const size_t cand[] = {16384, 32768, 49152, 65536, 98304};
-            cudaEvent_t e0, e1;
-            THM_CUDA(cudaEventCreate(&e0));
-            THM_CUDA(cudaEventCreate(&e1));
-            float best = 1e30f;
-            int best_rows = -1;
-            for (size_t t : cand) {
-                const BtCfg c = bt_config<V, F, FW>(m, t);
-                if (c.rows == best_rows) continue;                // same tiles as a faster-or-equal candidate
-                bt_launch<V, F, FW>(s, c, fac, cval, ab, av, cv, e8, ev, x, y);          // warm
-                THM_CUDA(cudaEventRecord(e0, s->st));
-                for (int r = 0; r < 2; ++r) bt_launch<V, F, FW>(s, c, fac, cval, ab, av, cv, e8, ev, x, y);
-                THM_CUDA(cudaEventRecord(e1, s->st));
-                THM_CUDA(cudaEventSynchronize(e1));
-                float ms = 0;
-                THM_CUDA(cudaEventElapsedTime(&ms, e0, e1));
-                if (ms < best) { best = ms; tile = t; best_rows = c.rows; }
-            }
-            cudaEventDestroy(e0);
-            cudaEventDestroy(e1);
-        }
-    }
-    bt_launch<V, F, FW>(s, bt_config<V, F, FW>(m, tile), fac, cval, ab, av, cv, e8, ev, x, y, act);
+    int u_glob = 0, y_glob = 0;
+    const int slt_smem = (size_t)z.nslt * sizeof(int2) <= 16 * 1024 ? 1 : 0;
+    if (nd_layout<V>(z, slt_smem, 0, 0).total > ND_SMEM_MAX) u_glob = 1;
+    if (nd_layout<V>(z, slt_smem, u_glob, 0).total > ND_SMEM_MAX) y_glob = 1;
+    const size_t smem = nd_layout<V>(z, slt_smem, u_glob, y_glob).total;
+    THM_REQUIRE(smem <= ND_SMEM_MAX, "subdomain too large for the shared-memory block solve");
+    const int64_t stride = (u_glob || y_glob) ? (int64_t)z.nu[0] + z.nu[1] + z.ny : 0;
+    if (stride > 0 && s->nd_glob.n < (size_t)(stride * m->n_sub * m->nd.C)) s->nd_glob.alloc(stride * m->n_sub * m->nd.C);
+    static std::once_flag once;
+    std::call_once(once, [] {
+        THM_CUDA(cudaFuncSetAttribute(k_nd_solve<V, FW>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ND_SMEM_MAX));
+    });
+    // the work counter follows the Eq. 7 (real-factor) applies only
+    unsigned long long* work = NdCplx<FW>::value ? nullptr : s->bt_work.p + (sizeof(FW) == 4 ? 2 : 0);
+    // the wait for the table copies gives up after THM_BT_WAIT_LIMIT_MS
+    // (default 1000 ms); THM_TEST_STALL_TMA=1 holds the copies back, so that a
+    // test can see the bounded wait expire and THM_ETIMEOUT come back
+    const char* lim = getenv("THM_BT_WAIT_LIMIT_MS");
+    const unsigned long long wait_ns = 1000000ull * (unsigned long long)(lim ? std::max(1, atoi(lim)) : 1000);
+    const char* stall = getenv("THM_TEST_STALL_TMA");
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(m->nd.C, m->n_sub);
+    cfg.blockDim = dim3(ND_NT);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s->st;
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeClusterDimension;
+    at.val.clusterDim.x = m->nd.C;
+    at.val.clusterDim.y = at.val.clusterDim.z = 1;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    THM_LAUNCH(THM_K_PINV, s->st,
+               THM_CUDA(cudaLaunchKernelEx(&cfg, k_nd_solve<V, FW>, nd_tables(m), z, slt_smem, u_glob, y_glob,
+                                           reinterpret_cast<V*>(s->nd_glob.p), stride, fac, wait_ns,
+                                           (int)(stall && atoi(stall) != 0), s->dev_err.p, act, work, x, y)));
 }
 
 // The full 2x2 block preconditioner (Section 3.2's alternative): T_i^{-1} from
 // the complex factors.
 template <class V>
 static void apply_Tinv_mode(const thm_sys* s, bool f32, const V* x, V* y, const int* act = nullptr) {
-    if (f32)
-        apply_Pinv<V, float, float2>(s, s->facc32.p, s->cpl32.p, s->tab_ab.p, s->tab_av32.p,
-                                     s->tab_cv32.p, s->tab_e8.p, s->tab_ev32.p, x, y, act);
-    else
-        apply_Pinv<V, double, double2>(s, s->facc64.p, s->cpl64.p, s->tab_ab.p, s->tab_av64.p,
-                                       s->tab_cv64.p, s->tab_e8.p, s->tab_ev64.p, x, y, act);
+    if (f32) nd_apply<V, float2>(s, s->facc32.p, x, y, act);
+    else if constexpr (sizeof(V) == 16) nd_apply<V, double2>(s, s->facc64.p, x, y, act);
 }
 
 template <class V>
 static void apply_Pinv_mode(const thm_sys* s, bool f32, const V* x, V* y, const int* act = nullptr) {
-    if (f32)
-        apply_Pinv<V, float>(s, s->fac32.p, s->cpl32.p, s->tab_ab.p, s->tab_av32.p, s->tab_cv32.p,
-                             s->tab_e8.p, s->tab_ev32.p, x, y, act);
-    else
-        apply_Pinv<V, double>(s, s->fac64.p, s->cpl64.p, s->tab_ab.p, s->tab_av64.p, s->tab_cv64.p,
-                              s->tab_e8.p, s->tab_ev64.p, x, y, act);
+    if (f32) nd_apply<V, float>(s, s->fac32.p, x, y, act);
+    else if constexpr (sizeof(V) == 16) nd_apply<V, double>(s, s->fac64.p, x, y, act);
 }
-
-
 
 static void add(RunStats& rs, const KStats& k) {
     rs.inner += k.iters;
