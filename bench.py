@@ -69,8 +69,7 @@ def parse():
 
 
 def ncu_sweep(args):
-    """Two sweeps of the bench workload (the first warms the factorisation and
-    the tile autotuner): the kernel mix of the timed solve, in a few seconds,
+    """Two sweeps of the bench workload (the first builds the factors): the kernel mix of the timed solve, in a few seconds,
     for ncu.  The interface data are seeded random values, so every
     subdomain's solve is active (with zero interface data only the subdomains
     on the Dirichlet side would have a right-hand side)."""
@@ -474,9 +473,7 @@ def main():
         u, stats = sysg.solve(mode=m, rtol=1e-8, relax=args.relax if relax is None else relax, **kw)
         return sysg, u, stats
 
-    # warm-up: module loading, first launches, and the block-solve tile
-    # autotuner (it runs on a mesh's first apply per precision; every later
-    # system on the mesh reuses its choice)
+    # warm-up: module loading, first launches
     for _ in range(args.warmup):
         step(mode)
     torch.cuda.synchronize()
@@ -509,29 +506,29 @@ def main():
     tt = [s["seconds"] for s in stats_all]
 
     # ---- instrumented steps (after the timed region): per-class CUDA-event
-    # timing of every launch, and the block-solve work counted on the device ----
-    classes = (thm.K_PINV, thm.K_SPMV, thm.K_DOTS, thm.K_UPDATE, thm.K_KRYLOV, thm.K_DDM, thm.K_SETUP)
+    # timing of every launch, and the work of the subdomain solves counted on the device ----
+    classes = (thm.K_SUBSOLVE, thm.K_PINV, thm.K_SPMV, thm.K_DOTS, thm.K_UPDATE, thm.K_KRYLOV, thm.K_DDM, thm.K_SETUP)
     thm.profile_enable(sum(1 << c for c in classes))
     torch.cuda.synchronize()
     p0 = torch.cuda.Event(enable_timing=True)
     p1 = torch.cuda.Event(enable_timing=True)
     p0.record(st)
-    pinv_work = 0.0          # algorithmic bytes the block solve actually processed (converged subdomains skipped)
-    other_work = {thm.K_SPMV: 0.0, thm.K_DOTS: 0.0, thm.K_UPDATE: 0.0}
+    names = {thm.K_PINV: "block-preconditioner applies", thm.K_SPMV: "subdomain operator applies",
+             thm.K_DOTS: "Gram-Schmidt dot products", thm.K_UPDATE: "Gram-Schmidt updates"}
+    work = {c: 0.0 for c in names}
     pstats = []
     for _ in range(max(1, args.prof_steps)):
         sysg, _, s1 = step(mode)
         pstats.append(s1)
-        pinv_work += thm.work_bytes(sysg, mode, thm.K_PINV)
-        for c in other_work:
-            other_work[c] += thm.work_bytes(sysg, mode, c)
+        for c in work:
+            work[c] += thm.work_bytes(sysg, mode, c)
     p1.record(st)
     torch.cuda.synchronize()
     prof_ms = p0.elapsed_time(p1)
     prof = {c: thm.profile_read(c) for c in classes}
     thm.profile_enable(0)
 
-    # roofline of the dominant kernel (block-preconditioner apply)
+    # roofline of the dominant kernel (the subdomain solves of a sweep, one launch)
     peaks = {}
     try:
         peaks = json.load(open(os.path.join(ROOT, "MEASURED_PEAKS.json")))
@@ -539,45 +536,27 @@ def main():
         pass
     hbm_peak = peaks.get("hbm_gbs", 6800.0)
     peak_src = "measured" if "hbm_gbs" in peaks else "fallback"
-    n_launch, pinv_ms = prof[thm.K_PINV]
-    per_launch_s = pinv_ms / 1e3 / max(1, n_launch)
-    alg_bytes = thm.algorithmic_bytes(sysg, mode, thm.K_PINV)
-    # inside the Arnoldi steps the kernel skips converged subdomains, so a
-    # launch moves between 0 and alg_bytes; the kernel counts the work it did
-    achieved = pinv_work / (pinv_ms / 1e3) / 1e9 if n_launch and pinv_ms > 0 else None
-    roofline = {"kernel": "k_bt_solve (block-preconditioner apply, Eq. 7)", "bound": "hbm",
+    n_launch, sub_ms = prof[thm.K_SUBSOLVE]
+    total_work = sum(work.values())
+    achieved = total_work / (sub_ms / 1e3) / 1e9 if n_launch and sub_ms > 0 else None
+    roofline = {"kernel": "k_subsolve (subdomain GMRES solves, one launch per sweep)", "bound": "hbm",
                 "achieved": achieved, "peak": hbm_peak, "unit": "GB/s",
                 "frac": (achieved / hbm_peak) if achieved else None,
-                "traffic": measured_traffic("k_bt_solve", mode),
-                "peak_source": peak_src, "launches": n_launch, "avg_launch_us": 1e6 * per_launch_s,
-                "alg_bytes_full_launch": alg_bytes,
-                "alg_bytes_processed": pinv_work,
-                "achieved_definition": "algorithmic bytes of the subdomains processed (counted on the device) / "
-                                       "summed CUDA-event time of its launches, over "
-                                       f"{max(1, args.prof_steps)} instrumented step(s) run after the timed region",
-                "share_of_step": (pinv_ms / prof_ms) if prof_ms > 0 else None,
+                "traffic": measured_traffic("k_subsolve", mode),
+                "peak_source": peak_src, "launches": n_launch, "avg_launch_us": 1e3 * sub_ms / max(1, n_launch),
+                "alg_bytes_processed": total_work,
+                "alg_bytes_by_part": {names[c]: work[c] for c in names},
+                "achieved_definition": "algorithmic bytes of the Arnoldi steps done (counted on the device: factors, "
+                                       "operator, basis vectors read and written) / summed CUDA-event time of its "
+                                       f"launches, over {max(1, args.prof_steps)} instrumented step(s) run after the "
+                                       "timed region",
+                "share_of_step": (sub_ms / prof_ms) if prof_ms > 0 else None,
                 "classes": kernel_classes_report(thm, prof, prof_ms),
                 "instrumented_ms_per_step": prof_ms / max(1, args.prof_steps),
                 "instrumented_time_to_1e8_s": statistics.median(s["seconds"] for s in pstats)}
-    # the other per-iteration kernels, the same way (bytes counted on the device)
-    names = {thm.K_SPMV: "k_spmv (subdomain operator T_i)",
-             thm.K_DOTS: "k_dcgs_dots (Gram-Schmidt dot-product pass)",
-             thm.K_UPDATE: "k_dcgs_update (Gram-Schmidt update pass)"}
-    others = {}
-    for c, work in other_work.items():
-        n_c, ms_c = prof[c]
-        ach = work / (ms_c / 1e3) / 1e9 if n_c and ms_c > 0 else None
-        others[names[c]] = {"bound": "hbm", "achieved": ach, "peak": hbm_peak, "unit": "GB/s",
-                            "frac": (ach / hbm_peak) if ach else None, "launches": n_c,
-                            "avg_launch_us": 1e3 * ms_c / max(1, n_c), "alg_bytes_processed": work}
-    roofline["other_kernels"] = others
-    roofline["other_kernels_definition"] = (
-        "per launch class: algorithmic bytes counted on the device / summed CUDA-event time of the class's "
-        "launches in the instrumented steps (the class time also holds the interface GMRES's few small "
-        "Gram-Schmidt launches, whose FP64 bytes are counted apart)")
 
-    # plain FP64 form, timed beside (time-to-1e-8); warmed first: FP64 kernels,
-    # the FP64 factorisation path and the FP64 tile autotuning on this mesh.
+    # plain FP64 form, timed beside (time-to-1e-8); warmed first (FP64 kernels
+    # and factorisation).
     # It runs without the relaxation of the subdomain tolerance (its FP64
     # subdomain solves stop exactly at the relaxed tolerance, which costs the
     # interface GMRES more steps than it saves: 1,000 against 361 measured)
@@ -605,8 +584,7 @@ def main():
 
     # Section 3.2's alternative preconditioner: the exact inverse of the full
     # 2x2 block operator (T_i^{-1}, complex factors: twice the memory), timed
-    # beside the Eq. 7 form on the same workload; warmed first (its kernels and
-    # the complex-factor tile autotuning on this mesh)
+    # beside the Eq. 7 form on the same workload; warmed first
     full = None
     if mode == "mixed" and args.full_steps > 0:
         step(mode, precond="full", outer_maxit=3, max_refine=1, check=False)

@@ -368,7 +368,8 @@ int thm_dirichlet_values(thm_sys* s, double* u_d);
 #define THM_K_KRYLOV    4   /* other Krylov kernels (scale, Givens, reductions) */
 #define THM_K_DDM       5   /* right-hand sides, exchange, glue, residual, IR   */
 #define THM_K_SETUP     6   /* numbering, assembly, factorisation               */
-#define THM_K_NCLASSES  7
+#define THM_K_SUBSOLVE  7   /* subdomain solves: whole GMRES solves, one launch a sweep */
+#define THM_K_NCLASSES  8
 
 /* Algorithmic bytes one launch of class cls must move in mode (THM_MODE_*),
  * from the system's sizes (index streams and SELL padding are layout

@@ -111,8 +111,8 @@ def load():
     return lib
 
 
-K_SPMV, K_PINV, K_DOTS, K_UPDATE, K_KRYLOV, K_DDM, K_SETUP = range(7)
-K_NAMES = ["spmv", "pinv", "dots", "update", "krylov", "ddm", "setup"]
+K_SPMV, K_PINV, K_DOTS, K_UPDATE, K_KRYLOV, K_DDM, K_SETUP, K_SUBSOLVE = range(8)
+K_NAMES = ["spmv", "pinv", "dots", "update", "krylov", "ddm", "setup", "subsolve"]
 
 
 def kernel_launches() -> int:

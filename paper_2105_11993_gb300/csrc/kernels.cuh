@@ -23,56 +23,45 @@ __device__ __forceinline__ double2 cadd(double2 a, double2 b) { return make_doub
 // 3-D: the face terms are not diagonal; their values (times kappa*omega) ride
 // on the same SELL pattern (bvg: Gamma^inf, bvs: Sigma), non-null only then.
 // Column indices: int32 local indices, or (CI = uint16_t) indices relative
-// to the row's subdomain (subs[row_seg[r]].off added back), half the bytes of
-// the index stream.
-template <class V, class F, class CI = int32_t>
-__global__ void __launch_bounds__(256) k_spmv(int64_t n, const int64_t* __restrict__ slice_ptr,
-                                              const CI* __restrict__ col, const Sub* __restrict__ subs,
-                                              const F* __restrict__ val,
-                                              const F* __restrict__ bg, const F* __restrict__ bs, int use_bs,
-                                              const F* __restrict__ bvg, const F* __restrict__ bvs,
-                                              const V* __restrict__ x, V* __restrict__ y,
-                                              const int32_t* __restrict__ row_seg, const int* __restrict__ act,
-                                              unsigned long long* __restrict__ work) {
+// to the row's subdomain (origin: its first local row), half the bytes of the
+// index stream.  xs: x at the column origin.
+// The matrix arrays of one precision.
+template <class F>
+struct SpmvMat {
+    const F *val, *bg, *bs;
+    const F *bvg, *bvs;       // 3-D only
+};
+// Row r times x: slots in groups of 8, so that the 8 index and value loads,
+// then the 8 gathers of x, are in flight together.
+template <class V, class F, class CI>
+__device__ __forceinline__ V spmv_row(int64_t r, const int64_t* __restrict__ slice_ptr, const CI* __restrict__ col,
+                                      const SpmvMat<F>& A, int use_bs, const V* xs, int64_t origin) {
     using R = typename VT<V>::R;
-    int64_t r = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    // a converged subdomain's rows are not needed
-    const bool on = r < n && !(act && !act[row_seg[r < n ? r : 0]]);
-    if (work) {                                // rows processed (uniform branch: every thread reaches the count)
-        const int cnt = __syncthreads_count(on);
-        if (threadIdx.x == 0 && cnt) atomicAdd(work, (unsigned long long)cnt);
-    }
-    if (!on) return;
-    int64_t sl = r >> 5;
-    int lane = (int)(r & 31);
-    int64_t base = slice_ptr[sl];
-    int w = (int)((slice_ptr[sl + 1] - base) >> 5);
+    const int64_t base = __ldg(slice_ptr + (r >> 5));
+    const int w = (int)((__ldg(slice_ptr + (r >> 5) + 1) - base) >> 5);
+    const int64_t at = base + (r & 31);
+    const CI* cp = col + at;
+    const F* vp = A.val + at;
     R ar = 0, ai = 0;
-    const CI* cp = col + base + lane;
-    const V* xs = x;                           // column origin
-    if constexpr (sizeof(CI) == 2) xs = x + subs[row_seg[r]].off;
-    const F* vp = val + base + lane;
-    if (bvg) {
-        const F* gp = bvg + base + lane;
-        const F* sp = bvs + base + lane;
+    if (A.bvg) {
+        const F* gp = A.bvg + at;
+        const F* sp = A.bvs + at;
         for (int t = 0; t < w; ++t) {
-            int32_t c = (int32_t)__ldg(cp + (t << 5));
-            R v = (R)__ldg(vp + (t << 5));
+            const int32_t c = (int32_t)__ldg(cp + (t << 5));
+            const R v = (R)__ldg(vp + (t << 5));
             R b = (R)__ldg(gp + (t << 5));
             if (use_bs) b += (R)__ldg(sp + (t << 5));
-            V xv = xs[c];
+            const V xv = xs[c];
             ar += v * xv.x - b * xv.y;
             ai += v * xv.y + b * xv.x;
         }
     } else {
-        // slots in groups of 8: the 8 index and value loads, then the 8
-        // gathers of x, are in flight together
         for (int t0 = 0; t0 < w; t0 += 8) {
             int32_t c[8];
             R v[8];
 #pragma unroll
             for (int u = 0; u < 8; ++u) {
-                c[u] = (int32_t)(r - (xs - x));    // own row (its x is read below anyway)
+                c[u] = (int32_t)(r - origin);      // own row (its x is read below anyway)
                 v[u] = 0;
                 if (t0 + u < w) {
                     c[u] = (int32_t)__ldg(cp + ((t0 + u) << 5));
@@ -89,10 +78,27 @@ __global__ void __launch_bounds__(256) k_spmv(int64_t n, const int64_t* __restri
             }
         }
     }
-    R b = (R)bg[r];
-    if (use_bs) b += (R)bs[r];
-    V xr = x[r];
-    y[r] = mk<V>(ar - b * xr.y, ai + b * xr.x);
+    R b = (R)__ldg(A.bg + r);
+    if (use_bs) b += (R)__ldg(A.bs + r);
+    const V xr = xs[r - origin];
+    return mk<V>(ar - b * xr.y, ai + b * xr.x);
+}
+
+template <class V, class F, class CI = int32_t>
+__global__ void __launch_bounds__(256) k_spmv(int64_t n, const int64_t* __restrict__ slice_ptr,
+                                              const CI* __restrict__ col, const Sub* __restrict__ subs,
+                                              SpmvMat<F> A, int use_bs, const V* __restrict__ x,
+                                              V* __restrict__ y, const int32_t* __restrict__ row_seg,
+                                              unsigned long long* __restrict__ work) {
+    const int64_t r = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    if (work) {                                // rows processed (uniform branch: every thread reaches the count)
+        const int cnt = __syncthreads_count(r < n);
+        if (threadIdx.x == 0 && cnt) atomicAdd(work, (unsigned long long)cnt);
+    }
+    if (r >= n) return;
+    int64_t origin = 0;
+    if constexpr (sizeof(CI) == 2) origin = subs[row_seg[r]].off;
+    y[r] = spmv_row<V, F, CI>(r, slice_ptr, col, A, use_bs, x + origin, origin);
 }
 
 // ---- TMA 1-D bulk copies completing on an mbarrier (sm_90+ PTX) ----------

@@ -218,73 +218,142 @@ __host__ __device__ inline NdLayout nd_layout(const NdSizes& z, int slt_smem, in
     return L;
 }
 
-template <class V, class FW>
-__global__ void __launch_bounds__(ND_NT, 2)
-k_nd_solve(NdTables T, NdSizes z, int slt_smem, int u_glob, int y_glob, V* __restrict__ glob, int64_t glob_stride,
-           const FW* __restrict__ fac, unsigned long long wait_ns, int stall, int* __restrict__ err,
-           const int* __restrict__ act, unsigned long long* __restrict__ work, const V* __restrict__ x,
-           V* __restrict__ y) {
-    namespace cg = cooperative_groups;
-    extern __shared__ __align__(128) unsigned char smem[];
-    __shared__ int s_abort;
-    // a subdomain whose Krylov segment has converged is skipped by every CTA
-    // of its cluster (same flag, read before any cluster barrier)
-    if (act && !act[blockIdx.y]) return;
-    cg::cluster_group cluster = cg::this_cluster();
-    const int rank = (int)blockIdx.x, C = (int)gridDim.x;
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const NdPart P = T.parts[(int64_t)blockIdx.y * C + rank];
-    const NdLayout lay = nd_layout<V>(z, slt_smem, u_glob, y_glob);
+// Launch options that the host decides from the sizes (nd_memory).
+struct NdMem {
+    int slt_smem, u_glob, y_glob, prefetch;
+    int64_t glob_stride;
+};
+
+// Where a CTA's pieces are: built once per launch, used by every apply in it.
+template <class V>
+struct NdCta {
+    NdPart P;
+    const NdLev* lev;
+    const int2* slt;
+    V *vec, *ysc, *u_even, *u_odd, *part;
+    V* glob;                  // this subdomain's u_odd of rank 0 in the global workspace (u_glob), its ranks glob_stride apart
+    int64_t glob_stride;
+    int rank, C, u_glob, ny, prefetch;
+    bool ok;                  // the tables came
+};
+
+// Start of a solve CTA: its level and slice tables come by TMA (stall:
+// failure-detection test, the copies never come).  GLOB: some of the tables
+// and vectors are in global memory; else all are in shared memory, which the
+// compiler must see (through pointers that may be either, an apply takes 126
+// registers instead of 69 and its shared-memory loads several times as long).
+template <bool GLOB, class V>
+__device__ __forceinline__ void nd_enter(NdCta<V>& c, const NdTables& T, const NdSizes& z, const NdMem& mm, V* glob,
+                                         unsigned char* smem, int sub, int rank, int C, unsigned long long wait_ns, int stall,
+                                         int* s_abort, int* err) {
+    const int tid = threadIdx.x;
+    c.P = T.parts[(int64_t)sub * C + rank];
+    const NdLayout lay = nd_layout<V>(z, mm.slt_smem, mm.u_glob, mm.y_glob);
     uint64_t* bar = reinterpret_cast<uint64_t*>(smem);
     NdLev* lev = reinterpret_cast<NdLev*>(smem + lay.lev);
-    V* vec = reinterpret_cast<V*>(smem + lay.vec);
-    V* gl = glob + ((int64_t)blockIdx.y * C + rank) * glob_stride;
-    V* ysc = y_glob ? gl + z.nu[0] + z.nu[1] : reinterpret_cast<V*>(smem + lay.ysc);
-    V* u_even = u_glob ? gl : reinterpret_cast<V*>(smem + lay.u0);          // u of the even depths
-    V* u_odd = u_glob ? gl + z.nu[0] : reinterpret_cast<V*>(smem + lay.u1);
-    V* part = reinterpret_cast<V*>(smem + lay.part);
-    const int2* slt = slt_smem ? reinterpret_cast<const int2*>(smem + lay.slt) : T.slt + P.slt0;
-
-    // the CTA's level and slice tables come by TMA while the threads gather r
+    c.lev = lev;
+    c.vec = reinterpret_cast<V*>(smem + lay.vec);
+    c.part = reinterpret_cast<V*>(smem + lay.part);
+    c.slt = reinterpret_cast<const int2*>(smem + lay.slt);
+    c.ysc = reinterpret_cast<V*>(smem + lay.ysc);
+    c.u_even = reinterpret_cast<V*>(smem + lay.u0);        // u of the even depths
+    c.u_odd = reinterpret_cast<V*>(smem + lay.u1);
+    if constexpr (GLOB) {
+        V* gl = glob + ((int64_t)sub * C + rank) * mm.glob_stride;
+        if (!mm.slt_smem) c.slt = T.slt + c.P.slt0;
+        if (mm.y_glob) c.ysc = gl + z.nu[0] + z.nu[1];
+        if (mm.u_glob) {
+            c.u_even = gl;
+            c.u_odd = gl + z.nu[0];
+        }
+    }
+    c.glob = glob + (int64_t)sub * C * mm.glob_stride + z.nu[0];
+    c.glob_stride = mm.glob_stride;
+    c.rank = rank;
+    c.C = C;
+    c.u_glob = mm.u_glob;
+    c.ny = z.ny;
+    c.prefetch = mm.prefetch;
     if (tid == 0) {
-        s_abort = 0;
+        *s_abort = 0;
         mbar_init(bar, 1);
         mbar_fence_init();
         fence_proxy_async();
-        if (!stall) {                          // (stall: failure-detection test, the copies never come)
-            const unsigned lb = (unsigned)((P.nlev + 1) * sizeof(NdLev));
-            const unsigned sb = slt_smem ? (unsigned)((P.nslt + 1) / 2 * 16) : 0u;
+        if (!stall) {
+            const unsigned lb = (unsigned)((c.P.nlev + 1) * sizeof(NdLev));
+            const unsigned sb = mm.slt_smem ? (unsigned)((c.P.nslt + 1) / 2 * 16) : 0u;
             mbar_expect_tx(bar, lb + sb);
-            tma_load_1d(lev, T.levs + P.lev0, lb, bar);
-            if (sb) tma_load_1d(smem + lay.slt, T.slt + P.slt0, sb, bar);
+            tma_load_1d(lev, T.levs + c.P.lev0, lb, bar);
+            if (sb) tma_load_1d(smem + lay.slt, T.slt + c.P.slt0, sb, bar);
         }
-        if (work && rank == 0) {               // instrumentation: the work this launch does
-            atomicAdd(&work[0], (unsigned long long)T.welem[blockIdx.y]);
-            atomicAdd(&work[1], (unsigned long long)T.subs[blockIdx.y].n);
+        if (!mbar_try(bar, 0)) {
+            const unsigned long long t0 = nd_now_ns();
+            while (!mbar_try(bar, 0))
+                if (nd_now_ns() - t0 > wait_ns) {          // bounded: give up, skip the work, keep the barriers
+                    *s_abort = 1;
+                    atomicExch(err, 1);
+                    break;
+                }
         }
-    }
-    const int32_t* perm = T.perm + P.perm0;
-    for (int p = tid; p < P.nvec; p += ND_NT) {
-        const int32_t r = __ldg(perm + p);
-        vec[p] = r >= 0 ? x[r] : mk<V>(0, 0);
-    }
-    for (int p = tid; p < z.ny; p += ND_NT) ysc[p] = mk<V>(0, 0);     // rows are padded to the widest node of their slice
-    if (tid == 0 && !mbar_try(bar, 0)) {
-        const unsigned long long t0 = nd_now_ns();
-        while (!mbar_try(bar, 0))
-            if (nd_now_ns() - t0 > wait_ns) {  // bounded: give up, skip the work, keep the barriers
-                s_abort = 1;
-                atomicExch(err, 1);
-                break;
-            }
     }
     __syncthreads();
-    const bool ok = s_abort == 0;
+    c.ok = *s_abort == 0;
+}
+
+// Asks for the factor entries of n slices from slice s0 on to come to L2.
+template <class FW>
+__device__ __forceinline__ void nd_prefetch(const FW* fac, const int2* slt, int s0, int n) {
+    if (n <= 0) return;
+    const int64_t a = slt[s0].x, b = (int64_t)slt[s0 + n - 1].x + slt[s0 + n - 1].y;
+    asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;\n" ::"l"(fac + a * 128),
+                 "r"((unsigned)((b - a) * 128 * sizeof(FW)))
+                 : "memory");
+}
+
+// One apply y = P_i^{-1} x by the CTAs of a cluster.  x may have been written
+// by other CTAs of the cluster in this launch (before a cluster barrier), so
+// it is read with ordinary loads.
+template <bool GLOB, class V, class FW>
+__device__ __forceinline__ void nd_apply_cta(const NdCta<V>& c, const NdTables& T, const FW* __restrict__ fac, const V* x,
+                                             V* y) {
+    namespace cg = cooperative_groups;
+    cg::cluster_group cluster = cg::this_cluster();
+    const NdPart& P = c.P;
+    const NdLev* lev = c.lev;
+    const int2* slt = c.slt;
+    V *vec = c.vec, *ysc = c.ysc, *u_even = c.u_even, *u_odd = c.u_odd, *part = c.part;
+    const bool ok = c.ok;
+    const int C = c.C, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int nlev = ok ? P.nlev : 0;
+    // the rows of step st: up 0..nlev-1, the root nlev, down
+    auto prefetch = [&](int st) {
+        if (!c.prefetch || tid != 0 || !ok || st > 2 * nlev) return;
+        const NdLev& L = lev[st <= nlev ? st : 2 * nlev - st];
+        if (st < nlev || (st == nlev && P.sroot > 0)) nd_prefetch(fac, slt, L.sltf, L.nsf);
+        else if (st > nlev) nd_prefetch(fac, slt, L.sltb, L.nsb);
+    };
+    prefetch(0);
+    prefetch(1);
+    const int32_t* perm = T.perm + P.perm0;
+    constexpr int G = 4;                       // gathers in flight per thread
+    for (int p0 = tid; p0 < P.nvec; p0 += G * ND_NT) {
+        int32_t r[G];
+        V v[G];
+#pragma unroll
+        for (int g = 0; g < G; ++g) r[g] = p0 + g * ND_NT < P.nvec ? __ldg(perm + p0 + g * ND_NT) : -1;
+#pragma unroll
+        for (int g = 0; g < G; ++g) v[g] = r[g] >= 0 ? x[r[g]] : mk<V>(0, 0);
+#pragma unroll
+        for (int g = 0; g < G; ++g)
+            if (p0 + g * ND_NT < P.nvec) vec[p0 + g * ND_NT] = v[g];
+    }
+    for (int p = tid; p < c.ny; p += ND_NT) ysc[p] = mk<V>(0, 0);     // rows are padded to the widest node of their slice
+    __syncthreads();
 
     // ---- up: the CTA's subtrees, deepest level first
     for (int l = 0; l < nlev; ++l) {
         const NdLev L = lev[l];
+        prefetch(l + 2);
         const V* uin = (L.depth & 1) ? u_even : u_odd;
         V* uout = (L.depth & 1) ? u_odd : u_even;
         for (int e = tid; e < L.nv; e += ND_NT) {
@@ -331,14 +400,16 @@ k_nd_solve(NdTables T, NdSizes z, int slt_smem, int u_glob, int y_glob, V* __res
         cluster.sync();                        // every rank's u is complete, and its r of the root is staged
         if (ok) {
             const NdLev L = lev[nlev];
+            prefetch(nlev + 2);
             for (int e = tid; e < P.sroot; e += ND_NT) {
                 V v = ysc[e];
-                for (int c = 0; c < 2 * T.mw; ++c) {
-                    const uint32_t a = __ldg(T.rmap + ((int64_t)P.rmap0 + e) * 2 * T.mw + c);
+                for (int q = 0; q < 2 * T.mw; ++q) {
+                    const uint32_t a = __ldg(T.rmap + ((int64_t)P.rmap0 + e) * 2 * T.mw + q);
                     if (a == 0xffffffffu) break;
                     const int rk = (int)(a >> 16);
-                    const V* src = u_glob ? glob + ((int64_t)blockIdx.y * C + rk) * glob_stride + z.nu[0]
-                                          : cluster.map_shared_rank(u_odd, rk);
+                    const V* src;
+                    if constexpr (GLOB) src = c.u_glob ? c.glob + rk * c.glob_stride : cluster.map_shared_rank(u_odd, rk);
+                    else src = cluster.map_shared_rank(u_odd, rk);
                     v = nd_add(v, src[a & 0xffffu]);
                 }
                 ysc[e] = v;
@@ -376,6 +447,7 @@ k_nd_solve(NdTables T, NdSizes z, int slt_smem, int u_glob, int y_glob, V* __res
     // ---- down
     for (int l = nlev - 1; l >= 0; --l) {
         const NdLev L = lev[l];
+        prefetch(2 * nlev - l + 2);
         auto put = [&](uint32_t d, V a) { vec[d >> 16] = nd_add(vec[d >> 16], a); };
         if (L.ksb == 1) {
             for (int sl = warp; sl < L.nsb; sl += ND_NW) {
@@ -408,6 +480,22 @@ k_nd_solve(NdTables T, NdSizes z, int slt_smem, int u_glob, int y_glob, V* __res
             const int32_t r = __ldg(perm + p);
             if (r >= 0 && (p >= P.sroot || (p >= P.rr0 && p < P.rr0 + P.nrr))) y[r] = vec[p];
         }
+}
+
+template <bool GLOB, class V, class FW>
+__global__ void __launch_bounds__(ND_NT, 2)
+k_nd_solve(NdTables T, NdSizes z, NdMem mm, V* __restrict__ glob, const FW* __restrict__ fac, unsigned long long wait_ns,
+           int stall, int* __restrict__ err, unsigned long long* __restrict__ work, const V* __restrict__ x,
+           V* __restrict__ y) {
+    extern __shared__ __align__(128) unsigned char smem[];
+    __shared__ int s_abort;
+    NdCta<V> c;
+    nd_enter<GLOB>(c, T, z, mm, glob, smem, (int)blockIdx.y, (int)blockIdx.x, (int)gridDim.x, wait_ns, stall, &s_abort, err);
+    nd_apply_cta<GLOB>(c, T, fac, x, y);
+    if (work && blockIdx.x == 0 && threadIdx.x == 0) {     // instrumentation: the work this launch does
+        atomicAdd(&work[0], (unsigned long long)T.welem[blockIdx.y]);
+        atomicAdd(&work[1], (unsigned long long)T.subs[blockIdx.y].n);
+    }
 }
 
 }  // namespace thm

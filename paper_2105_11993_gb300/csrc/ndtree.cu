@@ -489,7 +489,6 @@ void build_nd(thm_mesh* m) {
     // many that a CTA has less than a warp pass of unknowns
     int p = 0;
     while (p < 3 && (int64_t)ns * (2 << p) <= 2 * (int64_t)sms && m->n_loc / ns >= (int64_t)(64 << (p + 1))) ++p;
-    if (const char* e = getenv("THM_ND_P")) p = atoi(e);
     for (;; ++p) {
         m->nd_ok = build_tables(m, cells, p) && smallest_smem(m->nd.z) <= ND_SMEM_MAX;
         if (m->nd_ok || p == 3) break;

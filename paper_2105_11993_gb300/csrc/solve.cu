@@ -7,12 +7,13 @@
 #include <cstdio>
 #include <cstdlib>
 #include <functional>
-#include <mutex>
 #include <string>
 
 #include "kernels.cuh"
+#include "krylov.cuh"
 #include "ndsolve.cuh"
 #include "solver.cuh"
+#include "subsolve.cuh"
 
 namespace thm {
 
@@ -47,137 +48,6 @@ __global__ void k_cycle_start(int nseg, int m, const double* __restrict__ nrm2, 
     if (a) atomicAdd(nact, 1);
 }
 
-// Column j of the Hessenberg matrix (h1 + h2 from the two Gram-Schmidt passes,
-// ||w|| below the diagonal), previous Givens rotations, a new rotation, the
-// updated residual estimate |g_{j+1}| and the per-segment convergence flag.
-struct GivensArgs {
-    int j, m, ldh;
-    const double2* h1;
-    const double2* h2;
-    double2* Rm;
-    double* cs;
-    double2* sn;
-    double2* gv;
-    const double* target;
-    int* active;
-    int* kused;
-    double* beta;
-    int* nact;                 // active segments after this step (the first dots pass of the step zeroes it)
-    int* flag;                 // breakdown (non-finite norm)
-    double2* gmon;             // g_{j+1} of segment 0 for the host monitor (single-segment solves), or null
-    const int32_t* seg_ch;
-    int* cnt;                  // per-segment arrival counters of the last-block reduction
-};
-
-__device__ __forceinline__ double2 gv_mul(double2 a, double2 b) {
-    return make_double2(a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x);
-}
-__device__ __forceinline__ double2 gv_fma(double2 a, double2 b, double2 c) {     // a * b + c
-    return make_double2(fma(a.x, b.x, fma(-a.y, b.y, c.x)), fma(a.x, b.y, fma(a.y, b.x, c.y)));
-}
-
-// One warp.  Applying the previous rotations to the new column is a chain:
-// with a_0 = h_0 and, for i < j,
-//     r_i     = c_i a_i + s_i h_{i+1}               (entry i of the rotated column)
-//     a_{i+1} = -conj(s_i) a_i + c_i h_{i+1}         (carried into rotation i + 1)
-// the carry follows the affine maps a -> A_i a + B_i (A_i = -conj(s_i),
-// B_i = c_i h_{i+1}), which compose associatively.  Each lane composes the
-// maps of its range of i, a shuffle scan gives every lane the composition of
-// the ranges below it (so its incoming carry), and the lanes then walk their
-// ranges in parallel.  FP64 instructions cost a full warp slot on this part
-// whatever the active lanes, so the serial chain of about 12 of them per
-// rotation on one lane becomes about (j / 32) * 16 + 5 * 8 per lane.
-// Column j of segment s: hin[0..j] (shared memory, unrotated), hn = the
-// subdiagonal entry (||w||); the rotated column goes to col[0..j] (shared
-// memory, another array) and to R.  stop: the segment stops after this
-// column whatever its residual (the last column of a cycle).
-__device__ bool givens_core(const GivensArgs& ga, int s, int j, const double2* hin, double hn, double2* col,
-                            bool stop = false) {
-    const int m = ga.m;
-    const int lane = threadIdx.x & 31;
-    if (!isfinite(hn)) {
-        if (lane == 0) {
-            atomicExch(ga.flag, 1);
-            ga.active[s] = 0;
-            ga.beta[s] = 0.0;
-        }
-        return false;
-    }
-    const double* cs = ga.cs + (int64_t)s * m;
-    const double2* sn = ga.sn + (int64_t)s * m;
-    const double2 h0 = hin[0];
-    const int per = (j + 31) / 32;
-    const int b = min(j, lane * per), e = min(j, b + per);
-    // this lane's maps composed: (A, B) = M_{e-1} o ... o M_b
-    double2 A = make_double2(1, 0), B = make_double2(0, 0);
-    for (int i = b; i < e; ++i) {
-        const double2 Ai = make_double2(-sn[i].x, sn[i].y);
-        const double2 hi1 = hin[i + 1];
-        const double2 Bi = make_double2(cs[i] * hi1.x, cs[i] * hi1.y);
-        B = gv_fma(Ai, B, Bi);
-        A = gv_mul(Ai, A);
-    }
-    // inclusive scan over the lanes: (A, B) <- (A, B) o (A, B) of lane - d
-    for (int d = 1; d < 32; d <<= 1) {
-        const double2 Ao = make_double2(__shfl_up_sync(0xffffffffu, A.x, d), __shfl_up_sync(0xffffffffu, A.y, d));
-        const double2 Bo = make_double2(__shfl_up_sync(0xffffffffu, B.x, d), __shfl_up_sync(0xffffffffu, B.y, d));
-        if (lane >= d) {
-            B = gv_fma(A, Bo, B);
-            A = gv_mul(A, Ao);
-        }
-    }
-    // exclusive prefix: the composition of the lanes below
-    double2 Ae = make_double2(__shfl_up_sync(0xffffffffu, A.x, 1), __shfl_up_sync(0xffffffffu, A.y, 1));
-    double2 Be = make_double2(__shfl_up_sync(0xffffffffu, B.x, 1), __shfl_up_sync(0xffffffffu, B.y, 1));
-    if (lane == 0) { Ae = make_double2(1, 0); Be = make_double2(0, 0); }
-    double2 a = gv_fma(Ae, h0, Be);                 // a_b
-    for (int i = b; i < e; ++i) {
-        const double c = cs[i];
-        const double2 si = sn[i];
-        const double2 hi1 = hin[i + 1];
-        col[i] = gv_fma(si, hi1, make_double2(c * a.x, c * a.y));
-        a = gv_fma(make_double2(-si.x, si.y), a, make_double2(c * hi1.x, c * hi1.y));
-    }
-    // a_j: the carry out of the last non-empty range (h_0 when j = 0)
-    const int last = j > 0 ? (j - 1) / per : 0;
-    a = make_double2(__shfl_sync(0xffffffffu, a.x, last), __shfl_sync(0xffffffffu, a.y, last));
-    if (j == 0) a = h0;
-    // the new rotation, from (a_j, ||w||): c = |a| / d, s = (a / |a|) ||w|| / d, d = sqrt(|a|^2 + ||w||^2)
-    const double n2a = a.x * a.x + a.y * a.y, d2 = n2a + hn * hn;
-    double cj;
-    double2 sj;
-    if (d2 == 0.0) { cj = 1.0; sj = make_double2(0, 0); }
-    else if (n2a == 0.0) { cj = 0.0; sj = make_double2(1.0, 0.0); }
-    else {
-        const double ia = rsqrt(n2a), id = rsqrt(d2);
-        cj = n2a * ia * id;
-        const double f = hn * ia * id;
-        sj = make_double2(a.x * f, a.y * f);
-    }
-    int keep = 0;
-    if (lane == 0) {
-        ga.cs[(int64_t)s * m + j] = cj;
-        ga.sn[(int64_t)s * m + j] = sj;
-        col[j] = make_double2(cj * a.x + sj.x * hn, cj * a.y + sj.y * hn);
-        double2* g = ga.gv + (int64_t)s * (m + 1);
-        const double2 gj = g[j];
-        const double2 gn = make_double2(-(sj.x * gj.x + sj.y * gj.y), -(sj.x * gj.y - sj.y * gj.x));   // -conj(s) g_j
-        g[j + 1] = gn;
-        g[j] = make_double2(cj * gj.x, cj * gj.y);
-        if (ga.gmon && s == 0) *ga.gmon = gn;
-        ga.kused[s] = j + 1;
-        ga.beta[s] = hn;
-        const double t = ga.target[s];
-        keep = !(stop || gn.x * gn.x + gn.y * gn.y <= t * t || hn == 0.0);
-        if (!keep) ga.active[s] = 0;
-        else atomicAdd(ga.nact, 1);
-    }
-    __syncwarp();
-    double2* out = ga.Rm + ((int64_t)s * m + j) * m;          // column j, rows 0..j
-    for (int i = lane; i <= j; i += 32) out[i] = col[i];
-    return __shfl_sync(0xffffffffu, keep, 0) != 0;
-}
-
 // Second Gram-Schmidt update w -= V h2 with the per-chunk ||w||^2; the last
 // block of each segment sums the segment's norm partials in chunk order and
 // runs that segment's Givens step (so no separate reduction or Givens launch).
@@ -210,347 +80,12 @@ __global__ void __launch_bounds__(KT) k_update_givens(const Chunk* __restrict__ 
     }
 }
 
-// ---------------------------------------------------------------------------
-// Flexible cycles with delayed re-orthogonalisation (DCGS2): two passes over
-// the basis per Arnoldi step instead of four.
-//
-// Step j holds the orthonormal v_0..v_{j-1} and, in basis slot j, u_j: the
-// next vector orthogonalised once.  z_j = M u_j (kept in the flexible basis),
-// w_j = A z_j.  One pass over the basis gives s = V^H u_j, b = V^H w_j,
-// c1 = u_j^H u_j and c2 = u_j^H w_j, and then
-//     gamma_j = sqrt(c1 - |s|^2),      v_j = (u_j - V s) / gamma_j,
-//     d_j     = v_j^H w_j = (c2 - s^H b) / gamma_j,
-//     u_{j+1} = (w_j - V b - v_j d_j) / gamma_j
-//             = w_j / gamma_j - u_j d_j / gamma_j^2 - V (b - s d_j / gamma_j) / gamma_j,
-// which the second pass writes (v_j over u_j in slot j, u_{j+1} into slot
-// j + 1).  (Without the division by gamma_j the norms of the u_j grow
-// geometrically, ~1e13 after 40 steps, and the cycle loses its accuracy;
-// with it |u_{j+1}| is about h_{j+1,j}.)  One step later
-// u_{j+1} = V_{0..j} s_{j+1} + gamma_{j+1} v_{j+1}, so
-//     A z_j = V_{0..j} ([b_j; d_j] + gamma_j s_{j+1}) + gamma_j gamma_{j+1} v_{j+1}:
-// Hessenberg column j becomes final at step j + 1, where its Givens step and
-// the residual test run.  The directions z_j span the same space as the
-// M v_j, and x = x_0 + Z y minimises the residual over it as in flexible
-// GMRES.  v_0 = r / ||r|| is taken as it is (gamma_0 = 1); a cycle of m
-// columns ends with a step that only finalises column m - 1 (no M, no A).
-struct DcgsArgs {
-    int j, last;
-    double2* pre;              // [nseg][m+1]: [b; d] of the previous step (column j-1 before gamma_{j-1} s_j is
-                               // added) at 0..j-1, gamma_{j-1} at m
-    double2* coef;             // [nseg][2m+2]: alpha_k = -s_k / gamma (k < j) at 0, beta_k = -(b_k - s_k d / gamma) / gamma
-                               // at m, 1 / gamma at 2m, -d / gamma^2 at 2m + 1
-    int* nact;                 // active-segment count of this step (the step's update zeroes the next one's)
-    GivensArgs g;              // rotations, R, g, targets, activity (h1 and h2 unused)
-};
-
-// Sums NV values per lane over the warp by recursive halving (NV/2 + NV/4 +
-// ... + 1 shuffles, then plain ones): lane l ends with the total of value
-// l >> (5 - log2 NV).
-template <int NV, class R>
-__device__ __forceinline__ R warp_sum_many(R (&a)[NV], int lane) {
-    int off = 16;
-#pragma unroll
-    for (int n = NV; n > 1; n >>= 1, off >>= 1) {
-        const bool up = (lane & off) != 0;
-#pragma unroll
-        for (int i = 0; i < n / 2; ++i) {
-            const R send = up ? a[i] : a[i + n / 2];
-            const R keep = up ? a[i + n / 2] : a[i];
-            a[i] = keep + __shfl_xor_sync(0xffffffffu, send, off);
-        }
-    }
-    R v = a[0];
-    for (; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
-    return v;
-}
-
-// First pass of step j: per chunk the dot products of v_0..v_{j-1} with u_j
-// and w (w = null on the finalising step), u_j^H u_j and u_j^H w; the last
-// block of each segment sums them in chunk order and runs the segment's
-// scalar step (gamma, d, Hessenberg column j-1 and its Givens step, the
-// coefficients of the second pass).  Partial layout: 2k = v_k^H u_j,
-// 2k + 1 = v_k^H w, 2j = (c1, 0), 2j + 1 = c2.
-template <class V>
-__global__ void __launch_bounds__(KT, 4) k_dcgs_dots(const Chunk* __restrict__ chunks, const V* __restrict__ basis,
-                                                  int64_t ld, const V* __restrict__ w, double2* __restrict__ partial,
-                                                  int ldp, const int* __restrict__ act, DcgsArgs da,
-                                                  unsigned long long* __restrict__ work) {
-    using R = typename VT<V>::R;
-    extern __shared__ double2 sred[];          // [2j+2][KT/32]; the last block reuses it
-    constexpr int NW = KT / 32;
-    const Chunk c = chunks[blockIdx.x];
-    if (!act[c.seg]) return;
-    const int j = da.j, nv = 2 * j + 2;
-    if (work && threadIdx.x == 0)                 // v_0..v_{j-1}, u_j and w (none on the finalising step)
-        atomicAdd(work, (unsigned long long)((j + 1 + (w ? 1 : 0)) * (c.end - c.begin) * sizeof(V)));
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const bool full = c.end - c.begin == CHUNK;
-    const V* u = basis + (int64_t)j * ld;
-    V ur[EPT], wr[EPT];
-#pragma unroll
-    for (int q = 0; q < EPT; ++q) {
-        const int64_t e = c.begin + threadIdx.x + (int64_t)q * KT;
-        const bool ok = full || e < c.end;
-        ur[q] = ok ? u[e] : mk<V>(0, 0);
-        wr[q] = (ok && w) ? w[e] : mk<V>(0, 0);
-    }
-    // warp sums in the vector precision, [2j+2][KT/32] pairs (a float pair
-    // takes half a double2 slot; the FP64 sums start at the chunk partials)
-    R* sd = reinterpret_cast<R*>(sred);
-    constexpr int KB = 4;
-    for (int k0 = 0; k0 < j; k0 += KB) {
-        V v[KB][EPT];
-#pragma unroll
-        for (int b = 0; b < KB; ++b) {
-            const V* vk = basis + (int64_t)(k0 + b) * ld;
-#pragma unroll
-            for (int q = 0; q < EPT; ++q) {
-                const int64_t e = c.begin + threadIdx.x + (int64_t)q * KT;
-                v[b][q] = mk<V>(0, 0);
-                if (k0 + b < j && (full || e < c.end)) v[b][q] = vk[e];
-            }
-        }
-        R a[4 * KB];                            // per vector: conj(v).u (re, im), conj(v).w (re, im)
-#pragma unroll
-        for (int b = 0; b < KB; ++b) {
-            a[4 * b] = a[4 * b + 1] = a[4 * b + 2] = a[4 * b + 3] = 0;
-#pragma unroll
-            for (int q = 0; q < EPT; ++q) {
-                a[4 * b] += v[b][q].x * ur[q].x + v[b][q].y * ur[q].y;
-                a[4 * b + 1] += v[b][q].x * ur[q].y - v[b][q].y * ur[q].x;
-                a[4 * b + 2] += v[b][q].x * wr[q].x + v[b][q].y * wr[q].y;
-                a[4 * b + 3] += v[b][q].x * wr[q].y - v[b][q].y * wr[q].x;
-            }
-        }
-        const R tot = warp_sum_many<4 * KB>(a, lane);
-        const int idx = lane >> 1, b = idx >> 2, comp = idx & 3;
-        if ((lane & 1) == 0 && k0 + b < j)                   // value (2(k0+b) + comp/2), component comp%2
-            sd[((2 * (k0 + b) + (comp >> 1)) * NW + warp) * 2 + (comp & 1)] = tot;
-    }
-    {
-        R a[4] = {0, 0, 0, 0};                  // u.u, 0, conj(u).w (re, im)
-#pragma unroll
-        for (int q = 0; q < EPT; ++q) {
-            a[0] += ur[q].x * ur[q].x + ur[q].y * ur[q].y;
-            a[2] += ur[q].x * wr[q].x + ur[q].y * wr[q].y;
-            a[3] += ur[q].x * wr[q].y - ur[q].y * wr[q].x;
-        }
-        const R tot = warp_sum_many<4>(a, lane);
-        const int comp = lane >> 3;
-        if ((lane & 7) == 0) sd[((2 * j + (comp >> 1)) * NW + warp) * 2 + (comp & 1)] = tot;
-    }
-    __syncthreads();
-    for (int kk = threadIdx.x; kk < nv; kk += KT) {
-        R tr = 0, ti = 0;                     // the block's sum in the vector precision, then FP64
-        for (int q = 0; q < NW; ++q) {
-            tr += sd[(kk * NW + q) * 2];
-            ti += sd[(kk * NW + q) * 2 + 1];
-        }
-        partial[(int64_t)blockIdx.x * ldp + kk] = make_double2((double)tr, (double)ti);
-    }
-    if (!last_block_of_segment(c.seg, da.g.seg_ch, da.g.cnt)) return;
-    double2* tot = sred;                        // [2j+2] segment totals
-    for (int kk = threadIdx.x; kk < nv; kk += KT) {
-        double2 t = make_double2(0, 0);
-        for (int cc = da.g.seg_ch[c.seg]; cc < da.g.seg_ch[c.seg + 1]; ++cc) t = cadd(t, __ldcg(&partial[(int64_t)cc * ldp + kk]));
-        tot[kk] = t;
-    }
-    __syncthreads();
-    // ---- the segment's scalar step, FP64, on warps 0-3 (one per SM
-    // sub-partition, so that their FP64 work runs side by side): the sums
-    // |s|^2 and s^H b, gamma and d; then warp 0 finalises Hessenberg column
-    // j-1 and its Givens step while warps 1-3 write the second pass's
-    // coefficients (harmless, and unused, if the segment stops here) ----
-    constexpr int NSC = 128;
-    if (threadIdx.x >= NSC) return;
-    __shared__ double s_red[NSC / 32][3];
-    const int sg = c.seg, m = da.g.m;
-    double ss = 0, sbr = 0, sbi = 0;            // |s|^2, s^H b
-    for (int k = threadIdx.x; k < j; k += NSC) {
-        const double2 sk = tot[2 * k], bk = tot[2 * k + 1];
-        ss += sk.x * sk.x + sk.y * sk.y;
-        sbr += sk.x * bk.x + sk.y * bk.y;
-        sbi += sk.x * bk.y - sk.y * bk.x;
-    }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        ss += __shfl_xor_sync(0xffffffffu, ss, o);
-        sbr += __shfl_xor_sync(0xffffffffu, sbr, o);
-        sbi += __shfl_xor_sync(0xffffffffu, sbi, o);
-    }
-    if (lane == 0) {
-        s_red[warp][0] = ss;
-        s_red[warp][1] = sbr;
-        s_red[warp][2] = sbi;
-    }
-    asm volatile("bar.sync 2, %0;\n" ::"n"(NSC) : "memory");
-    ss = (s_red[0][0] + s_red[1][0]) + (s_red[2][0] + s_red[3][0]);
-    sbr = (s_red[0][1] + s_red[1][1]) + (s_red[2][1] + s_red[3][1]);
-    sbi = (s_red[0][2] + s_red[1][2]) + (s_red[2][2] + s_red[3][2]);
-    const double c1 = tot[2 * j].x;
-    const double2 c2 = tot[2 * j + 1];
-    double gamma = 1.0;
-    if (j > 0) {
-        const double g2 = c1 - ss;
-        gamma = g2 > 0 ? sqrt(g2) : 0.0;        // 0: u_j lies in span(V) (a lucky breakdown)
-    }
-    if (!isfinite(c1) || !isfinite(c2.x) || !isfinite(c2.y) || !isfinite(gamma)) {
-        if (threadIdx.x == 0) {
-            atomicExch(da.g.flag, 1);
-            da.g.active[sg] = 0;
-        }
-        return;
-    }
-    double2* pre = da.pre + (int64_t)sg * (m + 1);
-    // Hessenberg column j-1: [b_{j-1}; d_{j-1}] + gamma_{j-1} s_j over gamma_{j-1} gamma_j,
-    // built from the old pre before warps 1-3 overwrite it
-    const double gp = j > 0 ? pre[m].x : 1.0;
-    double2* hin = tot + nv;
-    double2* col = hin + j;
-    for (int i = threadIdx.x; i < j; i += NSC) {
-        const double2 si = tot[2 * i];
-        hin[i] = make_double2(pre[i].x + gp * si.x, pre[i].y + gp * si.y);
-    }
-    asm volatile("bar.sync 2, %0;\n" ::"n"(NSC) : "memory");
-    if (warp == 0) {
-        if (j > 0) {
-            GivensArgs ga = da.g;
-            ga.nact = da.nact;
-            givens_core(ga, sg, j - 1, hin, gp * gamma, col, da.last != 0);
-        } else if (lane == 0) {
-            atomicAdd(da.nact, 1);              // no column yet: the segment goes on
-        }
-        return;
-    }
-    if (da.last) return;
-    const double ig = 1.0 / gamma;
-    const double2 d = make_double2((c2.x - sbr) * ig, (c2.y - sbi) * ig);
-    double2* cf = da.coef + (int64_t)sg * (2 * m + 2);
-    for (int k = threadIdx.x - 32; k < j; k += NSC - 32) {
-        const double2 sk = tot[2 * k], bk = tot[2 * k + 1];
-        pre[k] = bk;
-        cf[k] = make_double2(-sk.x * ig, -sk.y * ig);
-        const double2 sd_ = make_double2((sk.x * d.x - sk.y * d.y) * ig, (sk.x * d.y + sk.y * d.x) * ig);
-        cf[m + k] = make_double2(-(bk.x - sd_.x) * ig, -(bk.y - sd_.y) * ig);
-    }
-    if (threadIdx.x == 32) {
-        pre[j] = d;
-        pre[m] = make_double2(gamma, 0.0);
-        cf[2 * m] = make_double2(ig, 0.0);
-        cf[2 * m + 1] = make_double2(-d.x * ig * ig, -d.y * ig * ig);
-    }
-}
-
-// Second pass of step j: v_j = u_j / gamma + sum_k alpha_k v_k over slot j and
-// u_{j+1} = w / gamma - (d / gamma^2) u_j + sum_k beta_k v_k into slot j + 1.
-// Block 0 first zeroes the active count of the next step.
-template <class V>
-__global__ void __launch_bounds__(KT, 4) k_dcgs_update(const Chunk* __restrict__ chunks, V* __restrict__ basis,
-                                                    int64_t ld, int j, int m, const V* __restrict__ w,
-                                                    const double2* __restrict__ coef, const int* __restrict__ act,
-                                                    int* __restrict__ nact_next, unsigned long long* __restrict__ work) {
-    using R = typename VT<V>::R;
-    using C2 = V;                              // coefficient pairs in the vector precision
-    extern __shared__ double2 sc_raw[];        // [2j+2]: alpha_k, beta_k, 1/gamma, -d/gamma^2
-    C2* sc = reinterpret_cast<C2*>(sc_raw);
-    if (blockIdx.x == 0 && threadIdx.x == 0) *nact_next = 0;
-    const Chunk c = chunks[blockIdx.x];
-    if (!act[c.seg]) return;
-    if (work && threadIdx.x == 0)                 // v_0..v_{j-1}, u_j, w read; v_j (j > 0) and u_{j+1} written
-        atomicAdd(work, (unsigned long long)((j + 2 + (j > 0 ? 2 : 1)) * (c.end - c.begin) * sizeof(V)));
-    // the coefficients are rounded to the vector precision once per block
-    // (a double-to-float conversion per use would run on the slow FP64 path)
-    const double2* cf = coef + (int64_t)c.seg * (2 * m + 2);
-    for (int k = threadIdx.x; k < j; k += KT) {
-        sc[k] = mk<V>((R)cf[k].x, (R)cf[k].y);
-        sc[j + k] = mk<V>((R)cf[m + k].x, (R)cf[m + k].y);
-    }
-    if (threadIdx.x == 0) {
-        sc[2 * j] = mk<V>((R)cf[2 * m].x, (R)cf[2 * m].y);
-        sc[2 * j + 1] = mk<V>((R)cf[2 * m + 1].x, (R)cf[2 * m + 1].y);
-    }
-    __syncthreads();
-    const bool full = c.end - c.begin == CHUNK;
-    V* u = basis + (int64_t)j * ld;
-    V* un = basis + (int64_t)(j + 1) * ld;
-    const R cv = sc[2 * j].x, cur = sc[2 * j + 1].x, cui = sc[2 * j + 1].y;
-    R xr[EPT], xi[EPT], yr[EPT], yi[EPT];       // v_j and u_{j+1}
-#pragma unroll
-    for (int q = 0; q < EPT; ++q) {
-        const int64_t e = c.begin + threadIdx.x + (int64_t)q * KT;
-        const bool ok = full || e < c.end;
-        const V a = ok ? u[e] : mk<V>(0, 0), b = ok ? w[e] : mk<V>(0, 0);
-        xr[q] = cv * a.x;
-        xi[q] = cv * a.y;
-        yr[q] = cv * b.x + cur * a.x - cui * a.y;
-        yi[q] = cv * b.y + cur * a.y + cui * a.x;
-    }
-    constexpr int KB = 4;
-    for (int k0 = 0; k0 < j; k0 += KB) {
-        V v[KB][EPT];
-#pragma unroll
-        for (int b = 0; b < KB; ++b) {
-            const V* vk = basis + (int64_t)(k0 + b) * ld;
-#pragma unroll
-            for (int q = 0; q < EPT; ++q) {
-                const int64_t e = c.begin + threadIdx.x + (int64_t)q * KT;
-                v[b][q] = mk<V>(0, 0);
-                if (k0 + b < j && (full || e < c.end)) v[b][q] = vk[e];
-            }
-        }
-#pragma unroll
-        for (int b = 0; b < KB; ++b) {
-            const int kk = min(k0 + b, j - 1);
-            const bool in = k0 + b < j;
-            const C2 al = sc[kk], be = sc[j + kk];
-            const R ar = in ? al.x : (R)0, ai = in ? al.y : (R)0;
-            const R br = in ? be.x : (R)0, bi = in ? be.y : (R)0;
-#pragma unroll
-            for (int q = 0; q < EPT; ++q) {
-                xr[q] += ar * v[b][q].x - ai * v[b][q].y;
-                xi[q] += ar * v[b][q].y + ai * v[b][q].x;
-                yr[q] += br * v[b][q].x - bi * v[b][q].y;
-                yi[q] += br * v[b][q].y + bi * v[b][q].x;
-            }
-        }
-    }
-#pragma unroll
-    for (int q = 0; q < EPT; ++q) {
-        const int64_t e = c.begin + threadIdx.x + (int64_t)q * KT;
-        if (full || e < c.end) {
-            if (j > 0) u[e] = mk<V>(xr[q], xi[q]);
-            un[e] = mk<V>(yr[q], yi[q]);
-        }
-    }
-}
-
-// y = R^{-1} g (upper triangular, k = kused[s]), one warp per segment, by
-// columns: y_q = g_q / R_qq, then g_i -= R_iq y_q for i < q (column q of R is
-// contiguous).  The updated g lives in shared memory.
 __global__ void __launch_bounds__(32) k_backsolve(int nseg, int m, const double2* __restrict__ Rm,
                                                   const double2* __restrict__ gv, const int* __restrict__ kused,
                                                   double2* __restrict__ y) {
-    extern __shared__ double2 gsh[];           // [m]
-    const int s = blockIdx.x, lane = threadIdx.x;
-    if (s >= nseg) return;
-    const int k = kused[s];
-    const double2* R = Rm + (int64_t)s * m * m;          // R[col * m + row]
-    for (int i = lane; i < k; i += 32) gsh[i] = gv[(int64_t)s * (m + 1) + i];
-    __syncwarp();
-    for (int q = k - 1; q >= 0; --q) {
-        const double2 d = R[(int64_t)q * m + q];
-        const double2 a = gsh[q];
-        const double den = d.x * d.x + d.y * d.y;
-        const double2 yq = den > 0 ? make_double2((a.x * d.x + a.y * d.y) / den, (a.y * d.x - a.x * d.y) / den)
-                                   : make_double2(0, 0);
-        if (lane == 0) y[(int64_t)s * m + q] = yq;
-        for (int i = lane; i < q; i += 32) {
-            const double2 r = R[(int64_t)q * m + i];
-            gsh[i].x -= r.x * yq.x - r.y * yq.y;
-            gsh[i].y -= r.x * yq.y + r.y * yq.x;
-        }
-        __syncwarp();
-    }
+    extern __shared__ double2 gsh[];           // [2m]
+    const int s = blockIdx.x;
+    if (s < nseg) backsolve(m, kused[s], Rm + (int64_t)s * m * m, gv + (int64_t)s * (m + 1), gsh, y + (int64_t)s * m, threadIdx.x);
 }
 
 // Right-hand side of every subdomain: sources + sum of received interface data.
@@ -637,75 +172,31 @@ __global__ void k_norm2_blocks(int64_t n, const double2* __restrict__ x, double*
     }
 }
 
-// Mixed-precision refinement of the subdomain solves: a subdomain stays
-// active while its FP64 residual is above tol * ||b_s|| and still falling.
-__global__ void k_ir_mask(int nseg, double tol, int first, const double* __restrict__ bn2,
-                          const double* __restrict__ rn2, double* __restrict__ prev, int* __restrict__ active,
-                          int* __restrict__ nact) {
-    int s = blockIdx.x * blockDim.x + threadIdx.x;
-    if (s >= nseg) return;
-    double rn = sqrt(rn2[s]), bn = sqrt(bn2[s]);
-    if (first) prev[s] = INFINITY;
-    int a = rn > tol * bn && rn < 0.5 * prev[s];
-    prev[s] = rn;
-    active[s] = a;
-    if (a) atomicAdd(nact, 1);
-}
-
-__global__ void k_ir_to_f32(const Chunk* __restrict__ chunks, const int* __restrict__ active,
-                            const double2* __restrict__ r, float2* __restrict__ r32) {
-    const Chunk c = chunks[blockIdx.x];
-    const int a = active[c.seg];
-    for (int64_t e = c.begin + threadIdx.x; e < c.end; e += blockDim.x) {
-        double2 v = r[e];
-        r32[e] = a ? make_float2((float)v.x, (float)v.y) : make_float2(0.f, 0.f);
-    }
-}
-
-__global__ void k_ir_update(int64_t n, const float2* __restrict__ d, double2* __restrict__ x) {
-    int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (i < n) {
-        float2 v = d[i];
-        double2 u = x[i];
-        x[i] = make_double2(u.x + (double)v.x, u.y + (double)v.y);
-    }
-}
-
 static inline unsigned nblk(int64_t n, int th = 256) { return (unsigned)((n + th - 1) / th); }
 
 // ---------------------------------------------------------------------------
-// Batched restarted GMRES over segments (subdomains, or the one interface
-// segment), right-preconditioned, classical Gram-Schmidt with one full
-// re-orthogonalisation (CGS2), Givens rotations in FP64.
+// Restarted GMRES on the interface system, one segment per problem: classical
+// Gram-Schmidt with one full re-orthogonalisation (CGS2), Givens rotations in
+// FP64.
 // ---------------------------------------------------------------------------
 struct KStats {
     int64_t iters = 0;       // sum over segments of Arnoldi steps
-    int64_t dof_iters = 0;   // sum over segments of n_s * steps
-    int max_iters = 0;       // largest per-segment count of this solve
     int status = THM_OK;
 };
 
-template <class V>
 struct Krylov {
+    using V = double2;
     int64_t n = 0;
     int nseg = 0, m = 0, nch = 0;
-    const Chunk* d_chunks = nullptr;
-    DArr<Chunk> own_chunks;
+    DArr<Chunk> d_chunks;
     DArr<int32_t> seg_ch;
-    std::vector<int64_t> seg_n;
-    DArr<V> basis, w, z, r, t;
-    DArr<V> zbasis;            // flexible variant: Z_j = M v_j (x = Z y)
-    bool flexible = false;
+    DArr<V> basis, w, r, t;
     DArr<double2> partial, h1, h2, Rm, sn, gv, y;
     DArr<double> nrm_part, nrm, cs, beta, target, prev;
     DArr<int> active, kused, cnt;
-    // monitor record of the latest Arnoldi step, 32 bytes: two active-segment
-    // counts (the CGS2 steps use the first; the DCGS2 steps alternate between
-    // them, each step's update zeroing the next one's), the breakdown flag,
-    // then g_{j+1} of segment 0
+    // monitor record of the latest Arnoldi step, 32 bytes: the active-segment
+    // count, unused, the breakdown flag, then g_{j+1} of segment 0
     DArr<double2> mon;
-    DArr<double2> pre, coef;   // DCGS2: previous step's [b; d] and the second pass's coefficients
-    bool dcgs = false;
     unsigned long long* work = nullptr;   // [2]: dot-product and update pass bytes (the system's counters), or null
     int* nact = nullptr;
     int* flag = nullptr;
@@ -719,7 +210,7 @@ struct Krylov {
     double2* h_ring = nullptr;       // [RING][2] copies of the monitor record
     double h_beta0 = 0;              // ||r_0|| of segment 0 at the first cycle
     double last_rel = 1.0;           // latest residual estimate of segment 0 seen by the host, relative
-    const int* step_mask = nullptr;  // device per-segment activity while an Arnoldi step applies A and M
+    bool fresh = false;              // wait for each step's record before the next step (the operator uses last_rel)
     cudaEvent_t ring_ev[RING] = {};
 
     ~Krylov() {
@@ -729,25 +220,15 @@ struct Krylov {
             if (e) cudaEventDestroy(e);
     }
 
-    void init(int64_t n_, int nseg_, int m_, const std::vector<Chunk>& chunks, const Chunk* dch,
-              const std::vector<int64_t>& segn, bool flexible_ = false) {
+    void init(int64_t n_, int nseg_, int m_, const std::vector<Chunk>& chunks) {
         n = n_; nseg = nseg_; m = m_; nch = (int)chunks.size();
-        flexible = flexible_;
-        dcgs = flexible && !(getenv("THM_GS") && std::string(getenv("THM_GS")) == "cgs2");
-        if (flexible) zbasis.alloc((size_t)m * n);
-        if (dcgs) {
-            pre.alloc((size_t)nseg_ * (m_ + 1));
-            coef.alloc((size_t)nseg_ * (2 * m_ + 2));
-        }
-        seg_n = segn;
-        if (dch) d_chunks = dch;
-        else { own_chunks.upload(chunks); d_chunks = own_chunks.p; }
+        d_chunks.upload(chunks);
         std::vector<int32_t> sc(nseg + 1, 0);
         for (const Chunk& c : chunks) sc[c.seg + 1]++;
         for (int s = 0; s < nseg; ++s) sc[s + 1] += sc[s];
         seg_ch.upload(sc);
         basis.alloc((size_t)(m + 1) * n);
-        w.alloc(n); z.alloc(n); r.alloc(n); t.alloc(n);
+        w.alloc(n); r.alloc(n); t.alloc(n);
         partial.alloc((size_t)nch * (2 * m + 2));
         h1.alloc((size_t)nseg * (m + 1)); h2.alloc((size_t)nseg * (m + 1));
         Rm.alloc((size_t)nseg * m * m);
@@ -767,17 +248,10 @@ struct Krylov {
             THM_CUDA(cudaMallocHost(&h_ring, 2 * RING * sizeof(double2)));
             for (auto& e : ring_ev) THM_CUDA(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
         }
-        // the kernels are shared by every Krylov instance of this vector
-        // type (inner and outer solvers): only ever raise their limit
+        // the kernels are shared by every instance: only ever raise their limit
         size_t dots_smem = (size_t)(m + 1) * (KT / 32) * sizeof(double2);
-        THM_REQUIRE((dcgs ? dcgs_smem(m) : dots_smem) <= 200 * 1024, "restart length too large");
-        static size_t dots_attr = 0, dcgs_attr = 0;
-        if (dcgs && dcgs_smem(m) > dcgs_attr) {
-            THM_CUDA(cudaFuncSetAttribute(k_dcgs_dots<V>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dcgs_smem(m)));
-            THM_CUDA(cudaFuncSetAttribute(k_dcgs_update<V>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                          (int)((2 * m + 2) * sizeof(double2))));
-            dcgs_attr = dcgs_smem(m);
-        }
+        THM_REQUIRE(dots_smem <= 200 * 1024, "restart length too large");
+        static size_t dots_attr = 0;
         if (dots_smem > dots_attr) {
             THM_CUDA(cudaFuncSetAttribute(k_chunk_dots<V>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dots_smem));
             THM_CUDA(cudaFuncSetAttribute(k_update_givens<V>, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -789,16 +263,13 @@ struct Krylov {
     }
 
     void seg_norm2(const V* x, cudaStream_t st) {
-        THM_LAUNCH(THM_K_KRYLOV, st, k_chunk_norm2<V><<<nch, KT, 0, st>>>(d_chunks, x, nrm_part.p));
+        THM_LAUNCH(THM_K_KRYLOV, st, k_chunk_norm2<V><<<nch, KT, 0, st>>>(d_chunks.p, x, nrm_part.p));
         THM_LAUNCH(THM_K_KRYLOV, st, k_seg_reduce_real<<<nblk(nseg), 256, 0, st>>>(nseg, seg_ch.p, nrm_part.p, nrm.p));
     }
 
     // dynamic shared memory of k_update_givens at step j <= m-1: the nk = j+1
     // coefficients, or the Givens column and its rotated copy
     static size_t givens_smem(int mm) { return 2 * (size_t)mm * sizeof(double2); }
-    // dynamic shared memory of k_dcgs_dots at step j <= m: the warp sums of
-    // its 2j + 2 dot products (the last block reuses them for the scalar step)
-    static size_t dcgs_smem(int j) { return (size_t)(2 * j + 2) * (KT / 32) * sizeof(double2); }
 
     unsigned long long* kw(int k) const { return work ? work + k : nullptr; }
 
@@ -808,21 +279,14 @@ struct Krylov {
         return h_pinned[0];
     }
 
-    // Solve A x = b for all segments (x in/out).  A(in, out); M(in, out) or empty.
-    KStats solve(const std::function<void(const V*, V*)>& A, const std::function<void(const V*, V*)>& M,
-                 const V* b, V* x, bool x_zero, double tol, int maxit, cudaStream_t st, bool single_cycle = false) {
+    // Solve A x = b for all segments, from x = 0.  A(in, out).
+    KStats solve(const std::function<void(const V*, V*)>& A, const V* b, V* x, double tol, int maxit, cudaStream_t st) {
         KStats ks;
-        std::vector<int64_t> per_seg(nseg, 0);
         int total = 0;
         bool first = true;
         THM_CUDA(cudaMemsetAsync(flag, 0, sizeof(int), st));
-        if (x_zero) {
-            THM_CUDA(cudaMemsetAsync(x, 0, n * sizeof(V), st));
-            THM_CUDA(cudaMemcpyAsync(r.p, b, n * sizeof(V), cudaMemcpyDeviceToDevice, st));
-        } else {
-            A(x, w.p);
-            THM_LAUNCH(THM_K_KRYLOV, st, k_sub<V><<<nblk(n), 256, 0, st>>>(n, b, w.p, r.p));
-        }
+        THM_CUDA(cudaMemsetAsync(x, 0, n * sizeof(V), st));
+        THM_CUDA(cudaMemcpyAsync(r.p, b, n * sizeof(V), cudaMemcpyDeviceToDevice, st));
         while (true) {
             seg_norm2(r.p, st);
             THM_CUDA(cudaMemsetAsync(nact, 0, sizeof(int), st));
@@ -838,18 +302,19 @@ struct Krylov {
             first = false;
             if (read_nact(st) == 0) break;
             if (total >= maxit) { ks.status = THM_ENOCONV; break; }
-            THM_LAUNCH(THM_K_KRYLOV, st, k_chunk_scale<V><<<nch, 256, 0, st>>>(d_chunks, r.p, beta.p, basis.p, nullptr));
+            THM_LAUNCH(THM_K_KRYLOV, st, k_chunk_scale<V><<<nch, 256, 0, st>>>(d_chunks.p, r.p, beta.p, basis.p, nullptr));
             int j = 0, checked = 0;
             // the monitor record of step jj is in the ring; true when the host
             // has seen every segment stop or a breakdown (reads run a few
             // steps behind the GPU and block only when the ring is full)
-            auto monitor = [&](int jj, int cnt_slot_of_step) -> bool {
+            auto monitor = [&](int jj) -> bool {
                 const int slot = jj % RING;
                 THM_CUDA(cudaMemcpyAsync(h_ring + 2 * slot, mon.p, 2 * sizeof(double2), cudaMemcpyDeviceToHost, st));
                 THM_CUDA(cudaEventRecord(ring_ev[slot], st));
                 while (checked <= jj) {
                     const int rs_ = checked % RING;
-                    cudaError_t q = (jj - checked >= RING - 1) ? cudaEventSynchronize(ring_ev[rs_]) : cudaEventQuery(ring_ev[rs_]);
+                    cudaError_t q = (fresh || jj - checked >= RING - 1) ? cudaEventSynchronize(ring_ev[rs_])
+                                                                        : cudaEventQuery(ring_ev[rs_]);
                     if (q == cudaErrorNotReady) break;
                     THM_CUDA(q);
                     const int* rec = reinterpret_cast<const int*>(h_ring + 2 * rs_);
@@ -858,107 +323,75 @@ struct Krylov {
                         const double2 g1 = h_ring[2 * rs_ + 1];
                         last_rel = std::hypot(g1.x, g1.y) / h_beta0;
                     }
-                    if (rec[cnt_slot_of_step < 0 ? 0 : (checked & 1)] == 0) return true;
+                    if (rec[0] == 0) return true;
                     ++checked;
                 }
                 return false;
             };
-            if (dcgs && M) {
-                // DCGS2 steps 0..m (step m, or the step after the iteration
-                // cap, only finalises the last column)
-                THM_CUDA(cudaMemsetAsync(nact, 0, 2 * sizeof(int), st));
-                for (; j <= m; ++j) {
-                    const bool last = j == m || total >= maxit;
-                    V* uj = basis.p + (int64_t)j * n;
-                    if (!last) {
-                        V* zj = zbasis.p + (int64_t)j * n;
-                        step_mask = active.p;
-                        M(uj, zj);
-                        A(zj, w.p);
-                        step_mask = nullptr;
-                    }
-                    GivensArgs ga{j, m, m + 1, nullptr, nullptr, Rm.p, cs.p, sn.p, gv.p, target.p, active.p, kused.p,
-                                  beta.p, nact, flag, nullptr, seg_ch.p, cnt.p};
-                    DcgsArgs da{j, last ? 1 : 0, pre.p, coef.p, nact + (j & 1), ga};
-                    THM_LAUNCH(THM_K_DOTS, st, k_dcgs_dots<V><<<nch, KT, dcgs_smem(j), st>>>(d_chunks, basis.p, n,
-                                                                                             last ? nullptr : w.p,
-                                                                                             partial.p, 2 * m + 2,
-                                                                                             active.p, da, kw(0)));
-                    if (!last) {
-                        THM_LAUNCH(THM_K_UPDATE, st, k_dcgs_update<V><<<nch, KT, (size_t)(2 * j + 2) * sizeof(double2), st>>>(
-                                                         d_chunks, basis.p, n, j, m, w.p, coef.p, active.p,
-                                                         nact + ((j + 1) & 1), kw(1)));
-                        ++total;
-                    }
-                    if (monitor(j, 1) || last) break;
-                }
-                ++j;                        // steps 0..j-1 ran: the drain below reads them all
-            } else
             for (; j < m && total < maxit; ++j) {
                 V* vj = basis.p + (int64_t)j * n;
-                const V* zin = vj;
-                V* zj = flexible ? zbasis.p + (int64_t)j * n : z.p;
-                // inside the Arnoldi steps the operators and the step kernels skip
-                // segments that have converged (their columns are final)
-                step_mask = active.p;
-                if (M) { M(vj, zj); zin = zj; }
-                A(zin, w.p);
-                step_mask = nullptr;
+                A(vj, w.p);
                 const int nk = j + 1;
                 size_t sm = (size_t)nk * (KT / 32) * sizeof(double2);
                 // CGS2: h1 = V^H w, then w -= V h1 and h2 = V^H w in one pass, then
                 // w -= V h2 (the dot kernels reduce their segments themselves); the
                 // second update also forms ||w|| and the Givens step of each segment
-                THM_LAUNCH(THM_K_DOTS, st, k_chunk_dots<V><<<nch, KT, sm, st>>>(d_chunks, basis.p, n, nk, w.p, partial.p, m + 1,
+                THM_LAUNCH(THM_K_DOTS, st, k_chunk_dots<V><<<nch, KT, sm, st>>>(d_chunks.p, basis.p, n, nk, w.p, partial.p, m + 1,
                                                                                active.p, seg_ch.p, cnt.p, h1.p, m + 1, nact,
                                                                                kw(0)));
-                THM_LAUNCH(THM_K_UPDATE, st, k_update_dots<V><<<nch, KT, sm, st>>>(d_chunks, basis.p, n, nk, h1.p, m + 1, w.p,
+                THM_LAUNCH(THM_K_UPDATE, st, k_update_dots<V><<<nch, KT, sm, st>>>(d_chunks.p, basis.p, n, nk, h1.p, m + 1, w.p,
                                                                                   partial.p, m + 1, active.p, seg_ch.p,
                                                                                   cnt.p, h2.p, kw(1)));
                 GivensArgs ga{j, m, m + 1, h1.p, h2.p, Rm.p, cs.p, sn.p, gv.p, target.p, active.p, kused.p, beta.p,
                               nact, flag, nseg == 1 ? gmon : nullptr, seg_ch.p, cnt.p};
                 const size_t gsm = 2 * (size_t)(j + 1) * sizeof(double2);      // coefficients, or column + rotated column
-                THM_LAUNCH(THM_K_UPDATE, st, k_update_givens<V><<<nch, KT, gsm, st>>>(d_chunks, basis.p, n, nk, w.p, nrm_part.p,
+                THM_LAUNCH(THM_K_UPDATE, st, k_update_givens<V><<<nch, KT, gsm, st>>>(d_chunks.p, basis.p, n, nk, w.p, nrm_part.p,
                                                                                       active.p, ga, kw(1)));
-                THM_LAUNCH(THM_K_KRYLOV, st, k_chunk_scale<V><<<nch, 256, 0, st>>>(d_chunks, w.p, beta.p, basis.p + (int64_t)(j + 1) * n, active.p));
+                THM_LAUNCH(THM_K_KRYLOV, st, k_chunk_scale<V><<<nch, 256, 0, st>>>(d_chunks.p, w.p, beta.p, basis.p + (int64_t)(j + 1) * n, active.p));
                 ++total;
                 // monitor: one copy of the step's record into the ring
-                if (monitor(j, -1)) break;
+                if (monitor(j)) break;
             }
             // drain the monitor: any later step may still report breakdown
             THM_CUDA(cudaStreamSynchronize(st));
             for (; checked < j && ks.status != THM_EBREAKDOWN; ++checked)
                 if (reinterpret_cast<const int*>(h_ring + 2 * (checked % RING))[2]) ks.status = THM_EBREAKDOWN;
             THM_CUDA(cudaGetLastError());
-            // x += M (V y)
-            THM_LAUNCH(THM_K_KRYLOV, st, k_backsolve<<<nseg, 32, (size_t)m * sizeof(double2), st>>>(nseg, m, Rm.p, gv.p,
+            // x += V y
+            THM_LAUNCH(THM_K_KRYLOV, st, k_backsolve<<<nseg, 32, 2 * (size_t)m * sizeof(double2), st>>>(nseg, m, Rm.p, gv.p,
                                                                                                   kused.p, y.p));
-            if (flexible && M) {
-                // x += Z y: the preconditioned directions actually used by the Arnoldi process
-                THM_LAUNCH(THM_K_KRYLOV, st, k_chunk_combine<V><<<nch, KT, (size_t)m * sizeof(double2), st>>>(d_chunks, zbasis.p, n, kused.p, y.p, m, t.p));
-                THM_LAUNCH(THM_K_KRYLOV, st, k_axpy<V><<<nblk(n), 256, 0, st>>>(n, t.p, x));
-            } else {
-            THM_LAUNCH(THM_K_KRYLOV, st, k_chunk_combine<V><<<nch, KT, (size_t)m * sizeof(double2), st>>>(d_chunks, basis.p, n, kused.p, y.p, m, t.p));
-            if (M) {
-                M(t.p, z.p);
-                THM_LAUNCH(THM_K_KRYLOV, st, k_axpy<V><<<nblk(n), 256, 0, st>>>(n, z.p, x));
-            } else {
-                THM_LAUNCH(THM_K_KRYLOV, st, k_axpy<V><<<nblk(n), 256, 0, st>>>(n, t.p, x));
-            }
-            }
+            THM_LAUNCH(THM_K_KRYLOV, st, k_chunk_combine<V><<<nch, KT, (size_t)m * sizeof(double2), st>>>(d_chunks.p, basis.p, n, kused.p, y.p, m, t.p));
+            THM_LAUNCH(THM_K_KRYLOV, st, k_axpy<V><<<nblk(n), 256, 0, st>>>(n, t.p, x));
             kused.download(h_kused, st);
-            for (int s = 0; s < nseg; ++s) {
-                per_seg[s] += h_kused[s];
-                ks.iters += h_kused[s];
-                ks.dof_iters += (int64_t)h_kused[s] * seg_n[s];
-            }
-            if (ks.status == THM_EBREAKDOWN || single_cycle) break;
+            for (int s = 0; s < nseg; ++s) ks.iters += h_kused[s];
+            if (ks.status == THM_EBREAKDOWN) break;
             A(x, w.p);
             THM_LAUNCH(THM_K_KRYLOV, st, k_sub<V><<<nblk(n), 256, 0, st>>>(n, b, w.p, r.p));
         }
-        for (int s = 0; s < nseg; ++s) ks.max_iters = std::max<int>(ks.max_iters, (int)per_seg[s]);
         THM_CUDA(cudaGetLastError());
         return ks;
+    }
+};
+
+// Workspace of the subdomain solves in one precision (k_subsolve).
+template <class V>
+struct SubWork {
+    int m = 0;
+    DArr<V> basis, zbasis, w;
+    DArr<double2> partial, pre, Rm, y;
+    DArr<double> beta, target;
+    DArr<int> active, kused, flag;
+    void init(const thm_mesh* mesh, int m_) {
+        m = m_;
+        const size_t n = mesh->n_loc, ns = mesh->n_sub;
+        basis.alloc((size_t)(m + 1) * n);
+        zbasis.alloc((size_t)m * n);
+        w.alloc(n);
+        partial.alloc(ns * mesh->nd.C * (2 * m + 2));
+        pre.alloc(ns * (m + 1));
+        Rm.alloc(ns * m * m);
+        y.alloc(ns * m);
+        beta.alloc(ns); target.alloc(ns); active.alloc(ns); kused.alloc(ns); flag.alloc(1);
     }
 };
 
@@ -966,14 +399,11 @@ struct Krylov {
 struct Work {
     int m_in = 0, m_out = 0;
     bool has64 = false, has32 = false;
-    Krylov<double2> in64;
-    Krylov<float2> in32;
-    Krylov<double2> outer;
-    DArr<double2> b64, x64, src, g0, gtmp, gb, gsol, uglob, uloc, rloc, rglob, ytmp;
-    DArr<float2> b32, x32;
-    DArr<double2> r64, ytmp2;
-    DArr<double> bn2, rn2, rprev;
-    DArr<int> ir_active, nact_ir;
+    SubWork<double2> in64;
+    SubWork<float2> in32;
+    Krylov outer;
+    DArr<SolveTotals> totals;
+    DArr<double2> b64, x64, r64, src, g0, gtmp, gb, gsol, uglob, uloc, rloc, rglob, ytmp;
     DArr<double> npart;
     // per-problem norms of global vectors (batches)
     DArr<double> pnpart, pnrm;
@@ -995,36 +425,29 @@ static void ensure_work(thm_sys* s, bool fp32, int m_in, int m_out) {
     Work* w = s->w;
     unsigned long long* kw = kwork(s);
     if (w->m_in != m_in) { w->has64 = w->has32 = false; w->m_in = m_in; }
-    std::vector<int64_t> segn(m->n_sub);
-    for (int i = 0; i < m->n_sub; ++i) segn[i] = m->subs[i].n;
+    require_nd(m);
     if (!fp32 && !w->has64) {
-        w->in64.init(m->n_loc, m->n_sub, m_in, m->chunks, m->d_chunks.p, segn);
+        w->in64.init(m, m_in);
         w->has64 = true;
     }
     if (fp32 && !w->has32) {
-        w->in32.init(m->n_loc, m->n_sub, m_in, m->chunks, m->d_chunks.p, segn, true);
-        w->b32.alloc(m->n_loc); w->x32.alloc(m->n_loc);
-        w->r64.alloc(m->n_loc); w->ytmp2.alloc(m->n_loc);
-        w->bn2.alloc(m->n_sub); w->rn2.alloc(m->n_sub); w->rprev.alloc(m->n_sub);
-        w->ir_active.alloc(m->n_sub); w->nact_ir.alloc(1);
+        w->in32.init(m, m_in);
         w->has32 = true;
     }
     if (w->m_out != m_out && m->n_if > 0) {
         // one Krylov segment per problem (its contiguous range of interface
         // entries); a single problem is one segment over all of them
         std::vector<Chunk> oc;
-        std::vector<int64_t> on(m->n_prob);
         for (int p = 0; p < m->n_prob; ++p) {
             const int64_t b0 = m->n_prob > 1 ? m->prob_if_ptr[p] : 0;
             const int64_t b1 = m->n_prob > 1 ? m->prob_if_ptr[p + 1] : m->n_if;
-            on[p] = b1 - b0;
             for (int64_t b = b0; b < b1; b += CHUNK) {
                 Chunk c{};
                 c.seg = p; c.begin = b; c.end = std::min<int64_t>(b1, b + CHUNK);
                 oc.push_back(c);
             }
         }
-        w->outer.init(m->n_if, m->n_prob, m_out, oc, nullptr, on);
+        w->outer.init(m->n_if, m->n_prob, m_out, oc);
         w->m_out = m_out;
     }
     if (m->n_prob > 1 && w->pnrm.n == 0) {
@@ -1036,18 +459,17 @@ static void ensure_work(thm_sys* s, bool fp32, int m_in, int m_out) {
         w->pnrm.alloc(m->n_prob);
     }
     if (w->b64.n == 0) {
-        w->b64.alloc(m->n_loc); w->x64.alloc(m->n_loc); w->src.alloc(m->n_loc);
+        w->b64.alloc(m->n_loc); w->x64.alloc(m->n_loc); w->r64.alloc(m->n_loc); w->src.alloc(m->n_loc);
+        w->totals.alloc(1);
         w->uloc.alloc(m->n_loc); w->rloc.alloc(m->n_loc); w->ytmp.alloc(m->n_loc);
         size_t ni = m->n_if > 0 ? m->n_if : 1;
         w->g0.alloc(ni); w->gtmp.alloc(ni); w->gb.alloc(ni); w->gsol.alloc(ni);
         w->uglob.alloc(m->n_dof); w->rglob.alloc(m->n_dof);
         w->npart.alloc(1024);
     }
-    // Gram-Schmidt pass bytes of every Krylov process go to the counters of
-    // its precision (the interface GMRES is FP64)
-    w->in64.work = kw + 1;
-    w->in32.work = kw + 5;
+    // the interface GMRES counts its Gram-Schmidt bytes as FP64
     w->outer.work = kw + 1;
+    THM_CUDA(cudaMemsetAsync(w->totals.p, 0, sizeof(SolveTotals), s->st));
 }
 
 
@@ -1084,10 +506,8 @@ static inline void bv_arrays(const thm_sys* s, const float*, const float** g, co
     *sg = s->m->dim == 3 ? s->bvs32.p : nullptr;
 }
 
-// act (optional): per-subdomain activity; rows of inactive subdomains are skipped.
 template <class V, class F>
-static void apply_T(const thm_sys* s, const F* val, const F* bg, const F* bs, int use_bs, const V* x, V* y,
-                    const int* act = nullptr) {
+static void apply_T(const thm_sys* s, const F* val, const F* bg, const F* bs, int use_bs, const V* x, V* y) {
     const thm_mesh* m = s->m;
     const F *bvg, *bvs;
     bv_arrays(s, val, &bvg, &bvs);
@@ -1095,21 +515,26 @@ static void apply_T(const thm_sys* s, const F* val, const F* bg, const F* bs, in
     if (m->col16)
         THM_LAUNCH(THM_K_SPMV, s->st,
                    (k_spmv<V, F, uint16_t><<<nblk(m->n_loc), 256, 0, s->st>>>(
-                       m->n_loc, m->d_slice_ptr.p, m->d_sell_col16.p, m->d_subs.p, val, bg, bs, use_bs, bvg, bvs, x, y,
-                       m->d_loc_sub.p, act, work)));
+                       m->n_loc, m->d_slice_ptr.p, m->d_sell_col16.p, m->d_subs.p, SpmvMat<F>{val, bg, bs, bvg, bvs},
+                       use_bs, x, y,
+                       m->d_loc_sub.p, work)));
     else
         THM_LAUNCH(THM_K_SPMV, s->st,
                    (k_spmv<V, F, int32_t><<<nblk(m->n_loc), 256, 0, s->st>>>(
-                       m->n_loc, m->d_slice_ptr.p, m->d_sell_col.p, m->d_subs.p, val, bg, bs, use_bs, bvg, bvs, x, y,
-                       m->d_loc_sub.p, act, work)));
+                       m->n_loc, m->d_slice_ptr.p, m->d_sell_col.p, m->d_subs.p, SpmvMat<F>{val, bg, bs, bvg, bvs},
+                       use_bs, x, y,
+                       m->d_loc_sub.p, work)));
 }
 
 // The block preconditioner of every subdomain: one cluster of nd.C CTAs each.
 // Two CTAs to an SM where their vectors fit (each hides the other's barriers
 // and L2 latency); vectors that outgrow shared memory leave the u buffers,
 // then the staged y, in a workspace of the system.
+// more: bytes that other phases of the kernel need in place of the vectors;
+// keep: bytes beside everything.  False: it does not fit (glob: with vectors
+// moved to the global workspace as need be).
 template <class V, class FW>
-static void nd_apply(const thm_sys* s, const FW* fac, const V* x, V* y, const int* act) {
+static bool nd_memory(const thm_sys* s, bool glob, size_t more, size_t keep, NdMem* out, size_t* keep_off, size_t* smem) {
     const thm_mesh* m = s->m;
     require_nd(m);
     const NdSizes& z = m->nd.z;
@@ -1117,26 +542,51 @@ static void nd_apply(const thm_sys* s, const FW* fac, const V* x, V* y, const in
         s->bt_work.alloc(4);
         s->bt_work.zero(s->st);
     }
-    int u_glob = 0, y_glob = 0;
-    const int slt_smem = (size_t)z.nslt * sizeof(int2) <= 16 * 1024 ? 1 : 0;
-    if (nd_layout<V>(z, slt_smem, 0, 0).total > ND_SMEM_MAX) u_glob = 1;
-    if (nd_layout<V>(z, slt_smem, u_glob, 0).total > ND_SMEM_MAX) y_glob = 1;
-    const size_t smem = nd_layout<V>(z, slt_smem, u_glob, y_glob).total;
-    THM_REQUIRE(smem <= ND_SMEM_MAX, "subdomain too large for the shared-memory block solve");
-    const int64_t stride = (u_glob || y_glob) ? (int64_t)z.nu[0] + z.nu[1] + z.ny : 0;
-    if (stride > 0 && s->nd_glob.n < (size_t)(stride * m->n_sub * m->nd.C)) s->nd_glob.alloc(stride * m->n_sub * m->nd.C);
-    static std::once_flag once;
-    std::call_once(once, [] {
-        THM_CUDA(cudaFuncSetAttribute(k_nd_solve<V, FW>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ND_SMEM_MAX));
-    });
-    // the work counter follows the Eq. 7 (real-factor) applies only
-    unsigned long long* work = NdCplx<FW>::value ? nullptr : s->bt_work.p + (sizeof(FW) == 4 ? 2 : 0);
-    // the wait for the table copies gives up after THM_BT_WAIT_LIMIT_MS
-    // (default 1000 ms); THM_TEST_STALL_TMA=1 holds the copies back, so that a
-    // test can see the bounded wait expire and THM_ETIMEOUT come back
+    NdMem mm{};
+    mm.slt_smem = (size_t)z.nslt * sizeof(int2) <= 16 * 1024 ? 1 : 0;
+    // L2 prefetch of the factor two levels ahead of its use where all factors
+    // together are more than a small part of L2 (129 MB), which the bases of
+    // the solves share: FP32 sweeps with 80 to 140 MB of factors 18.1 -> 17.0 ms
+    // (64 cubes of 8^3 cells) and 26.6 -> 25.6 ms (64 squares of 32^2, order 2);
+    // factors of a few MB are in L2 anyway, and asking costs 1% (4 squares of
+    // 24^2, order 2: 641 -> 648 ms a solve).
+    mm.prefetch = m->nd.fac_elems * (int64_t)sizeof(FW) >= (int64_t)16 << 20;
+    auto need = [&]() {
+        const NdLayout L = nd_layout<V>(z, mm.slt_smem, mm.u_glob, mm.y_glob);
+        return (std::max(L.total, L.vec + more) + 15) / 16 * 16 + keep;
+    };
+    if (glob) {
+        if (need() > ND_SMEM_MAX) mm.u_glob = 1;
+        if (need() > ND_SMEM_MAX) mm.y_glob = 1;
+    }
+    if ((!glob && !mm.slt_smem) || need() > ND_SMEM_MAX) return false;
+    mm.glob_stride = (mm.u_glob || mm.y_glob) ? (int64_t)z.nu[0] + z.nu[1] + z.ny : 0;
+    const size_t entries = (size_t)(mm.glob_stride * m->n_sub * m->nd.C);
+    if (s->nd_glob.n < entries) s->nd_glob.alloc(entries);
+    *out = mm;
+    *smem = need();
+    *keep_off = *smem - keep;
+    return true;
+}
+
+// The wait for a solve kernel's table copies gives up after
+// THM_BT_WAIT_LIMIT_MS (default 1000 ms); THM_TEST_STALL_TMA=1 holds the
+// copies back, so that a test can see the bounded wait expire and
+// THM_ETIMEOUT come back.
+static unsigned long long nd_wait_ns() {
     const char* lim = getenv("THM_BT_WAIT_LIMIT_MS");
-    const unsigned long long wait_ns = 1000000ull * (unsigned long long)(lim ? std::max(1, atoi(lim)) : 1000);
+    return 1000000ull * (unsigned long long)(lim ? std::max(1, atoi(lim)) : 1000);
+}
+static int nd_stall() {
     const char* stall = getenv("THM_TEST_STALL_TMA");
+    return stall && atoi(stall) != 0;
+}
+
+// Launches a solve kernel, one cluster of nd.C CTAs per subdomain.
+template <class... P, class... A>
+static void nd_launch(const thm_sys* s, int cls, void (*kernel)(P...), size_t smem, A... args) {
+    const thm_mesh* m = s->m;
+    THM_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ND_SMEM_MAX));
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3(m->nd.C, m->n_sub);
     cfg.blockDim = dim3(ND_NT);
@@ -1148,90 +598,96 @@ static void nd_apply(const thm_sys* s, const FW* fac, const V* x, V* y, const in
     at.val.clusterDim.y = at.val.clusterDim.z = 1;
     cfg.attrs = &at;
     cfg.numAttrs = 1;
-    THM_LAUNCH(THM_K_PINV, s->st,
-               THM_CUDA(cudaLaunchKernelEx(&cfg, k_nd_solve<V, FW>, nd_tables(m), z, slt_smem, u_glob, y_glob,
-                                           reinterpret_cast<V*>(s->nd_glob.p), stride, fac, wait_ns,
-                                           (int)(stall && atoi(stall) != 0), s->dev_err.p, act, work, x, y)));
+    THM_LAUNCH(cls, s->st, THM_CUDA(cudaLaunchKernelEx(&cfg, kernel, P(args)...)));
 }
 
-// The full 2x2 block preconditioner (Section 3.2's alternative): T_i^{-1} from
-// the complex factors.
-template <class V>
-static void apply_Tinv_mode(const thm_sys* s, bool f32, const V* x, V* y, const int* act = nullptr) {
-    if (f32) nd_apply<V, float2>(s, s->facc32.p, x, y, act);
-    else if constexpr (sizeof(V) == 16) nd_apply<V, double2>(s, s->facc64.p, x, y, act);
+template <class V, class FW>
+static void nd_apply(const thm_sys* s, const FW* fac, const V* x, V* y) {
+    size_t smem = 0, keep_off = 0;
+    NdMem mm{};
+    const bool glob = !nd_memory<V, FW>(s, false, 0, 0, &mm, &keep_off, &smem);
+    THM_REQUIRE(!glob || (nd_memory<V, FW>(s, true, 0, 0, &mm, &keep_off, &smem)),
+                "subdomain too large for the shared-memory block solve");
+    // the work counter follows the Eq. 7 (real-factor) applies only
+    unsigned long long* work = NdCplx<FW>::value ? nullptr : s->bt_work.p + (sizeof(FW) == 4 ? 2 : 0);
+    nd_launch(s, THM_K_PINV, glob ? k_nd_solve<true, V, FW> : k_nd_solve<false, V, FW>, smem, nd_tables(s->m), s->m->nd.z, mm, reinterpret_cast<V*>(s->nd_glob.p),
+              fac, nd_wait_ns(), nd_stall(), s->dev_err.p, work, x, y);
 }
 
-template <class V>
-static void apply_Pinv_mode(const thm_sys* s, bool f32, const V* x, V* y, const int* act = nullptr) {
-    if (f32) nd_apply<V, float>(s, s->fac32.p, x, y, act);
-    else if constexpr (sizeof(V) == 16) nd_apply<V, double>(s, s->fac64.p, x, y, act);
+// The solve totals counted on the device since prepare (or the last call).
+static void collect(thm_sys* s, RunStats& rs) {
+    SolveTotals t;
+    THM_CUDA(cudaMemcpyAsync(&t, s->w->totals.p, sizeof(t), cudaMemcpyDeviceToHost, s->st));
+    THM_CUDA(cudaStreamSynchronize(s->st));
+    THM_CUDA(cudaMemsetAsync(s->w->totals.p, 0, sizeof(t), s->st));
+    rs.inner += (int64_t)t.iters;
+    rs.dof_iters += (int64_t)t.dof_iters;
+    rs.max_inner = std::max(rs.max_inner, t.max_iters);
+    if (t.no_conv && rs.status == THM_OK) rs.status = THM_ENOCONV;
+    if (t.breakdown && rs.status == THM_OK) rs.status = THM_EBREAKDOWN;
 }
 
-static void add(RunStats& rs, const KStats& k) {
-    rs.inner += k.iters;
-    rs.dof_iters += k.dof_iters;
-    rs.max_inner = std::max(rs.max_inner, k.max_iters);
-    if (k.status != THM_OK && rs.status == THM_OK) rs.status = k.status;
-}
-
-// Solve all subdomain problems T_i x_i = b_i (b, x FP64 local vectors).
-static void subdomain_solves(thm_sys* s, const SolveCfg& c, const double2* b, double2* x, RunStats& rs) {
+template <class V, class FW, class F>
+static void subsolve(thm_sys* s, const SolveCfg& c, SubWork<V>& k, const FW* fac, const F* val, const F* bg, const F* bs,
+                     const double2* b, double2* x) {
     const thm_mesh* m = s->m;
     Work* w = s->w;
-    cudaStream_t st = s->st;
-    if (!c.fp32) {
-        auto A = [&](const double2* in, double2* out) {
-            apply_T<double2, double>(s, s->val64.p, s->bg64.p, s->bs64.p, 1, in, out, w->in64.step_mask);
-        };
-        auto M = [&](const double2* in, double2* out) {
-            if (c.precond == THM_PRECOND_FULL) apply_Tinv_mode<double2>(s, false, in, out, w->in64.step_mask);
-            else apply_Pinv_mode<double2>(s, false, in, out, w->in64.step_mask);
-        };
-        add(rs, w->in64.solve(A, M, b, x, true, c.inner_tol, c.inner_maxit, st));
+    int64_t nmax = 0;
+    for (const auto& S : m->subs) nmax = std::max(nmax, S.n);
+    const int rows = sub_rows(nmax, m->nd.C);
+    size_t smem = 0, keep_off = 0;
+    NdMem mm{};
+    const size_t keep = sub_keep_bytes(k.m);
+    // glob: u and w of the rows stay in global memory, like the apply's vectors as need be
+    const bool glob = !m->col16 ||
+                      !nd_memory<V, FW>(s, false, sub_krylov_bytes<V>(rows, k.m, 0), keep, &mm, &keep_off, &smem);
+    THM_REQUIRE(!glob || (nd_memory<V, FW>(s, true, sub_krylov_bytes<V>(rows, k.m, 1), keep, &mm, &keep_off, &smem)),
+                "restart length too large");
+    SubArgs<V, F> a{};
+    const bool f32 = sizeof(F) == 4;
+    a.m = k.m;
+    a.maxit = f32 ? k.m : c.inner_maxit;
+    a.max_cycles = std::max(1, c.inner_maxit / std::max(1, c.m_in));
+    a.tol = c.inner_tol;
+    a.cycle_tol = c.cycle_tol;
+    a.col16 = m->col16;
+    a.n = m->n_loc;
+    a.b = b; a.x = x; a.r = w->r64.p;
+    a.basis = k.basis.p; a.zbasis = k.zbasis.p; a.w = k.w.p;
+    a.partial = k.partial.p; a.pre = k.pre.p; a.y = k.y.p;
+    a.g = GivensArgs{0, k.m, k.m + 1, nullptr, nullptr, k.Rm.p, nullptr, nullptr, nullptr, k.target.p, k.active.p, k.kused.p,
+                     k.beta.p, nullptr, k.flag.p, nullptr, nullptr, nullptr};
+    a.subs = m->d_subs.p;
+    a.slice_ptr = m->d_slice_ptr.p;
+    a.col = m->d_sell_col.p;
+    a.col_rel = m->d_sell_col16.p;
+    a.A.val = val; a.A.bg = bg; a.A.bs = bs;
+    bv_arrays(s, val, &a.A.bvg, &a.A.bvs);
+    a.A64.val = s->val64.p; a.A64.bg = s->bg64.p; a.A64.bs = s->bs64.p;
+    bv_arrays(s, a.A64.val, &a.A64.bvg, &a.A64.bvs);
+    a.totals = w->totals.p;
+    a.kw64 = kwork(s);
+    a.kw = a.kw64 + (f32 ? 4 : 0);
+    a.bt = NdCplx<FW>::value ? nullptr : s->bt_work.p + (f32 ? 2 : 0);
+    nd_launch(s, THM_K_SUBSOLVE, glob ? k_subsolve<true, V, FW, F> : k_subsolve<false, V, FW, F>, smem, nd_tables(m), m->nd.z, mm, reinterpret_cast<V*>(s->nd_glob.p),
+              fac, a, (int)keep_off, nd_wait_ns(), nd_stall(), s->dev_err.p);
+}
+
+// Solve all subdomain problems T_i x_i = b_i (b, x FP64 local vectors).  Each
+// mixed cycle runs to cycle_tol relative to its own right-hand side (the FP32
+// limit), also when the refined solve needs less: with the relaxed interface
+// tolerances the margin is what keeps the interface GMRES from stalling (a
+// floor at a quarter of the subdomain tolerance took 937 interface steps
+// against 362 on the 256x256 order-2 workload, measured).
+static void subdomain_solves(thm_sys* s, const SolveCfg& c, const double2* b, double2* x) {
+    Work* w = s->w;
+    const bool full = c.precond == THM_PRECOND_FULL;
+    if (c.fp32) {
+        if (full) subsolve<float2, float2, float>(s, c, w->in32, s->facc32.p, s->val32.p, s->bg32.p, s->bs32.p, b, x);
+        else subsolve<float2, float, float>(s, c, w->in32, s->fac32.p, s->val32.p, s->bg32.p, s->bs32.p, b, x);
     } else {
-        // Mixed: GMRES-IR.  Each cycle solves T d = r in FP32 (FP32 operator,
-        // FP32 preconditioner, FP32 Krylov basis; flexible form, so d is built
-        // from the very preconditioned vectors the Arnoldi process used) to a
-        // relative 1e-5; x and the true residual r = b - T x are kept in FP64,
-        // so the subdomain solves reach the same tolerance as in FP64 mode.
-        auto A = [&](const float2* in, float2* out) {
-            apply_T<float2, float>(s, s->val32.p, s->bg32.p, s->bs32.p, 1, in, out, w->in32.step_mask);
-        };
-        auto M = [&](const float2* in, float2* out) {
-            if (c.precond == THM_PRECOND_FULL) apply_Tinv_mode<float2>(s, true, in, out, w->in32.step_mask);
-            else apply_Pinv_mode<float2>(s, true, in, out, w->in32.step_mask);
-        };
-        Krylov<float2>& K = w->in32;
-        THM_CUDA(cudaMemsetAsync(x, 0, m->n_loc * sizeof(double2), st));
-        THM_CUDA(cudaMemcpyAsync(w->r64.p, b, m->n_loc * sizeof(double2), cudaMemcpyDeviceToDevice, st));
-        // per-subdomain ||b|| -> target
-        THM_LAUNCH(THM_K_KRYLOV, st, k_chunk_norm2<double2><<<K.nch, KT, 0, st>>>(K.d_chunks, b, K.nrm_part.p));
-        THM_LAUNCH(THM_K_KRYLOV, st, k_seg_reduce_real<<<nblk(K.nseg), 256, 0, st>>>(K.nseg, K.seg_ch.p, K.nrm_part.p, w->bn2.p));
-        const int max_cycles = std::max(1, c.inner_maxit / std::max(1, c.m_in));
-        for (int cyc = 0; cyc < max_cycles; ++cyc) {
-            THM_LAUNCH(THM_K_KRYLOV, st, k_chunk_norm2<double2><<<K.nch, KT, 0, st>>>(K.d_chunks, w->r64.p, K.nrm_part.p));
-            THM_LAUNCH(THM_K_KRYLOV, st, k_seg_reduce_real<<<nblk(K.nseg), 256, 0, st>>>(K.nseg, K.seg_ch.p, K.nrm_part.p, w->rn2.p));
-            w->nact_ir.zero(st);
-            THM_LAUNCH(THM_K_DDM, st, k_ir_mask<<<nblk(K.nseg), 256, 0, st>>>(K.nseg, c.inner_tol, cyc == 0 ? 1 : 0, w->bn2.p, w->rn2.p,
-                                                  w->rprev.p, w->ir_active.p, w->nact_ir.p));
-            THM_LAUNCH(THM_K_DDM, st, k_ir_to_f32<<<K.nch, 256, 0, st>>>(K.d_chunks, w->ir_active.p, w->r64.p, w->b32.p));
-            std::vector<int> na;
-            w->nact_ir.download(na, st);
-            if (na[0] == 0) break;
-            // each cycle runs to cycle_tol relative to its own right-hand side
-            // (the FP32 limit).  It stops there even when the refined solve
-            // needs less: with the relaxed interface tolerances the margin is
-            // what keeps the interface GMRES from stalling (a floor at a
-            // quarter of the subdomain tolerance took 937 interface steps
-            // against 362 on the 256x256 order-2 workload, measured)
-            KStats ks = K.solve(A, M, w->b32.p, w->x32.p, true, c.cycle_tol, c.m_in, st, true);
-            ks.status = THM_OK;      // the refinement loop owns convergence
-            add(rs, ks);
-            THM_LAUNCH(THM_K_DDM, st, k_ir_update<<<nblk(m->n_loc), 256, 0, st>>>(m->n_loc, w->x32.p, x));
-            apply_T<double2, double>(s, s->val64.p, s->bg64.p, s->bs64.p, 1, x, w->ytmp2.p);
-            THM_LAUNCH(THM_K_KRYLOV, st, k_sub<double2><<<nblk(m->n_loc), 256, 0, st>>>(m->n_loc, b, w->ytmp2.p, w->r64.p));
-        }
+        if (full) subsolve<double2, double2, double>(s, c, w->in64, s->facc64.p, s->val64.p, s->bg64.p, s->bs64.p, b, x);
+        else subsolve<double2, double, double>(s, c, w->in64, s->fac64.p, s->val64.p, s->bg64.p, s->bs64.p, b, x);
     }
 }
 
@@ -1243,7 +699,7 @@ static void sweep(thm_sys* s, const SolveCfg& c, const double2* src, const doubl
     cudaStream_t st = s->st;
     THM_LAUNCH(THM_K_DDM, st, k_rhs<<<nblk(m->n_loc), 256, 0, st>>>(m->n_loc, src, m->d_rowg_ptr.p, m->d_rowg_idx.p,
                                           m->n_if > 0 ? g_in : nullptr, w->b64.p));
-    subdomain_solves(s, c, w->b64.p, x, rs);
+    subdomain_solves(s, c, w->b64.p, x);
     if (m->n_if > 0 && g_out)
         THM_LAUNCH(THM_K_DDM, st, k_exchange<<<nblk(m->n_if), 256, 0, st>>>(m->n_if, m->d_if_partner.p, m->d_if_ptr.p,
                                                                            m->d_if_tcol.p, s->if_val.p,
@@ -1304,19 +760,20 @@ static void ddm_solve(thm_sys* s, const SolveCfg& c, const double2* src, double2
         sweep(s, cr, nullptr, v, w->gtmp.p, w->ytmp.p, rs);
         THM_LAUNCH(THM_K_KRYLOV, st, k_sub<double2><<<nblk(m->n_if), 256, 0, st>>>(m->n_if, v, w->gtmp.p, out));   // (I - A) v
     };
-    std::function<void(const double2*, double2*)> none;
+    w->outer.fresh = c.relax != 0;
     static const bool verbose = getenv("THM_VERBOSE") != nullptr;
     std::function<void(const double2*, double2*)> Av = A;
     if (verbose) {
         Av = [&, t0 = std::chrono::steady_clock::now()](const double2* v, double2* out) {
             int64_t before = rs.inner;
             A(v, out);
+            collect(s, rs);
             double el = std::chrono::duration<double>(std::chrono::steady_clock::now() - t0).count();
             fprintf(stderr, "[thm] sweep %d: inner %lld (max %d) t=%.3fs\n", rs.sweeps,
                     (long long)(rs.inner - before), rs.max_inner, el);
         };
     }
-    KStats ko = w->outer.solve(Av, none, w->gb.p, w->gsol.p, true, c.outer_tol, c.outer_maxit, st);
+    KStats ko = w->outer.solve(Av, w->gb.p, w->gsol.p, c.outer_tol, c.outer_maxit, st);
     rs.outer += (int)ko.iters;
     if (ko.status != THM_OK && rs.status == THM_OK) rs.status = ko.status;
     sweep(s, c, src, w->gsol.p, nullptr, uloc, rs, uD);
@@ -1427,7 +884,7 @@ int solve_rhs(thm_sys* s, const SolveCfg& c, const double2* f_src, const double2
         THM_LAUNCH(THM_K_DDM, st, k_owner_split<<<nblk(m->n_loc), 256, 0, st>>>(m->n_loc, m->d_loc_gdof.p, m->d_loc_is_owner.p,
                                                                                w->rglob.p, w->src.p));
     }
-    THM_CUDA(cudaStreamSynchronize(st));
+    collect(s, rs);
     THM_CUDA(cudaGetLastError());
     check_device_error(s);
     if (rs.status == THM_EBREAKDOWN) return THM_EBREAKDOWN;
@@ -1473,9 +930,11 @@ void apply_local(thm_sys* s, int op, int mode, const double2* x, double2* y) {
         ensure_factor(s, f32);
         if (op == THM_OP_TINV) {
             ensure_factor_full(s, f32);
-            apply_Tinv_mode<double2>(s, f32, x, y);
+            if (f32) nd_apply<double2, float2>(s, s->facc32.p, x, y);
+            else nd_apply<double2, double2>(s, s->facc64.p, x, y);
         } else {
-            apply_Pinv_mode<double2>(s, f32, x, y);
+            if (f32) nd_apply<double2, float>(s, s->fac32.p, x, y);
+            else nd_apply<double2, double>(s, s->fac64.p, x, y);
         }
         THM_CUDA(cudaStreamSynchronize(s->st));
         check_device_error(s);
@@ -1494,7 +953,7 @@ int sweep_diag(thm_sys* s, const thm_solve_opts* opts, int with_sources, const d
     prepare(s, c);
     RunStats rs;
     sweep(s, c, with_sources ? s->f_loc.p : nullptr, g_in, g_out, uloc, rs, with_sources ? s->uD.p : nullptr);
-    THM_CUDA(cudaStreamSynchronize(s->st));
+    collect(s, rs);
     if (stats) {
         memset(stats, 0, sizeof(*stats));
         stats->sweeps = rs.sweeps;
