@@ -382,6 +382,7 @@ struct SubWork {
     DArr<double> beta, target;
     DArr<int> active, kused, flag;
     void init(const thm_mesh* mesh, int m_) {
+        THM_REQUIRE(m_ < (sizeof(V) == 8 ? 800 : 1600), "restart length too large");
         m = m_;
         const size_t n = mesh->n_loc, ns = mesh->n_sub;
         basis.alloc((size_t)(m + 1) * n);
@@ -637,16 +638,22 @@ static void subsolve(thm_sys* s, const SolveCfg& c, SubWork<V>& k, const FW* fac
     const int rows = sub_rows(nmax, m->nd.C);
     size_t smem = 0, keep_off = 0;
     NdMem mm{};
-    const size_t keep = sub_keep_bytes(k.m);
-    // glob: u and w of the rows stay in global memory, like the apply's vectors as need be
-    const bool glob = !m->col16 ||
-                      !nd_memory<V, FW>(s, false, sub_krylov_bytes<V>(rows, k.m, 0), keep, &mm, &keep_off, &smem);
-    THM_REQUIRE(!glob || (nd_memory<V, FW>(s, true, sub_krylov_bytes<V>(rows, k.m, 1), keep, &mm, &keep_off, &smem)),
-                "restart length too large");
+    // glob: u and w of the rows stay in global memory, like the apply's vectors
+    // as need be.  A restart length whose scalars outgrow shared memory (about
+    // 1,000) is cut to what fits: such a cycle restarts there.
+    int mr = k.m;
+    bool glob = false;
+    while (true) {
+        const size_t keep = sub_keep_bytes(mr);
+        glob = !m->col16 || !nd_memory<V, FW>(s, false, sub_krylov_bytes<V>(rows, mr, 0), keep, &mm, &keep_off, &smem);
+        if (!glob || nd_memory<V, FW>(s, true, sub_krylov_bytes<V>(rows, mr, 1), keep, &mm, &keep_off, &smem)) break;
+        THM_REQUIRE(mr > 128, "subdomain too large for the shared-memory block solve");
+        mr -= 64;
+    }
     SubArgs<V, F> a{};
     const bool f32 = sizeof(F) == 4;
-    a.m = k.m;
-    a.maxit = f32 ? k.m : c.inner_maxit;
+    a.m = mr;
+    a.maxit = f32 ? mr : c.inner_maxit;
     a.max_cycles = std::max(1, c.inner_maxit / std::max(1, c.m_in));
     a.tol = c.inner_tol;
     a.cycle_tol = c.cycle_tol;
@@ -655,7 +662,7 @@ static void subsolve(thm_sys* s, const SolveCfg& c, SubWork<V>& k, const FW* fac
     a.b = b; a.x = x; a.r = w->r64.p;
     a.basis = k.basis.p; a.zbasis = k.zbasis.p; a.w = k.w.p;
     a.partial = k.partial.p; a.pre = k.pre.p; a.y = k.y.p;
-    a.g = GivensArgs{0, k.m, k.m + 1, nullptr, nullptr, k.Rm.p, nullptr, nullptr, nullptr, k.target.p, k.active.p, k.kused.p,
+    a.g = GivensArgs{0, mr, mr + 1, nullptr, nullptr, k.Rm.p, nullptr, nullptr, nullptr, k.target.p, k.active.p, k.kused.p,
                      k.beta.p, nullptr, k.flag.p, nullptr, nullptr, nullptr};
     a.subs = m->d_subs.p;
     a.slice_ptr = m->d_slice_ptr.p;
