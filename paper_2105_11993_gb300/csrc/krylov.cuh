@@ -17,6 +17,7 @@ struct GivensArgs {
     double* cs;
     double2* sn;
     double2* gv;
+    double2 *pp, *pq, *ip;     // [m+1] p_i, [m] c_i / p_{i+1}, [1] 1 / p_j of the rotations so far (givens_core)
     const double* target;
     int* active;
     int* kused;
@@ -38,20 +39,25 @@ __device__ __forceinline__ double2 gv_fma(double2 a, double2 b, double2 c) {    
 // One warp.  Applying the previous rotations to the new column is a chain:
 // with a_0 = h_0 and, for i < j,
 //     r_i     = c_i a_i + s_i h_{i+1}               (entry i of the rotated column)
-//     a_{i+1} = -conj(s_i) a_i + c_i h_{i+1}         (carried into rotation i + 1)
-// the carry follows the affine maps a -> A_i a + B_i (A_i = -conj(s_i),
-// B_i = c_i h_{i+1}), which compose associatively.  Each lane composes the
-// maps of its range of i, a shuffle scan gives every lane the composition of
-// the ranges below it (so its incoming carry), and the lanes then walk their
-// ranges in parallel.  FP64 instructions cost a full warp slot on this part
-// whatever the active lanes, so the serial chain of about 12 of them per
-// rotation on one lane becomes about (j / 32) * 16 + 5 * 8 per lane.
+//     a_{i+1} = A_i a_i + c_i h_{i+1}, A_i = -conj(s_i)  (carried into rotation i + 1).
+// With the products p_i = A_0 .. A_{i-1}, which do not depend on the column
+// and grow by one factor a step,
+//     a_i = p_i (h_0 + sum_{k<i} (c_k / p_{k+1}) h_{k+1}),
+// so the chain is a prefix sum over the lanes.  (Every term p_i c_k / p_{k+1}
+// is at most 1 in magnitude, so the sum is as stable as the rotations; p_i
+// falls like the residual and 1 / p_i is formed beside it, by products.)
+// FP64 instructions cost a warp 64 cycles here whatever its active lanes:
+// a scan that composes the maps a -> A_i a + B_i took 40 of them where this
+// takes 10, and the two square roots run as one on two lanes.  With the scalar
+// step's own chain shortened (rsqrt for square root and division, the sums by
+// halving, the last step's scalars in shared memory), subdomain solves before
+// and after: 2.19 -> 2.07 ms (3^3-cell subdomains), 1.94 -> 1.88 ms (16^2,
+// FP64), 4.61 -> 4.53 ms (24^2, order 2).
 // Column j of segment s: hin[0..j] (shared memory, unrotated), hn = the
-// subdiagonal entry (||w||); the rotated column goes to col[0..j] (shared
-// memory, another array) and to R.  stop: the segment stops after this
-// column whatever its residual (the last column of a cycle).
-__device__ bool givens_core(const GivensArgs& ga, int s, int j, const double2* hin, double hn, double2* col,
-                            bool stop = false) {
+// subdiagonal entry (||w||), ihn = 1 / hn; the rotated column goes to R.
+// stop: the segment stops after this column whatever its residual (the last
+// column of a cycle).
+__device__ bool givens_core(const GivensArgs& ga, int s, int j, const double2* hin, double hn, double ihn, bool stop = false) {
     const int m = ga.m;
     const int lane = threadIdx.x & 31;
     if (!isfinite(hn)) {
@@ -64,78 +70,71 @@ __device__ bool givens_core(const GivensArgs& ga, int s, int j, const double2* h
     }
     const double* cs = ga.cs + (int64_t)s * m;
     const double2* sn = ga.sn + (int64_t)s * m;
-    const double2 h0 = hin[0];
+    double2* pp = ga.pp + (int64_t)s * (m + 1);
+    double2* pq = ga.pq + (int64_t)s * m;
+    double2* g = ga.gv + (int64_t)s * (m + 1);
+    const double t = ga.target[s];
+    const double2 h0 = hin[0], gj = g[j];
+    const double2 pj = j > 0 ? pp[j] : make_double2(1, 0), ipj = j > 0 ? ga.ip[s] : make_double2(1, 0);
     const int per = (j + 31) / 32;
     const int b = min(j, lane * per), e = min(j, b + per);
-    // this lane's maps composed: (A, B) = M_{e-1} o ... o M_b
-    double2 A = make_double2(1, 0), B = make_double2(0, 0);
-    for (int i = b; i < e; ++i) {
-        const double2 Ai = make_double2(-sn[i].x, sn[i].y);
-        const double2 hi1 = hin[i + 1];
-        const double2 Bi = make_double2(cs[i] * hi1.x, cs[i] * hi1.y);
-        B = gv_fma(Ai, B, Bi);
-        A = gv_mul(Ai, A);
-    }
-    // inclusive scan over the lanes: (A, B) <- (A, B) o (A, B) of lane - d
-#pragma unroll 1
+    // the terms of this lane's range, and of the ranges below it
+    double2 L = make_double2(0, 0);
+    for (int i = b; i < e; ++i) L = gv_fma(pq[i], hin[i + 1], L);
+#pragma unroll
     for (int d = 1; d < 32; d <<= 1) {
-        const double2 Ao = make_double2(__shfl_up_sync(0xffffffffu, A.x, d), __shfl_up_sync(0xffffffffu, A.y, d));
-        const double2 Bo = make_double2(__shfl_up_sync(0xffffffffu, B.x, d), __shfl_up_sync(0xffffffffu, B.y, d));
-        if (lane >= d) {
-            B = gv_fma(A, Bo, B);
-            A = gv_mul(A, Ao);
-        }
+        const double2 o = make_double2(__shfl_up_sync(0xffffffffu, L.x, d), __shfl_up_sync(0xffffffffu, L.y, d));
+        if (lane >= d) { L.x += o.x; L.y += o.y; }
     }
-    // exclusive prefix: the composition of the lanes below
-    double2 Ae = make_double2(__shfl_up_sync(0xffffffffu, A.x, 1), __shfl_up_sync(0xffffffffu, A.y, 1));
-    double2 Be = make_double2(__shfl_up_sync(0xffffffffu, B.x, 1), __shfl_up_sync(0xffffffffu, B.y, 1));
-    if (lane == 0) { Ae = make_double2(1, 0); Be = make_double2(0, 0); }
-    double2 a = gv_fma(Ae, h0, Be);                 // a_b
-    for (int i = b; i < e; ++i) {
-        const double c = cs[i];
-        const double2 si = sn[i];
-        const double2 hi1 = hin[i + 1];
-        col[i] = gv_fma(si, hi1, make_double2(c * a.x, c * a.y));
-        a = gv_fma(make_double2(-si.x, si.y), a, make_double2(c * hi1.x, c * hi1.y));
-    }
-    // a_j: the carry out of the last non-empty range (h_0 when j = 0)
-    const int last = j > 0 ? (j - 1) / per : 0;
-    a = make_double2(__shfl_sync(0xffffffffu, a.x, last), __shfl_sync(0xffffffffu, a.y, last));
-    if (j == 0) a = h0;
+    double2 S = make_double2(__shfl_up_sync(0xffffffffu, L.x, 1), __shfl_up_sync(0xffffffffu, L.y, 1));
+    if (lane == 0) S = make_double2(0, 0);
+    S.x += h0.x; S.y += h0.y;                       // a_b / p_b
+    double2 a = make_double2(h0.x + __shfl_sync(0xffffffffu, L.x, 31), h0.y + __shfl_sync(0xffffffffu, L.y, 31));
+    a = gv_mul(pj, a);                              // a_j
     // the new rotation, from (a_j, ||w||): c = |a| / d, s = (a / |a|) ||w|| / d, d = sqrt(|a|^2 + ||w||^2)
     const double n2a = a.x * a.x + a.y * a.y, d2 = n2a + hn * hn;
-    double cj;
-    double2 sj;
-    if (d2 == 0.0) { cj = 1.0; sj = make_double2(0, 0); }
-    else if (n2a == 0.0) { cj = 0.0; sj = make_double2(1.0, 0.0); }
-    else {
-        const double ia = rsqrt(n2a), id = rsqrt(d2);
-        cj = n2a * ia * id;
-        const double f = hn * ia * id;
-        sj = make_double2(a.x * f, a.y * f);
+    double cj = 1.0;
+    double2 sj = make_double2(0, 0);
+    const double rs = rsqrt((lane & 1) ? d2 : n2a);
+    const double ia = __shfl_sync(0xffffffffu, rs, 0), id = __shfl_sync(0xffffffffu, rs, 1);
+    if (n2a == 0.0) {
+        if (d2 != 0.0) { cj = 0.0; sj = make_double2(1.0, 0.0); }
+    } else {
+        const double f = ia * id;
+        cj = n2a * f;
+        sj = make_double2(a.x * (hn * f), a.y * (hn * f));
     }
-    int keep = 0;
+    // g_{j+1} = -conj(s) g_j
+    const double2 gn = make_double2(-(sj.x * gj.x + sj.y * gj.y), -(sj.x * gj.y - sj.y * gj.x));
+    const bool keep = !(stop || gn.x * gn.x + gn.y * gn.y <= t * t || hn == 0.0);
+    // the rotated column: rows of this lane's range, and row j
+    double2* out = ga.Rm + ((int64_t)s * m + j) * m;
+    for (int i = b; i < e; ++i) {
+        const double c = cs[i];
+        const double2 hi1 = hin[i + 1], p = i > 0 ? pp[i] : make_double2(1, 0), ai = gv_mul(p, S);
+        out[i] = gv_fma(sn[i], hi1, make_double2(c * ai.x, c * ai.y));
+        if (i + 1 < e) S = gv_fma(pq[i], hi1, S);
+    }
+    __syncwarp();
     if (lane == 0) {
+        out[j] = make_double2(cj * a.x + sj.x * hn, cj * a.y + sj.y * hn);
         ga.cs[(int64_t)s * m + j] = cj;
         ga.sn[(int64_t)s * m + j] = sj;
-        col[j] = make_double2(cj * a.x + sj.x * hn, cj * a.y + sj.y * hn);
-        double2* g = ga.gv + (int64_t)s * (m + 1);
-        const double2 gj = g[j];
-        const double2 gn = make_double2(-(sj.x * gj.x + sj.y * gj.y), -(sj.x * gj.y - sj.y * gj.x));   // -conj(s) g_j
         g[j + 1] = gn;
         g[j] = make_double2(cj * gj.x, cj * gj.y);
+        // p_{j+1} = -conj(s_j) p_j; 1 / conj(s_j) = s_j / |s_j|^2, |s_j| = ||w|| / d
+        pp[j + 1] = gv_mul(make_double2(-sj.x, sj.y), pj);
+        const double f = n2a == 0.0 ? 1.0 : d2 * ihn * ihn;
+        const double2 ip = gv_mul(make_double2(-sj.x * f, -sj.y * f), ipj);
+        ga.ip[s] = ip;
+        pq[j] = make_double2(cj * ip.x, cj * ip.y);
         if (ga.gmon && s == 0) *ga.gmon = gn;
         ga.kused[s] = j + 1;
         ga.beta[s] = hn;
-        const double t = ga.target[s];
-        keep = !(stop || gn.x * gn.x + gn.y * gn.y <= t * t || hn == 0.0);
         if (!keep) ga.active[s] = 0;
         else if (ga.nact) atomicAdd(ga.nact, 1);
     }
-    __syncwarp();
-    double2* out = ga.Rm + ((int64_t)s * m + j) * m;          // column j, rows 0..j
-    for (int i = lane; i <= j; i += 32) out[i] = col[i];
-    return __shfl_sync(0xffffffffu, keep, 0) != 0;
+    return keep;
 }
 
 // Sums NV values per lane over the warp by recursive halving (NV/2 + NV/4 +

@@ -72,11 +72,11 @@ __global__ void __launch_bounds__(KT) k_update_givens(const Chunk* __restrict__ 
     if (threadIdx.x < 32) {
         const int j = ga.j;
         double2* hin = sh;                   // [j+1] h1 + h2
-        double2* col = sh + (j + 1);         // [j+1] the rotated column
         for (int i = threadIdx.x; i <= j; i += 32)
             hin[i] = cadd(ga.h1[(int64_t)c.seg * ga.ldh + i], ga.h2[(int64_t)c.seg * ga.ldh + i]);
         __syncwarp();
-        givens_core(ga, c.seg, j, hin, sqrt(s_hn2), col);
+        const double hn = sqrt(s_hn2);
+        givens_core(ga, c.seg, j, hin, hn, 1.0 / hn);
     }
 }
 
@@ -191,7 +191,7 @@ struct Krylov {
     DArr<Chunk> d_chunks;
     DArr<int32_t> seg_ch;
     DArr<V> basis, w, r, t;
-    DArr<double2> partial, h1, h2, Rm, sn, gv, y;
+    DArr<double2> partial, h1, h2, Rm, sn, gv, pp, pq, ip, y;
     DArr<double> nrm_part, nrm, cs, beta, target, prev;
     DArr<int> active, kused, cnt;
     // monitor record of the latest Arnoldi step, 32 bytes: the active-segment
@@ -233,7 +233,9 @@ struct Krylov {
         h1.alloc((size_t)nseg * (m + 1)); h2.alloc((size_t)nseg * (m + 1));
         Rm.alloc((size_t)nseg * m * m);
         sn.alloc((size_t)nseg * m); cs.alloc((size_t)nseg * m);
-        gv.alloc((size_t)nseg * (m + 1)); y.alloc((size_t)nseg * m);
+        gv.alloc((size_t)nseg * (m + 1));
+        pp.alloc((size_t)nseg * (m + 1)); pq.alloc((size_t)nseg * m); ip.alloc(nseg);
+        y.alloc((size_t)nseg * m);
         nrm_part.alloc(nch); nrm.alloc(nseg); beta.alloc(nseg); target.alloc(nseg); prev.alloc(nseg);
         active.alloc(nseg); kused.alloc(nseg);
         cnt.alloc(nseg);
@@ -268,8 +270,8 @@ struct Krylov {
     }
 
     // dynamic shared memory of k_update_givens at step j <= m-1: the nk = j+1
-    // coefficients, or the Givens column and its rotated copy
-    static size_t givens_smem(int mm) { return 2 * (size_t)mm * sizeof(double2); }
+    // coefficients, or the Hessenberg column
+    static size_t givens_smem(int mm) { return (size_t)mm * sizeof(double2); }
 
     unsigned long long* kw(int k) const { return work ? work + k : nullptr; }
 
@@ -342,9 +344,9 @@ struct Krylov {
                 THM_LAUNCH(THM_K_UPDATE, st, k_update_dots<V><<<nch, KT, sm, st>>>(d_chunks.p, basis.p, n, nk, h1.p, m + 1, w.p,
                                                                                   partial.p, m + 1, active.p, seg_ch.p,
                                                                                   cnt.p, h2.p, kw(1)));
-                GivensArgs ga{j, m, m + 1, h1.p, h2.p, Rm.p, cs.p, sn.p, gv.p, target.p, active.p, kused.p, beta.p,
+                GivensArgs ga{j, m, m + 1, h1.p, h2.p, Rm.p, cs.p, sn.p, gv.p, pp.p, pq.p, ip.p, target.p, active.p, kused.p, beta.p,
                               nact, flag, nseg == 1 ? gmon : nullptr, seg_ch.p, cnt.p};
-                const size_t gsm = 2 * (size_t)(j + 1) * sizeof(double2);      // coefficients, or column + rotated column
+                const size_t gsm = (size_t)(j + 1) * sizeof(double2);
                 THM_LAUNCH(THM_K_UPDATE, st, k_update_givens<V><<<nch, KT, gsm, st>>>(d_chunks.p, basis.p, n, nk, w.p, nrm_part.p,
                                                                                       active.p, ga, kw(1)));
                 THM_LAUNCH(THM_K_KRYLOV, st, k_chunk_scale<V><<<nch, 256, 0, st>>>(d_chunks.p, w.p, beta.p, basis.p + (int64_t)(j + 1) * n, active.p));
@@ -378,8 +380,8 @@ template <class V>
 struct SubWork {
     int m = 0;
     DArr<V> basis, zbasis, w;
-    DArr<double2> partial, pre, Rm, y;
-    DArr<double> beta, target;
+    DArr<double2> partial, Rm, y;
+    DArr<double> beta;
     DArr<int> active, kused, flag;
     void init(const thm_mesh* mesh, int m_) {
         THM_REQUIRE(m_ < (sizeof(V) == 8 ? 800 : 1600), "restart length too large");
@@ -389,10 +391,9 @@ struct SubWork {
         zbasis.alloc((size_t)m * n);
         w.alloc(n);
         partial.alloc(ns * mesh->nd.C * (2 * m + 2));
-        pre.alloc(ns * (m + 1));
         Rm.alloc(ns * m * m);
         y.alloc(ns * m);
-        beta.alloc(ns); target.alloc(ns); active.alloc(ns); kused.alloc(ns); flag.alloc(1);
+        beta.alloc(ns); active.alloc(ns); kused.alloc(ns); flag.alloc(1);
     }
 };
 
@@ -661,8 +662,8 @@ static void subsolve(thm_sys* s, const SolveCfg& c, SubWork<V>& k, const FW* fac
     a.n = m->n_loc;
     a.b = b; a.x = x; a.r = w->r64.p;
     a.basis = k.basis.p; a.zbasis = k.zbasis.p; a.w = k.w.p;
-    a.partial = k.partial.p; a.pre = k.pre.p; a.y = k.y.p;
-    a.g = GivensArgs{0, mr, mr + 1, nullptr, nullptr, k.Rm.p, nullptr, nullptr, nullptr, k.target.p, k.active.p, k.kused.p,
+    a.partial = k.partial.p; a.y = k.y.p;
+    a.g = GivensArgs{0, mr, mr + 1, nullptr, nullptr, k.Rm.p, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, k.active.p, k.kused.p,
                      k.beta.p, nullptr, k.flag.p, nullptr, nullptr, nullptr};
     a.subs = m->d_subs.p;
     a.slice_ptr = m->d_slice_ptr.p;

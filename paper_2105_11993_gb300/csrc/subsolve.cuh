@@ -68,7 +68,7 @@ struct SubArgs {
     double2 *x, *r;             // solution; residual (workspace)
     V *basis, *zbasis, *w;
     double2* partial;           // [n_sub * C][2m + 2]
-    double2 *pre, *y;           // [n_sub][m + 1]: [b; d] of the previous step, gamma at m; [n_sub][m]
+    double2* y;                 // [n_sub][m]
     GivensArgs g;
     const Sub* subs;
     const int64_t* slice_ptr;
@@ -83,8 +83,9 @@ struct SubArgs {
 // Work items that a dot-product pass is cut into while there are few basis
 // vectors: three per warp, so that the last round is not nearly empty.
 constexpr int SUB_ITEMS = 3 * ND_NW;
-// Shared memory that outlives a step: rotations and g of the cycle.
-__host__ __device__ inline size_t sub_keep_bytes(int m) { return (size_t)m * 24 + (size_t)(m + 1) * 16 + 16; }
+// Shared memory that outlives a step: rotations and g of the cycle (givens_core)
+// and the previous step's [b; d].
+__host__ __device__ inline size_t sub_keep_bytes(int m) { return (size_t)m * 40 + (size_t)(m + 1) * 48 + 48; }
 
 // Bytes of the Krylov phases' shared memory (they reuse the apply's): u and w
 // of the CTA's rows, the totals and the Hessenberg column, the coefficients,
@@ -92,11 +93,15 @@ __host__ __device__ inline size_t sub_keep_bytes(int m) { return (size_t)m * 24 
 template <class V>
 __host__ __device__ inline size_t sub_krylov_bytes(int rows, int m, int k_glob) {
     const size_t red = (size_t)(m / 4 + 2 + SUB_ITEMS) * 16 * sizeof(typename VT<V>::R);
-    return (k_glob ? 0 : 2 * (size_t)rows * sizeof(V)) + (size_t)(2 * m + 2) * 16 + 2 * (size_t)(m + 1) * 16 +
+    return (k_glob ? 0 : 2 * (size_t)rows * sizeof(V)) + (size_t)(2 * m + 2) * 16 + (size_t)(m + 1) * 16 +
            (size_t)(2 * m + 2) * sizeof(V) + (red + 15) / 16 * 16;
 }
 // rows of a CTA: the subdomain's local rows in C equal parts of whole warps
-__host__ __device__ inline int sub_rows(int64_t n, int C) { return (int)(((n + C - 1) / C + 31) / 32 * 32); }
+// of the SELL slices, or of 8 where that would leave CTAs without rows
+__host__ __device__ inline int sub_rows(int64_t n, int C) {
+    const int64_t r = (n + C - 1) / C, g = r >= 512 ? 32 : 8;
+    return (int)((r + g - 1) / g * g);
+}
 
 // A sum with the rounding of its partial sums compensated (Kahan): FP32 sums
 // over a CTA's rows stay as accurate as sums over 8 rows.  FP64 sums plainly.
@@ -247,8 +252,7 @@ k_subsolve(NdTables T, NdSizes z, NdMem mm, V* __restrict__ glob, const FW* __re
     unsigned char* kp = smem + nd_layout<V>(z, mm.slt_smem, mm.u_glob, mm.y_glob).vec;
     double2* tot = reinterpret_cast<double2*>(kp);
     double2* hin = tot + 2 * m + 2;
-    double2* hcol = hin + m + 1;
-    V* sc = reinterpret_cast<V*>(hcol + m + 1);
+    V* sc = reinterpret_cast<V*>(hin + m + 1);
     R* red = reinterpret_cast<R*>(sc + 2 * m + 2);
     V* s_uw = reinterpret_cast<V*>(reinterpret_cast<unsigned char*>(red) + ((size_t)(m / 4 + 2 + SUB_ITEMS) * 16 * sizeof(R) + 15) / 16 * 16);
     double2* part = a.partial + ((int64_t)sub * C) * (2 * m + 2);
@@ -256,10 +260,15 @@ k_subsolve(NdTables T, NdSizes z, NdMem mm, V* __restrict__ glob, const FW* __re
     GivensArgs gl = a.g;
     gl.gv = reinterpret_cast<double2*>(smem + keep_off);
     gl.sn = gl.gv + m + 1;
-    gl.cs = reinterpret_cast<double*>(gl.sn + m);
+    gl.pp = gl.sn + m;
+    gl.pq = gl.pp + m + 1;
+    gl.ip = gl.pq + m;
+    double2* pre = gl.ip + 1;                  // [m + 1]
+    double* target = reinterpret_cast<double*>(pre + m + 1);
+    gl.cs = target + 2;
+    gl.target = target;
     gl.Rm += (int64_t)sub * m * m;
-    gl.target += sub; gl.active += sub; gl.kused += sub; gl.beta += sub;
-    double2* pre = a.pre + (int64_t)sub * (m + 1);
+    gl.active += sub; gl.kused += sub; gl.beta += sub;
     int turn = 0, total = 0, most = 0, steps = 0;
     unsigned long long w_dots = 0, w_upd = 0, n_apply = 0, n_res = 0;      // counted by thread 0 of rank 0
 
@@ -296,11 +305,12 @@ k_subsolve(NdTables T, NdSizes z, NdMem mm, V* __restrict__ glob, const FW* __re
         }
         if (rank == 0 && tid == 0) {
             gl.gv[0] = make_double2(beta, 0);
-            *const_cast<double*>(gl.target) = F64 ? a.tol * bn : a.cycle_tol * beta;
+            *target = F64 ? a.tol * bn : a.cycle_tol * beta;
         }
         cluster.sync();
         int j = 0;
         bool broke = false;
+        double gp = 1, igp = 1;                // gamma of the previous step, and its inverse
         for (;; ++j) {
             const bool last = j == m || total >= a.maxit;
             V* uj = a.basis + (int64_t)j * a.n;
@@ -359,30 +369,30 @@ k_subsolve(NdTables T, NdSizes z, NdMem mm, V* __restrict__ glob, const FW* __re
             }
             cluster.sync();
             // totals and the scalar step, the same in every CTA
-            double v3[3] = {0, 0, 0};          // |s|^2, s^H b
             for (int k = tid; k < 2 * j + 2; k += ND_NT) {
-                double2 t = make_double2(0, 0);
-                for (int q = 0; q < C; ++q) t = cadd(t, __ldcg(part + (int64_t)q * (2 * m + 2) + k));
-                tot[k] = t;
+                double2 t[8];
+#pragma unroll
+                for (int q = 0; q < 8; ++q)
+                    t[q] = q < C ? __ldcg(part + (int64_t)q * (2 * m + 2) + k) : make_double2(0, 0);
+#pragma unroll
+                for (int q = 1; q < 8; ++q)
+                    if (q < C) t[0] = cadd(t[0], t[q]);
+                tot[k] = t[0];
             }
             if (tid == 0) { s_task = 0; if (j == 0) s_keep = 1; }
             __syncthreads();
-            // FP64 instructions cost a warp 16 cycles of its SM whatever its
-            // active lanes, so they run on as few warps as the columns need
+            // |s|^2 and s^H b.  FP64 instructions cost a warp 64 cycles whatever
+            // its active lanes, so they run on as few warps as the columns need
             if (warp * 32 < j) {
+                double v4[4] = {0, 0, 0, 0};
                 for (int k = tid; k < j; k += ND_NT) {
                     const double2 sk = tot[2 * k], bk = tot[2 * k + 1];
-                    v3[0] += sk.x * sk.x + sk.y * sk.y;
-                    v3[1] += sk.x * bk.x + sk.y * bk.y;
-                    v3[2] += sk.x * bk.y - sk.y * bk.x;
+                    v4[0] += sk.x * sk.x + sk.y * sk.y;
+                    v4[1] += sk.x * bk.x + sk.y * bk.y;
+                    v4[2] += sk.x * bk.y - sk.y * bk.x;
                 }
-#pragma unroll
-                for (int o = 16; o > 0; o >>= 1)
-#pragma unroll
-                    for (int q = 0; q < 3; ++q) v3[q] += __shfl_xor_sync(0xffffffffu, v3[q], o);
-                if (lane == 0)
-#pragma unroll
-                    for (int q = 0; q < 3; ++q) s_red[warp][q] = v3[q];
+                const double t = warp_sum_many<4>(v4, lane);
+                if ((lane & 7) == 0 && lane < 24) s_red[warp][lane >> 3] = t;
             }
             __syncthreads();
             if (warp == 0) {                   // gamma, 1 / gamma and d for everybody
@@ -390,12 +400,12 @@ k_subsolve(NdTables T, NdSizes z, NdMem mm, V* __restrict__ glob, const FW* __re
                 for (int q = 0; q * 32 < min(j, ND_NT); ++q) { ss += s_red[q][0]; sbr += s_red[q][1]; sbi += s_red[q][2]; }
                 const double c1 = tot[2 * j].x;
                 const double2 c2 = tot[2 * j + 1];
-                double gamma = 1.0;
+                double gamma = 1.0, ig = 1.0;
                 if (j > 0) {
                     const double g2 = c1 - ss;
-                    gamma = g2 > 0 ? sqrt(g2) : 0.0;     // 0: u_j lies in span(V) (a lucky breakdown)
+                    ig = g2 > 0 ? rsqrt(g2) : INFINITY;
+                    gamma = g2 > 0 ? g2 * ig : 0.0;      // 0: u_j lies in span(V) (a lucky breakdown)
                 }
-                const double ig = 1.0 / gamma;
                 if (lane == 0) {
                     s_sc[0] = isfinite(c1) && isfinite(c2.x) && isfinite(c2.y) && isfinite(gamma) ? gamma : -1.0;
                     s_sc[1] = ig;
@@ -410,39 +420,34 @@ k_subsolve(NdTables T, NdSizes z, NdMem mm, V* __restrict__ glob, const FW* __re
                 broke = true;
                 break;                         // the totals are the same in every CTA: all of them leave here
             }
-            const double gp = (rank == 0 && j > 0) ? pre[m].x : 1.0;
-            if (rank == 0) {
-                // Hessenberg column j-1: [b_{j-1}; d_{j-1}] + gamma_{j-1} s_j over gamma_{j-1} gamma_j
-                for (int i = tid; i < j; i += ND_NT) {
-                    const double2 p = pre[i], si = tot[2 * i];
-                    hin[i] = make_double2(p.x + gp * si.x, p.y + gp * si.y);
-                }
-                __syncthreads();
-            }
-            if (!last) {
-                const double ig = s_sc[1];
+            const double ig = s_sc[1];
+            {
                 const double2 d = make_double2(s_sc[2], s_sc[3]);
                 for (int k = tid; k < j; k += ND_NT) {
                     const double2 sk = tot[2 * k], bk = tot[2 * k + 1];
-                    if (rank == 0) pre[k] = bk;
+                    if (rank == 0) {
+                        // Hessenberg column j-1: [b_{j-1}; d_{j-1}] + gamma_{j-1} s_j over gamma_{j-1} gamma_j
+                        const double2 p = pre[k];
+                        hin[k] = make_double2(p.x + gp * sk.x, p.y + gp * sk.y);
+                        pre[k] = bk;
+                    }
                     sc[k] = mk<V>((R)(-sk.x * ig), (R)(-sk.y * ig));
                     sc[j + k] = mk<V>((R)(-(bk.x - (sk.x * d.x - sk.y * d.y) * ig) * ig),
                                       (R)(-(bk.y - (sk.x * d.y + sk.y * d.x) * ig) * ig));
                 }
-                if (tid == 0) {
-                    if (rank == 0) {
-                        pre[j] = d;
-                        pre[m] = make_double2(gamma, 0.0);
-                    }
+                if (tid == ND_NT - 1) {
+                    if (rank == 0) pre[j] = d;
                     sc[2 * j] = mk<V>((R)ig, (R)0);
                     sc[2 * j + 1] = mk<V>((R)(-d.x * ig * ig), (R)(-d.y * ig * ig));
                 }
             }
             __syncthreads();
             if (rank == 0 && warp == 0 && j > 0) {     // the Givens step beside the update
-                const bool keep = givens_core(gl, 0, j - 1, hin, gp * gamma, hcol, last);
+                const bool keep = givens_core(gl, 0, j - 1, hin, gp * gamma, igp * ig, last);
                 if (lane < C) *cluster.map_shared_rank(&s_keep, lane) = keep;
             }
+            gp = gamma;
+            igp = ig;
             if (!last) {
                 // v_j over u_j and u_{j+1}: NU * 32 rows per warp and turn
                 V* un = uj + a.n;
