@@ -125,230 +125,11 @@ __device__ __forceinline__ void tma_load_1d(void* dst, const void* src, unsigned
 __device__ __forceinline__ void fence_proxy_async() { asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory"); }
 
 // ---------------------------------------------------------------------------
-// Segmented reductions for the batched Arnoldi process.  A chunk lies inside
-// one segment (subdomain); per-chunk partials are summed per segment in a
+// Segmented passes over vectors.  A chunk lies inside one segment (a problem
+// of a batch); per-chunk partials are summed per segment in a
 // fixed order, so every dot product is deterministic.
 // ---------------------------------------------------------------------------
 constexpr int KT = 256;                       // threads per chunk block
-constexpr int EPT = CHUNK / KT;               // elements per thread
-
-// The last block of a segment to finish (per-segment arrival counter) sums
-// the segment's per-chunk partials in chunk order, so the result does not
-// depend on which block finishes last, and resets the counter for the next
-// launch.  Partials of other blocks are read through L2 (__ldcg).
-__device__ __forceinline__ bool last_block_of_segment(int seg, const int32_t* __restrict__ seg_ch, int* cnt) {
-    __shared__ int s_last;
-    __threadfence();
-    __syncthreads();
-    if (threadIdx.x == 0) s_last = atomicAdd(&cnt[seg], 1) == seg_ch[seg + 1] - seg_ch[seg] - 1;
-    __syncthreads();
-    if (s_last) {
-        __threadfence();
-        if (threadIdx.x == 0) cnt[seg] = 0;
-    }
-    return s_last != 0;
-}
-
-// h[seg][k] = sum over the segment's chunks of v_k^H w (FP64), k < nk.
-// reset (optional): an int the first block sets to 0 (the active-segment
-// count that the Givens step of the same Arnoldi step accumulates).
-// h[seg][k] = v_k^H w for the chunk c of a block whose threads hold w in
-// wr (EPT elements each); the last block of the segment writes h.
-template <class V>
-__device__ __forceinline__ void chunk_dots_body(const Chunk& c, const V* __restrict__ basis, int64_t ld, int nk,
-                                                const V (&wr)[EPT], double2* __restrict__ partial, int ldp,
-                                                const int32_t* __restrict__ seg_ch, int* __restrict__ cnt,
-                                                double2* __restrict__ h, int ldh, double2* sred);
-
-template <class V>
-__global__ void __launch_bounds__(KT) k_chunk_dots(const Chunk* __restrict__ chunks, const V* __restrict__ basis,
-                                                   int64_t ld, int nk, const V* __restrict__ w,
-                                                   double2* __restrict__ partial, int ldp,
-                                                   const int* __restrict__ act, const int32_t* __restrict__ seg_ch,
-                                                   int* __restrict__ cnt, double2* __restrict__ h, int ldh,
-                                                   int* __restrict__ reset, unsigned long long* __restrict__ work) {
-    extern __shared__ double2 sred[];          // [nk][KT/32]
-    if (reset && blockIdx.x == 0 && threadIdx.x == 0) *reset = 0;
-    const Chunk c = chunks[blockIdx.x];
-    if (act && !act[c.seg]) return;            // converged segment: its partials are not read
-    if (work && threadIdx.x == 0) atomicAdd(work, (unsigned long long)((nk + 1) * (c.end - c.begin) * sizeof(V)));
-    V wr[EPT];
-#pragma unroll
-    for (int q = 0; q < EPT; ++q) {
-        int64_t e = c.begin + threadIdx.x + (int64_t)q * KT;
-        wr[q] = e < c.end ? w[e] : mk<V>(0, 0);
-    }
-    chunk_dots_body<V>(c, basis, ld, nk, wr, partial, ldp, seg_ch, cnt, h, ldh, sred);
-}
-
-template <class V>
-__device__ __forceinline__ void chunk_dots_body(const Chunk& c, const V* __restrict__ basis, int64_t ld, int nk,
-                                                const V (&wr)[EPT], double2* __restrict__ partial, int ldp,
-                                                const int32_t* __restrict__ seg_ch, int* __restrict__ cnt,
-                                                double2* __restrict__ h, int ldh, double2* sred) {
-    using R = typename VT<V>::R;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const bool full = c.end - c.begin == CHUNK;
-    // basis vectors in blocks of KB: their KB * EPT loads are issued together,
-    // so a block of vectors costs one memory latency instead of KB
-    constexpr int KB = 4;
-    for (int k0 = 0; k0 < nk; k0 += KB) {
-        V v[KB][EPT];
-#pragma unroll
-        for (int b = 0; b < KB; ++b) {
-            const V* vk = basis + (int64_t)(k0 + b) * ld;
-#pragma unroll
-            for (int q = 0; q < EPT; ++q) {
-                const int64_t e = c.begin + threadIdx.x + (int64_t)q * KT;
-                v[b][q] = mk<V>(0, 0);
-                if (k0 + b < nk && (full || e < c.end)) v[b][q] = vk[e];
-            }
-        }
-        R ar[KB], ai[KB];
-#pragma unroll
-        for (int b = 0; b < KB; ++b) {
-            ar[b] = 0;
-            ai[b] = 0;
-#pragma unroll
-            for (int q = 0; q < EPT; ++q) {
-                ar[b] += v[b][q].x * wr[q].x + v[b][q].y * wr[q].y;       // conj(v) * w
-                ai[b] += v[b][q].x * wr[q].y - v[b][q].y * wr[q].x;
-            }
-        }
-        // a warp sums its 4 * 32 products in the vector precision; from the
-        // cross-warp sum on every sum is FP64 (FP64 shuffles at the warp level
-        // cost 2.7x the kernel time on this part, measured)
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1)
-#pragma unroll
-            for (int b = 0; b < KB; ++b) {
-                ar[b] += __shfl_down_sync(0xffffffffu, ar[b], o);
-                ai[b] += __shfl_down_sync(0xffffffffu, ai[b], o);
-            }
-        if (lane == 0)
-#pragma unroll
-            for (int b = 0; b < KB; ++b)
-                if (k0 + b < nk) sred[(k0 + b) * (KT / 32) + warp] = make_double2((double)ar[b], (double)ai[b]);
-    }
-    __syncthreads();
-    for (int kk = threadIdx.x; kk < nk; kk += KT) {
-        double2 s = make_double2(0, 0);
-        for (int q = 0; q < KT / 32; ++q) s = cadd(s, sred[kk * (KT / 32) + q]);
-        partial[(int64_t)blockIdx.x * ldp + kk] = s;
-    }
-    if (!last_block_of_segment(c.seg, seg_ch, cnt)) return;
-    for (int kk = threadIdx.x; kk < nk; kk += KT) {
-        double2 s = make_double2(0, 0);
-        for (int cc = seg_ch[c.seg]; cc < seg_ch[c.seg + 1]; ++cc) {
-            const double2 p = __ldcg(&partial[(int64_t)cc * ldp + kk]);
-            s.x += p.x;
-            s.y += p.y;
-        }
-        h[(int64_t)c.seg * ldh + kk] = s;
-    }
-}
-
-// w -= sum_k h[seg][k] basis_k ;  optionally per-chunk ||w||^2
-template <class V>
-__device__ __forceinline__ void chunk_update_body(const Chunk& c, const V* __restrict__ basis, int64_t ld, int nk,
-                                                  const double2* __restrict__ h, int ldh, V* __restrict__ w,
-                                                  double* __restrict__ nrm_part, double2* sh, V* wout = nullptr);
-
-
-template <class V>
-__device__ __forceinline__ void chunk_update_body(const Chunk& c, const V* __restrict__ basis, int64_t ld, int nk,
-                                                  const double2* __restrict__ h, int ldh, V* __restrict__ w,
-                                                  double* __restrict__ nrm_part, double2* sh, V* wout) {
-    using R = typename VT<V>::R;
-    __shared__ double sw[KT / 32];
-    // the coefficients in the vector precision, rounded once per block (a
-    // double-to-float conversion per use would run on the slow FP64 path)
-    V* shv = reinterpret_cast<V*>(sh);
-    for (int k = threadIdx.x; k < nk; k += KT) {
-        const double2 hk = h[(int64_t)c.seg * ldh + k];
-        shv[k] = mk<V>((R)hk.x, (R)hk.y);
-    }
-    __syncthreads();
-    const bool full = c.end - c.begin == CHUNK;
-    R xr[EPT], xi[EPT];
-#pragma unroll
-    for (int q = 0; q < EPT; ++q) {
-        int64_t e = c.begin + threadIdx.x + (int64_t)q * KT;
-        V a = (full || e < c.end) ? w[e] : mk<V>(0, 0);
-        xr[q] = a.x;
-        xi[q] = a.y;
-    }
-    // basis vectors in blocks of KB: KB * EPT independent loads in flight
-    constexpr int KB = 4;
-    for (int k0 = 0; k0 < nk; k0 += KB) {
-        V v[KB][EPT];
-#pragma unroll
-        for (int b = 0; b < KB; ++b) {
-            const V* vk = basis + (int64_t)(k0 + b) * ld;
-#pragma unroll
-            for (int q = 0; q < EPT; ++q) {
-                const int64_t e = c.begin + threadIdx.x + (int64_t)q * KT;
-                v[b][q] = mk<V>(0, 0);
-                if (k0 + b < nk && (full || e < c.end)) v[b][q] = vk[e];
-            }
-        }
-#pragma unroll
-        for (int b = 0; b < KB; ++b) {
-            const int kk = min(k0 + b, nk - 1);
-            const V hv = shv[kk];
-            const R hr = k0 + b < nk ? hv.x : (R)0, hi = k0 + b < nk ? hv.y : (R)0;
-#pragma unroll
-            for (int q = 0; q < EPT; ++q) {
-                xr[q] -= hr * v[b][q].x - hi * v[b][q].y;
-                xi[q] -= hr * v[b][q].y + hi * v[b][q].x;
-            }
-        }
-    }
-    R nr = 0;
-#pragma unroll
-    for (int q = 0; q < EPT; ++q) {
-        int64_t e = c.begin + threadIdx.x + (int64_t)q * KT;
-        if (full || e < c.end) {
-            w[e] = mk<V>(xr[q], xi[q]);
-            nr += xr[q] * xr[q] + xi[q] * xi[q];
-        }
-        if (wout) wout[q] = (full || e < c.end) ? mk<V>(xr[q], xi[q]) : mk<V>(0, 0);
-    }
-    if (nrm_part) {
-        const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) nr += __shfl_down_sync(0xffffffffu, nr, o);
-        if (lane == 0) sw[warp] = (double)nr;
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            double s = 0;
-            for (int q = 0; q < KT / 32; ++q) s += sw[q];
-            nrm_part[blockIdx.x] = s;
-        }
-    }
-}
-
-// First Gram-Schmidt update and second projection in one pass over the
-// chunk: w <- w - V h1 (written back), then h2 = V^H w from the updated
-// values still in registers.  The block rereads its basis slab right after
-// the update, while it is in L2, so V is streamed from DRAM once for both.
-template <class V>
-__global__ void __launch_bounds__(KT) k_update_dots(const Chunk* __restrict__ chunks, const V* __restrict__ basis,
-                                                    int64_t ld, int nk, const double2* __restrict__ h1, int ldh,
-                                                    V* __restrict__ w, double2* __restrict__ partial, int ldp,
-                                                    const int* __restrict__ act, const int32_t* __restrict__ seg_ch,
-                                                    int* __restrict__ cnt, double2* __restrict__ h2,
-                                                    unsigned long long* __restrict__ work) {
-    extern __shared__ double2 sh[];            // [nk] coefficients, then [nk][KT/32] warp sums
-    const Chunk c = chunks[blockIdx.x];
-    if (act && !act[c.seg]) return;
-    // the basis twice, w read and written
-    if (work && threadIdx.x == 0) atomicAdd(work, (unsigned long long)((2 * nk + 2) * (c.end - c.begin) * sizeof(V)));
-    V wr[EPT];
-    chunk_update_body<V>(c, basis, ld, nk, h1, ldh, w, nullptr, sh, wr);
-    __syncthreads();                           // sh is reused for the warp sums
-    chunk_dots_body<V>(c, basis, ld, nk, wr, partial, ldp, seg_ch, cnt, h2, ldh, sh);
-}
 
 template <class V>
 __global__ void __launch_bounds__(KT) k_chunk_norm2(const Chunk* __restrict__ chunks, const V* __restrict__ x,

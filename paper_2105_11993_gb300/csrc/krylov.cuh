@@ -1,5 +1,6 @@
-// The scalar parts of a GMRES cycle, FP64, one warp per Krylov segment: the
-// Givens step of a Hessenberg column and the back substitution at its end.
+// The scalar parts of a GMRES cycle, FP64, one warp per Krylov segment (the
+// Givens step of a Hessenberg column, the back substitution at its end), and
+// the Gram-Schmidt passes of the interface GMRES.
 #pragma once
 
 #include "kernels.cuh"
@@ -204,6 +205,202 @@ __device__ __forceinline__ void backsolve(int m, int k, const double2* R, const 
         }
         __syncwarp();
     }
+}
+
+constexpr int KW = KT / 32;
+constexpr int KSUB = 128;                     // elements that a warp holds, 4 a lane; chunks are multiples of it
+constexpr int KEPT = KSUB / 32;
+
+// The last block of a segment to finish (per-segment arrival counter) sums
+// the segment's per-chunk partials in chunk order, so the result does not
+// depend on which block finishes last, and resets the counter for the next
+// launch.  Partials of other blocks are read through L2 (__ldcg).
+__device__ __forceinline__ bool last_block_of_segment(int seg, const int32_t* __restrict__ seg_ch, int* cnt) {
+    __shared__ int s_last;
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0) s_last = atomicAdd(&cnt[seg], 1) == seg_ch[seg + 1] - seg_ch[seg] - 1;
+    __syncthreads();
+    if (s_last) {
+        __threadfence();
+        if (threadIdx.x == 0) cnt[seg] = 0;
+    }
+    return s_last != 0;
+}
+
+// Gram-Schmidt passes of the interface GMRES.  A warp works on basis vectors
+// of its own (KB at a time, all of a chunk's elements), so a dot product needs
+// no sum over the warps, an update one, and a chunk can be as small as 128
+// elements: interface systems of a few hundred to ten thousand unknowns spread
+// over many SMs.  (Chunks of 1024 elements with the elements shared by the
+// warps ran the smaller systems on one SM, whose FP64 units, 2 FMA per clock,
+// then worked through zeros, and five rounds of FP64 shuffles a vector; per
+// launch, dot products and updates: 256 unknowns 80 -> 16 us and 97 -> 23 us,
+// 3-D interfaces of 6^3 cells 124 -> 21 us and 151 -> 29 us.)
+constexpr int KB = 4;
+
+// hs[k] += v_k^H w over the elements from e0 on (wr: w of them, by lane), k < nk;
+// entry k is one warp's.
+__device__ __forceinline__ void sub_chunk_dots(const double2* __restrict__ basis, int64_t ld, int nk, int64_t e0, int64_t end,
+                                               const double2 (&wr)[KEPT], double2* hs) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    for (int k0 = warp * KB; k0 < nk; k0 += KW * KB) {
+        double2 v[KB][KEPT];
+#pragma unroll
+        for (int b = 0; b < KB; ++b)
+#pragma unroll
+            for (int q = 0; q < KEPT; ++q) {
+                const int64_t e = e0 + lane + 32 * q;
+                v[b][q] = k0 + b < nk && e < end ? basis[(int64_t)(k0 + b) * ld + e] : make_double2(0, 0);
+            }
+        double a[2 * KB];
+#pragma unroll
+        for (int b = 0; b < 2 * KB; ++b) a[b] = 0;
+#pragma unroll
+        for (int q = 0; q < KEPT; ++q) {
+            if (e0 + 32 * q >= end) break;
+#pragma unroll
+            for (int b = 0; b < KB; ++b) {
+                a[2 * b] += v[b][q].x * wr[q].x + v[b][q].y * wr[q].y;         // conj(v) * w
+                a[2 * b + 1] += v[b][q].x * wr[q].y - v[b][q].y * wr[q].x;
+            }
+        }
+        const double t = warp_sum_many<2 * KB>(a, lane);     // lane l: value l / 4
+        if ((lane & 3) == 0 && k0 + (lane >> 3) < nk) reinterpret_cast<double*>(hs + k0)[lane >> 2] += t;
+    }
+}
+
+// The segment's h from its chunks' hs (the last block to finish adds them up in chunk order).
+__device__ __forceinline__ void chunk_dots_end(const Chunk& c, int nk, const double2* hs, double2* __restrict__ partial, int ldp,
+                                               const int32_t* __restrict__ seg_ch, int* __restrict__ cnt,
+                                               double2* __restrict__ h, int ldh) {
+    __syncthreads();
+    for (int kk = threadIdx.x; kk < nk; kk += KT) partial[(int64_t)blockIdx.x * ldp + kk] = hs[kk];
+    if (!last_block_of_segment(c.seg, seg_ch, cnt)) return;
+    const int c0 = seg_ch[c.seg], c1 = seg_ch[c.seg + 1];
+    for (int kk = threadIdx.x; kk < nk; kk += KT) {
+        double2 s = make_double2(0, 0);
+        constexpr int G = 8;                   // loads in flight
+        for (int cc = c0; cc < c1; cc += G) {
+            double2 p[G];
+#pragma unroll
+            for (int g = 0; g < G; ++g) p[g] = cc + g < c1 ? __ldcg(&partial[(int64_t)(cc + g) * ldp + kk]) : make_double2(0, 0);
+#pragma unroll
+            for (int g = 0; g < G; ++g)
+                if (cc + g < c1) s = cadd(s, p[g]);
+        }
+        h[(int64_t)c.seg * ldh + kk] = s;
+    }
+}
+
+// w -= sum_k h_k v_k over the KSUB elements from e0 on; the new w of element
+// e0 + tid is returned to thread tid < KSUB and kept in sw.  hk: the
+// coefficients; sa: [KW][KSUB] sums of the warps.
+__device__ __forceinline__ double2 sub_chunk_update(const double2* __restrict__ basis, int64_t ld, int nk, int64_t e0, int64_t end,
+                                                    const double2* hk, double2* __restrict__ w, double2* sa, double2* sw) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    double2 x[KEPT];
+#pragma unroll
+    for (int q = 0; q < KEPT; ++q) x[q] = make_double2(0, 0);
+    for (int k0 = warp * KB; k0 < nk; k0 += KW * KB) {
+        double2 v[KB][KEPT];
+#pragma unroll
+        for (int b = 0; b < KB; ++b)
+#pragma unroll
+            for (int q = 0; q < KEPT; ++q) {
+                const int64_t e = e0 + lane + 32 * q;
+                v[b][q] = k0 + b < nk && e < end ? basis[(int64_t)(k0 + b) * ld + e] : make_double2(0, 0);
+            }
+#pragma unroll
+        for (int q = 0; q < KEPT; ++q) {
+            if (e0 + 32 * q >= end) break;
+#pragma unroll
+            for (int b = 0; b < KB; ++b) {
+                const double2 hv = hk[min(k0 + b, nk - 1)];    // beyond nk - 1 the vectors are zeros
+                x[q].x += hv.x * v[b][q].x - hv.y * v[b][q].y;
+                x[q].y += hv.x * v[b][q].y + hv.y * v[b][q].x;
+            }
+        }
+    }
+#pragma unroll
+    for (int q = 0; q < KEPT; ++q) sa[warp * KSUB + lane + 32 * q] = x[q];
+    __syncthreads();
+    double2 a = make_double2(0, 0);
+    if (threadIdx.x < KSUB) {
+        const int64_t e = e0 + threadIdx.x;
+        if (e < end) {
+            const int nw = min(KW, (nk + KB - 1) / KB);        // warps that had vectors
+            double2 s = sa[threadIdx.x];
+            for (int q = 1; q < nw; ++q) s = cadd(s, sa[q * KSUB + threadIdx.x]);
+            a = w[e];
+            a = make_double2(a.x - s.x, a.y - s.y);
+            w[e] = a;
+        }
+        sw[threadIdx.x] = a;
+    }
+    __syncthreads();
+    return a;
+}
+
+// h[seg][k] = sum over the segment's chunks of v_k^H w, k < nk.
+// reset (optional): an int the first block sets to 0 (the active-segment
+// count that the Givens step of the same Arnoldi step accumulates).
+__global__ void __launch_bounds__(KT) k_chunk_dots(const Chunk* __restrict__ chunks, const double2* __restrict__ basis,
+                                                   int64_t ld, int nk, const double2* __restrict__ w,
+                                                   double2* __restrict__ partial, int ldp,
+                                                   const int* __restrict__ act, const int32_t* __restrict__ seg_ch,
+                                                   int* __restrict__ cnt, double2* __restrict__ h, int ldh,
+                                                   int* __restrict__ reset, unsigned long long* __restrict__ work) {
+    extern __shared__ double2 hs[];            // [nk]
+    if (reset && blockIdx.x == 0 && threadIdx.x == 0) *reset = 0;
+    const Chunk c = chunks[blockIdx.x];
+    if (act && !act[c.seg]) return;            // converged segment: its partials are not read
+    if (work && threadIdx.x == 0) atomicAdd(work, (unsigned long long)((nk + 1) * (c.end - c.begin) * sizeof(double2)));
+    for (int k = threadIdx.x; k < nk; k += KT) hs[k] = make_double2(0, 0);
+    __syncthreads();
+    for (int64_t e0 = c.begin; e0 < c.end; e0 += KSUB) {
+        double2 wr[KEPT];
+#pragma unroll
+        for (int q = 0; q < KEPT; ++q) {
+            const int64_t e = e0 + (threadIdx.x & 31) + 32 * q;
+            wr[q] = e < c.end ? w[e] : make_double2(0, 0);
+        }
+        sub_chunk_dots(basis, ld, nk, e0, c.end, wr, hs);
+    }
+    chunk_dots_end(c, nk, hs, partial, ldp, seg_ch, cnt, h, ldh);
+}
+
+// First Gram-Schmidt update and second projection in one pass over the
+// chunk: w <- w - V h1 (written back), then h2 = V^H w from the updated
+// values.  The block rereads its basis slab right after the update, while it
+// is in L2, so V is streamed from DRAM once for both.
+__global__ void __launch_bounds__(KT) k_update_dots(const Chunk* __restrict__ chunks, const double2* __restrict__ basis,
+                                                    int64_t ld, int nk, const double2* __restrict__ h1, int ldh,
+                                                    double2* __restrict__ w, double2* __restrict__ partial, int ldp,
+                                                    const int* __restrict__ act, const int32_t* __restrict__ seg_ch,
+                                                    int* __restrict__ cnt, double2* __restrict__ h2,
+                                                    unsigned long long* __restrict__ work) {
+    extern __shared__ double2 hk[];            // [nk] coefficients, [nk] dot products
+    __shared__ double2 sa[KW * KSUB], sw[KSUB];
+    const Chunk c = chunks[blockIdx.x];
+    if (act && !act[c.seg]) return;
+    // the basis twice, w read and written
+    if (work && threadIdx.x == 0) atomicAdd(work, (unsigned long long)((2 * nk + 2) * (c.end - c.begin) * sizeof(double2)));
+    double2* hs = hk + nk;
+    for (int k = threadIdx.x; k < nk; k += KT) {
+        hk[k] = h1[(int64_t)c.seg * ldh + k];
+        hs[k] = make_double2(0, 0);
+    }
+    __syncthreads();
+    for (int64_t e0 = c.begin; e0 < c.end; e0 += KSUB) {
+        sub_chunk_update(basis, ld, nk, e0, c.end, hk, w, sa, sw);
+        double2 wr[KEPT];
+#pragma unroll
+        for (int q = 0; q < KEPT; ++q) wr[q] = sw[(threadIdx.x & 31) + 32 * q];
+        sub_chunk_dots(basis, ld, nk, e0, c.end, wr, hs);
+        __syncthreads();                       // sa and sw are written again
+    }
+    chunk_dots_end(c, nk, hs, partial, ldp, seg_ch, cnt, h2, ldh);
 }
 
 }  // namespace thm

@@ -51,27 +51,42 @@ __global__ void k_cycle_start(int nseg, int m, const double* __restrict__ nrm2, 
 // Second Gram-Schmidt update w -= V h2 with the per-chunk ||w||^2; the last
 // block of each segment sums the segment's norm partials in chunk order and
 // runs that segment's Givens step (so no separate reduction or Givens launch).
-template <class V>
-__global__ void __launch_bounds__(KT) k_update_givens(const Chunk* __restrict__ chunks, const V* __restrict__ basis,
-                                                      int64_t ld, int nk, V* __restrict__ w,
+__global__ void __launch_bounds__(KT) k_update_givens(const Chunk* __restrict__ chunks, const double2* __restrict__ basis,
+                                                      int64_t ld, int nk, double2* __restrict__ w,
                                                       double* __restrict__ nrm_part, const int* __restrict__ act,
                                                       GivensArgs ga, unsigned long long* __restrict__ work) {
-    extern __shared__ double2 sh[];            // [nk] coefficients, then the Givens scratch
-    __shared__ double s_hn2;
+    extern __shared__ double2 hk[];            // [nk] coefficients, then the Hessenberg column
+    __shared__ double2 sa[KW * KSUB], sw[KSUB];
+    __shared__ double s_n[KW], s_hn2;
     const Chunk c = chunks[blockIdx.x];
     if (act && !act[c.seg]) return;
-    if (work && threadIdx.x == 0) atomicAdd(work, (unsigned long long)((nk + 2) * (c.end - c.begin) * sizeof(V)));
-    chunk_update_body<V>(c, basis, ld, nk, ga.h2, ga.ldh, w, nrm_part, sh);
-    if (!last_block_of_segment(c.seg, ga.seg_ch, ga.cnt)) return;
+    if (work && threadIdx.x == 0) atomicAdd(work, (unsigned long long)((nk + 2) * (c.end - c.begin) * sizeof(double2)));
+    for (int k = threadIdx.x; k < nk; k += KT) hk[k] = ga.h2[(int64_t)c.seg * ga.ldh + k];
+    __syncthreads();
+    double nr = 0;
+    for (int64_t e0 = c.begin; e0 < c.end; e0 += KSUB) {
+        const double2 a = sub_chunk_update(basis, ld, nk, e0, c.end, hk, w, sa, sw);
+        nr += a.x * a.x + a.y * a.y;
+    }
+    for (int o = 16; o > 0; o >>= 1) nr += __shfl_xor_sync(0xffffffffu, nr, o);
+    if ((threadIdx.x & 31) == 0) s_n[threadIdx.x >> 5] = nr;
+    __syncthreads();
     if (threadIdx.x == 0) {
+        double s = 0;
+        for (int q = 0; q < KSUB / 32; ++q) s += s_n[q];
+        nrm_part[blockIdx.x] = s;
+    }
+    if (!last_block_of_segment(c.seg, ga.seg_ch, ga.cnt)) return;
+    if (threadIdx.x < 32) {                    // the chunks' norms, lane by lane in chunk order
         double t = 0;
-        for (int cc = ga.seg_ch[c.seg]; cc < ga.seg_ch[c.seg + 1]; ++cc) t += __ldcg(&nrm_part[cc]);
-        s_hn2 = t;
+        for (int cc = ga.seg_ch[c.seg] + threadIdx.x; cc < ga.seg_ch[c.seg + 1]; cc += 32) t += __ldcg(&nrm_part[cc]);
+        for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+        if (threadIdx.x == 0) s_hn2 = t;
     }
     __syncthreads();
     if (threadIdx.x < 32) {
         const int j = ga.j;
-        double2* hin = sh;                   // [j+1] h1 + h2
+        double2* hin = hk;                     // [j+1] h1 + h2
         for (int i = threadIdx.x; i <= j; i += 32)
             hin[i] = cadd(ga.h1[(int64_t)c.seg * ga.ldh + i], ga.h2[(int64_t)c.seg * ga.ldh + i]);
         __syncwarp();
@@ -251,14 +266,13 @@ struct Krylov {
             for (auto& e : ring_ev) THM_CUDA(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
         }
         // the kernels are shared by every instance: only ever raise their limit
-        size_t dots_smem = (size_t)(m + 1) * (KT / 32) * sizeof(double2);
-        THM_REQUIRE(dots_smem <= 200 * 1024, "restart length too large");
+        const size_t dots_smem = 2 * (size_t)(m + 1) * sizeof(double2);
+        THM_REQUIRE((size_t)(m + 1) * KW * sizeof(double2) <= 200 * 1024, "restart length too large");
         static size_t dots_attr = 0;
         if (dots_smem > dots_attr) {
-            THM_CUDA(cudaFuncSetAttribute(k_chunk_dots<V>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dots_smem));
-            THM_CUDA(cudaFuncSetAttribute(k_update_givens<V>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                          (int)givens_smem(m)));
-            THM_CUDA(cudaFuncSetAttribute(k_update_dots<V>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dots_smem));
+            THM_CUDA(cudaFuncSetAttribute(k_chunk_dots, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dots_smem));
+            THM_CUDA(cudaFuncSetAttribute(k_update_givens, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dots_smem));
+            THM_CUDA(cudaFuncSetAttribute(k_update_dots, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dots_smem));
             dots_attr = dots_smem;
         }
         THM_CUDA(cudaDeviceSynchronize());
@@ -268,10 +282,6 @@ struct Krylov {
         THM_LAUNCH(THM_K_KRYLOV, st, k_chunk_norm2<V><<<nch, KT, 0, st>>>(d_chunks.p, x, nrm_part.p));
         THM_LAUNCH(THM_K_KRYLOV, st, k_seg_reduce_real<<<nblk(nseg), 256, 0, st>>>(nseg, seg_ch.p, nrm_part.p, nrm.p));
     }
-
-    // dynamic shared memory of k_update_givens at step j <= m-1: the nk = j+1
-    // coefficients, or the Hessenberg column
-    static size_t givens_smem(int mm) { return (size_t)mm * sizeof(double2); }
 
     unsigned long long* kw(int k) const { return work ? work + k : nullptr; }
 
@@ -334,20 +344,19 @@ struct Krylov {
                 V* vj = basis.p + (int64_t)j * n;
                 A(vj, w.p);
                 const int nk = j + 1;
-                size_t sm = (size_t)nk * (KT / 32) * sizeof(double2);
+                const size_t sm = (size_t)nk * sizeof(double2);
                 // CGS2: h1 = V^H w, then w -= V h1 and h2 = V^H w in one pass, then
                 // w -= V h2 (the dot kernels reduce their segments themselves); the
                 // second update also forms ||w|| and the Givens step of each segment
-                THM_LAUNCH(THM_K_DOTS, st, k_chunk_dots<V><<<nch, KT, sm, st>>>(d_chunks.p, basis.p, n, nk, w.p, partial.p, m + 1,
+                THM_LAUNCH(THM_K_DOTS, st, k_chunk_dots<<<nch, KT, sm, st>>>(d_chunks.p, basis.p, n, nk, w.p, partial.p, m + 1,
                                                                                active.p, seg_ch.p, cnt.p, h1.p, m + 1, nact,
                                                                                kw(0)));
-                THM_LAUNCH(THM_K_UPDATE, st, k_update_dots<V><<<nch, KT, sm, st>>>(d_chunks.p, basis.p, n, nk, h1.p, m + 1, w.p,
+                THM_LAUNCH(THM_K_UPDATE, st, k_update_dots<<<nch, KT, 2 * sm, st>>>(d_chunks.p, basis.p, n, nk, h1.p, m + 1, w.p,
                                                                                   partial.p, m + 1, active.p, seg_ch.p,
                                                                                   cnt.p, h2.p, kw(1)));
                 GivensArgs ga{j, m, m + 1, h1.p, h2.p, Rm.p, cs.p, sn.p, gv.p, pp.p, pq.p, ip.p, target.p, active.p, kused.p, beta.p,
                               nact, flag, nseg == 1 ? gmon : nullptr, seg_ch.p, cnt.p};
-                const size_t gsm = (size_t)(j + 1) * sizeof(double2);
-                THM_LAUNCH(THM_K_UPDATE, st, k_update_givens<V><<<nch, KT, gsm, st>>>(d_chunks.p, basis.p, n, nk, w.p, nrm_part.p,
+                THM_LAUNCH(THM_K_UPDATE, st, k_update_givens<<<nch, KT, sm, st>>>(d_chunks.p, basis.p, n, nk, w.p, nrm_part.p,
                                                                                       active.p, ga, kw(1)));
                 THM_LAUNCH(THM_K_KRYLOV, st, k_chunk_scale<V><<<nch, 256, 0, st>>>(d_chunks.p, w.p, beta.p, basis.p + (int64_t)(j + 1) * n, active.p));
                 ++total;
@@ -440,12 +449,14 @@ static void ensure_work(thm_sys* s, bool fp32, int m_in, int m_out) {
         // one Krylov segment per problem (its contiguous range of interface
         // entries); a single problem is one segment over all of them
         std::vector<Chunk> oc;
+        // chunks as small as a warp holds while there are SMs for them (152)
+        const int64_t step = KSUB * std::max<int64_t>(1, (m->n_if + 152 * KSUB - 1) / (152 * KSUB));
         for (int p = 0; p < m->n_prob; ++p) {
             const int64_t b0 = m->n_prob > 1 ? m->prob_if_ptr[p] : 0;
             const int64_t b1 = m->n_prob > 1 ? m->prob_if_ptr[p + 1] : m->n_if;
-            for (int64_t b = b0; b < b1; b += CHUNK) {
+            for (int64_t b = b0; b < b1; b += step) {
                 Chunk c{};
-                c.seg = p; c.begin = b; c.end = std::min<int64_t>(b1, b + CHUNK);
+                c.seg = p; c.begin = b; c.end = std::min<int64_t>(b1, b + step);
                 oc.push_back(c);
             }
         }
