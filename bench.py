@@ -406,7 +406,7 @@ def table1_arm(args):
             "unit": "iterations", "data": "synthetic",
             "config": {"workload": "block_benchmark: unit square, 64x64 order-2 quads (one domain), centre block "
                                    "[0.25,0.75]^2 with n=1.516 (eps=n^2), mu^-1=1, Dirichlet x=0, impedance elsewhere",
-                       "preconditioner": "Eq. 7 with the exact P^-1 (twisted block-tridiagonal factorisation)"},
+                       "preconditioner": "Eq. 7 with the exact P^-1 (nested dissection)"},
             "rows": rows,
             "paper_table1": {"omega": list(TABLE1_OMEGAS), "iters": list(TABLE1_PAPER),
                              "context": "AMG (MueLu) approximation of P^-1, mesh and order not stated, Xeon 8268"}}
@@ -589,7 +589,7 @@ def main():
     if mode == "mixed" and args.full_steps > 0:
         step(mode, precond="full", outer_maxit=3, max_refine=1, check=False)
         torch.cuda.synchronize()
-        full = {"precond": "full 2x2 block operator, exact inverse (T_i^-1 from complex twisted factors)",
+        full = {"precond": "full 2x2 block operator, exact inverse (T_i^-1 from complex factors)",
                 "eq7_inner_iters": stats_all[-1]["inner_iters"], "eq7_time_to_1e8_s": statistics.median(tt)}
         for rlx in (0, 1):
             g0 = torch.cuda.Event(enable_timing=True)

@@ -8,14 +8,15 @@
 // stopping test, with cluster barriers between them.  Step by step as kernels
 // over all subdomains (5 launches and a monitor copy per step) a step of the
 // 32x32 order-1 problem took 230 us, nearly all of it launch and tail latency;
-// in this kernel a step takes 43 us.  Whole solves, before and after: 32x32
-// order 1 FP64 1315 -> 284 ms, 48x48 order 2 mixed 978 -> 692 ms, the gradient
-// of a 6^3 cube 1900 -> 1000 ms; one sweep of 64 subdomains of 8^3 cells
-// 25.3 -> 17.1 ms, of 64 of 32^2 cells order 2 mixed 26.4 -> 25.7 ms, of 16 of
-// 32^2 cells order 2 FP64 49 -> 57 ms (slower: 128 of the SMs' FP64 units share
+// in this kernel a step takes about 45 us.  Whole solves, before and after
+// (with the shorter scalar step of krylov.cuh and the interface passes there):
+// 32x32 order 1 FP64 1315 -> 250 ms, 48x48 order 2 mixed 978 -> 623 ms, the
+// gradient of a 6^3 cube 1900 -> 829 ms; one sweep of 64 subdomains of 8^3
+// cells 25.3 -> 16.2 ms, of 64 of 32^2 cells order 2 mixed 26.4 -> 25.2 ms, of
+// 16 of 32^2 cells order 2 FP64 49 -> 58 ms (slower: 128 of the SMs' FP64 units share
 // the Gram-Schmidt passes that all of them took as kernels of their own).
 // What bounds it: latencies (a cluster barrier about 1k cycles, an L2 load
-// 700 to 1200, the scalar step's FP64 chain about 10k) on small subdomains;
+// 700 to 1200, the scalar step's FP64 chain 5 to 10k) on small subdomains;
 // on large ones the factor stream and, in FP64, the FP64 units (2 FMA per
 // clock and SM): the Gram-Schmidt passes of step 36 alone are 150k cycles.
 //
