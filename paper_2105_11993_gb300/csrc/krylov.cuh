@@ -194,14 +194,14 @@ __device__ __forceinline__ void backsolve(int m, int k, const double2* R, const 
         for (int p = 0; p < NP; ++p) {
             const int i = lane + 32 * p;
             if (i < q) {
-                gsh[i].x -= c[p].x * yq.x - c[p].y * yq.y;
-                gsh[i].y -= c[p].x * yq.y + c[p].y * yq.x;
+                gsh[i].x = fma(-c[p].x, yq.x, fma(c[p].y, yq.y, gsh[i].x));
+                gsh[i].y = fma(-c[p].x, yq.y, fma(-c[p].y, yq.x, gsh[i].y));
             }
         }
         for (int i = lane + 32 * NP; i < q; i += 32) {
             const double2 v = R[(int64_t)q * m + i];
-            gsh[i].x -= v.x * yq.x - v.y * yq.y;
-            gsh[i].y -= v.x * yq.y + v.y * yq.x;
+            gsh[i].x = fma(-v.x, yq.x, fma(v.y, yq.y, gsh[i].x));
+            gsh[i].y = fma(-v.x, yq.y, fma(-v.y, yq.x, gsh[i].y));
         }
         __syncwarp();
     }
@@ -261,8 +261,8 @@ __device__ __forceinline__ void sub_chunk_dots(const double2* __restrict__ basis
             if (e0 + 32 * q >= end) break;
 #pragma unroll
             for (int b = 0; b < KB; ++b) {
-                a[2 * b] += v[b][q].x * wr[q].x + v[b][q].y * wr[q].y;         // conj(v) * w
-                a[2 * b + 1] += v[b][q].x * wr[q].y - v[b][q].y * wr[q].x;
+                a[2 * b] = fma(v[b][q].x, wr[q].x, fma(v[b][q].y, wr[q].y, a[2 * b]));         // conj(v) * w
+                a[2 * b + 1] = fma(v[b][q].x, wr[q].y, fma(-v[b][q].y, wr[q].x, a[2 * b + 1]));
             }
         }
         const double t = warp_sum_many<2 * KB>(a, lane);     // lane l: value l / 4
@@ -317,8 +317,8 @@ __device__ __forceinline__ double2 sub_chunk_update(const double2* __restrict__ 
 #pragma unroll
             for (int b = 0; b < KB; ++b) {
                 const double2 hv = hk[min(k0 + b, nk - 1)];    // beyond nk - 1 the vectors are zeros
-                x[q].x += hv.x * v[b][q].x - hv.y * v[b][q].y;
-                x[q].y += hv.x * v[b][q].y + hv.y * v[b][q].x;
+                x[q].x = fma(hv.x, v[b][q].x, fma(-hv.y, v[b][q].y, x[q].x));
+                x[q].y = fma(hv.x, v[b][q].y, fma(hv.y, v[b][q].x, x[q].y));
             }
         }
     }

