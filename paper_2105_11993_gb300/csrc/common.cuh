@@ -4,6 +4,7 @@
 #include <cuda_runtime.h>
 #include <cstdint>
 #include <cstring>
+#include <memory>
 #include <string>
 #include <vector>
 
@@ -82,6 +83,34 @@ void prof_read(int cls, int64_t* launches, double* ms);
         ::thm::prof_end((cls), (st));       \
     } while (0)
 
+// Device copies of elimination-tree tables (nd.cuh).
+struct NdDev {
+    DArr<NdPart> parts;
+    DArr<NdLev> levs;
+    DArr<int2> slt;
+    DArr<uint32_t> rowd, rowm, ymap, rmap;
+    DArr<uint16_t> idx;
+    DArr<int32_t> perm, rows, cmap, childs;
+    DArr<int64_t> welem;
+    DArr<NdNode> nodes;
+};
+
+// Lengths of the arrays that tables are put behind.  place_tables: moves their
+// positions there; false if one outgrows 32 bits.
+struct NdPlace { size_t levs, slt, rowd, ymap, rmap, idx, perm, fac; };
+
+// Tables of a system that moved unknowns up the trees of some subdomains: the
+// mesh's tables followed by those of these subdomains, which `parts` points to.
+// (nodes, rows, cmap, childs: of the subdomains eliminated last.)
+struct NdOwn {
+    NdDev d;
+    NdSizes z;                // of both
+    int64_t fac_elems = 0;
+    std::vector<NdPart> parts;
+    std::vector<int64_t> welem;
+    std::vector<std::vector<NdMove>> moves;     // [n_sub]
+};
+
 constexpr int SELL_C = 32;       // rows per SELL slice (one warp)
 constexpr int CHUNK = 1024;      // elements per reduction chunk of a segment
 
@@ -153,16 +182,7 @@ struct thm_mesh {
     // elimination trees of the subdomains (the block preconditioner's factorisation)
     thm::NdHost nd;
     bool nd_ok = false;                             // false: a subdomain outgrows the solve kernel
-    struct {
-        thm::DArr<thm::NdPart> parts;
-        thm::DArr<thm::NdLev> levs;
-        thm::DArr<int2> slt;
-        thm::DArr<uint32_t> rowd, rowm, ymap, rmap;
-        thm::DArr<uint16_t> idx;
-        thm::DArr<int32_t> perm, rows, cmap, childs;
-        thm::DArr<int64_t> welem;
-        thm::DArr<thm::NdNode> nodes;
-    } ndd;
+    thm::NdDev ndd;
     // reduction chunks over subdomains
     std::vector<thm::Chunk> chunks;
     // interface entries (directed pairs i <- j, one per free DOF on Sigma_ij)
@@ -253,6 +273,12 @@ struct thm_sys {
     bool facc64_ok = false, facc32_ok = false;
     thm::DArr<double2> facc64;
     thm::DArr<float2> facc32;
+    // tables of the factors of P_i and of T_i where they are not the mesh's (else null)
+    std::unique_ptr<thm::NdOwn> own, ownc;
+    const thm::NdSizes& nd_sizes(bool cplx) const {
+        const auto& o = cplx ? ownc : own;
+        return o ? o->z : m->nd.z;
+    }
     thm::DArr<int> dev_err;            // set by a device-side bounded wait that gave up
     // workspace of the solve kernel for subdomains whose vectors outgrow shared memory
     mutable thm::DArr<double2> nd_glob;
@@ -272,7 +298,13 @@ namespace thm {
 void build_mesh(thm_mesh* m);
 void build_nd(thm_mesh* m);
 void require_nd(const thm_mesh* m);
-NdTables nd_tables(const thm_mesh* m);
+// Tables of the listed subdomains for 2^p CTAs each; moves: per subdomain of
+// the mesh, or null.  False: an index outgrows its 16 bits, or a CTA's vectors
+// its shared memory.
+bool build_tables(const thm_mesh* m, NdHost& H, const std::vector<int>& list, int p,
+                  const std::vector<std::vector<NdMove>>* moves);
+bool place_tables(NdHost& H, const NdPlace& at);
+NdTables nd_tables(const thm_sys* s, bool cplx);
 void assemble(thm_sys* s);
 void ensure_factor(thm_sys* s, bool fp32);
 void ensure_factor_full(thm_sys* s, bool fp32);

@@ -8,6 +8,11 @@
 // 4 bubbles of a cell are the DOFs of a leaf of their own.  The top
 // log2(C) cuts form one root node (C: CTAs per subdomain); below it small
 // nodes absorb their children, which trades a little arithmetic for depth.
+//
+// The order above knows the mesh only.  Where the elimination of a node is
+// unstable with a system's coefficients, some of its unknowns move to an
+// ancestor (ndfactor.cu): the trees of such subdomains are built again for that
+// system with those moves, and their tables follow the mesh's (NdOwn).
 #pragma once
 
 #include <cuda_runtime.h>
@@ -77,11 +82,15 @@ struct NdSizes {              // largest over the CTAs
     int32_t nlev = 0, nslt = 0, nvec = 0, ny = 0, nu[2] = {0, 0};
 };
 
-struct NdHost {               // what build_nd makes
+struct NdMove { int32_t row, node; };           // an unknown's node, where it is not the tree's choice
+struct NdRef { int32_t sub, node, parent; };    // tree node (numbered within its subdomain's tree) of a node
+
+struct NdHost {               // tables of a list of subdomains (the mesh's: of all)
     int C = 1, mw = 1;        // CTAs per subdomain; map words (of two children's entries)
     NdSizes z;
     int64_t fac_elems = 0;    // entries of a factor, with the padding of rows and slices
-    std::vector<int64_t> welem;                 // [n_sub] values of the factor that a solve multiplies by
+    std::vector<int64_t> welem;                 // per subdomain: values of the factor that a solve multiplies by
+    std::vector<NdRef> node_ref;                // per node
     std::vector<int64_t> depth_node, depth_front;   // per depth, deepest first: first node (one more at the end), front entries
     std::vector<int32_t> depth_s, depth_n;      // largest s and s + b
     std::vector<NdPart> parts;

@@ -7,6 +7,25 @@
 // and W, -H^T (forward rows) and -H (backward rows) go straight into the
 // sliced layout the solve reads.  The same kernel factorises the complex
 // T = P + iB (the full 2x2 block operator, 2-D: B diagonal).
+//
+// Pivoting stays inside a node, and that is not enough: a node's subtree is a
+// cavity with conducting walls, and near one of its resonances S = F_ss is
+// nearly singular though P is not.  H and U are then large and the digits of
+// F_bb are lost in U.  Such a node shows in the entries of H, which are of
+// order 1 elsewhere.  A node with |H| > ND_GROWTH names the unknowns that make
+// it singular (nd_pick: one for each near-null direction of S), they move to
+// the parent, the trees of these subdomains are built again and only they are
+// factorised again, until no node is left.  Measured on 64 subdomains of 32x32
+// order-2 cells with tile coefficients, 40 inputs, error of the FP64 solve
+// against a refined one: without the moves up to 3.5 (5 inputs above 1e-9),
+// with them at most 1.3e-11, for 0.02% more values.  4 subdomains of 32x32
+// order-2 cells, uniform, 16 cells per wavelength: error 9e-4 -> 9e-15, and
+// 2416 -> 509 Arnoldi steps of a mixed sweep.
+// The bound: 1000 leaves errors of 6e-9 on the 40 inputs; 30 moves 3 times as
+// many unknowns and factorises again more often (27 ms instead of 18 in the
+// mean) for errors that are no smaller in the worst input (9e-12).
+#include <algorithm>
+
 #include "common.cuh"
 #include "ndsolve.cuh"
 
@@ -22,6 +41,7 @@ template <> struct NdArith<double> {
     static __device__ __forceinline__ double zero() { return 0.0; }
     static __device__ __forceinline__ double one() { return 1.0; }
     static __device__ __forceinline__ double mag(double a) { return fabs(a); }
+    static __device__ __forceinline__ double size(double a) { return fabs(a); }      // mag within a factor of 1.5
     static __device__ __forceinline__ double inv(double a) { return 1.0 / a; }
     static __device__ __forceinline__ double mul(double a, double b) { return a * b; }
     static __device__ __forceinline__ double fma_(double a, double b, double c) { return fma(a, b, c); }
@@ -32,6 +52,7 @@ template <> struct NdArith<double2> {
     static __device__ __forceinline__ double2 zero() { return make_double2(0, 0); }
     static __device__ __forceinline__ double2 one() { return make_double2(1, 0); }
     static __device__ __forceinline__ double mag(double2 a) { return hypot(a.x, a.y); }
+    static __device__ __forceinline__ double size(double2 a) { return fabs(a.x) + fabs(a.y); }
     static __device__ __forceinline__ double2 inv(double2 a) {
         const double d = a.x * a.x + a.y * a.y;
         return make_double2(a.x / d, -a.y / d);
@@ -46,9 +67,9 @@ template <> struct NdArith<double2> {
 
 // In-place inverse of the m x m block W (row stride ld) by Gauss-Jordan with
 // partial pivoting, one CTA.  fcol, frow: m entries of shared memory each.
-// False on a zero or non-finite pivot.
+// 0, or on a zero pivot 1, on a non-finite one 2.
 template <class T>
-__device__ bool nd_invert(T* W, int m, int ld, int* perm, T* fcol, T* frow) {
+__device__ int nd_invert(T* W, int m, int ld, int* perm, T* fcol, T* frow) {
     using A = NdArith<T>;
     __shared__ double s_best[32];
     __shared__ int s_at[32];
@@ -78,11 +99,11 @@ __device__ bool nd_invert(T* W, int m, int ld, int* perm, T* fcol, T* frow) {
                     bi = s_at[w];
                 }
             perm[k] = bi;
-            s_piv = (best > 0 && isfinite(best)) ? bi : -1;
+            s_piv = (best > 0 && isfinite(best)) ? bi : best == 0 ? -1 : -2;
         }
         __syncthreads();
         const int p = s_piv;
-        if (p < 0) return false;
+        if (p < 0) return -p;
         // row k of the result (the pivot row over the pivot) and column k, staged
         const T ip = A::inv(W[(int64_t)p * ld + k]);
         for (int j = tid; j < m; j += nt) {
@@ -115,7 +136,97 @@ __device__ bool nd_invert(T* W, int m, int ld, int* perm, T* fcol, T* frow) {
             }
         }
     __syncthreads();
-    return true;
+    return 0;
+}
+
+// Largest over the block's threads (NaN if there is one); red: 32 entries.
+__device__ __forceinline__ double nd_block_max(double v, double* red) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        const double u = __shfl_xor_sync(0xffffffffu, v, o);
+        if (u > v || u != u) v = u;
+    }
+    __syncthreads();
+    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
+    __syncthreads();
+    v = red[0];
+    for (int w = 1; w < (int)(blockDim.x >> 5); ++w)
+        if (red[w] > v || red[w] != red[w]) v = red[w];
+    return v;
+}
+
+// Entries of H above this move unknowns to the parent.
+constexpr double ND_GROWTH = 100;
+
+// What a factorisation reports: status[0] a non-finite pivot, [1] a zero pivot,
+// [2] the number of moves {node, local row} (at most one per local row).
+struct NdReport {
+    int* status;
+    int2* moves;
+};
+
+// The unknowns of a node that must not be eliminated there.  G = [W | H], s x
+// (s + b): taking unknown d out of the block is a principal pivot step on G,
+//     G_ij -= G_id G_dj / G_dd   (i, j != d),   G_id = -G_id / G_dd,
+// after which column d belongs to the H of the rows that stay.  W is about
+// sum_k v_k v_k^T / lambda_k over the near-null directions of S, so the
+// largest diagonal entry is an unknown with a large part in one of them; they
+// go one by one until the H of the rest is below ND_GROWTH.  gone, col: s entries each.
+template <class T>
+__device__ __noinline__ void nd_pick(T* G, int s, int b, int ld, T* col, int* gone, const int32_t* rows, int node, NdReport rep) {
+    using A = NdArith<T>;
+    __shared__ double s_red[32], s_val[32];
+    __shared__ int s_idx[32];
+    const int tid = threadIdx.x, nt = blockDim.x, lane = tid & 31, warp = tid >> 5;
+    for (int i = tid; i < s; i += nt) gone[i] = 0;
+    __syncthreads();
+    for (int left = s; left > 0; --left) {
+        double best = -1;
+        int d = -1;
+        for (int i = tid; i < s; i += nt) {
+            const double v = gone[i] ? -1.0 : A::mag(G[(int64_t)i * ld + i]);
+            if (v > best) { best = v; d = i; }
+        }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            const double ov = __shfl_xor_sync(0xffffffffu, best, o);
+            const int od = __shfl_xor_sync(0xffffffffu, d, o);
+            if (od >= 0 && (d < 0 || ov > best || (ov == best && od < d))) { best = ov; d = od; }
+        }
+        __syncthreads();
+        if (lane == 0) { s_val[warp] = best; s_idx[warp] = d; }
+        __syncthreads();
+        best = s_val[0];
+        d = s_idx[0];
+        for (int w = 1; w < (nt >> 5); ++w)
+            if (s_idx[w] >= 0 && (d < 0 || s_val[w] > best || (s_val[w] == best && s_idx[w] < d))) { best = s_val[w]; d = s_idx[w]; }
+        if (d < 0 || !(best > 0)) {            // (not reached from finite entries but for a zero diagonal) all of them go
+            for (int i = tid; i < s; i += nt)
+                if (!gone[i]) rep.moves[atomicAdd(&rep.status[2], 1)] = make_int2(node, rows[i]);
+            return;
+        }
+        const T id = A::inv(G[(int64_t)d * ld + d]);
+        for (int i = tid; i < s; i += nt) col[i] = A::neg(A::mul(G[(int64_t)i * ld + d], id));
+        __syncthreads();
+        if (tid == 0) {
+            gone[d] = 1;
+            rep.moves[atomicAdd(&rep.status[2], 1)] = make_int2(node, rows[d]);
+        }
+        __syncthreads();
+        double hm = 0;
+        for (int t = tid; t < s * (s + b); t += nt) {
+            const int i = t / (s + b), j = t - i * (s + b);
+            if (gone[i]) continue;
+            T* g = G + (int64_t)i * ld + j;
+            const T v = j == d ? col[i] : A::fma_(col[i], G[(int64_t)d * ld + j], *g);
+            *g = v;
+            if (j >= s || gone[j]) {
+                const double a = A::size(v);
+                if (!(a <= hm)) hm = a;
+            }
+        }
+        if (nd_block_max(hm, s_red) <= ND_GROWTH) return;
+    }
 }
 
 __device__ __forceinline__ int nd_find(const int32_t* a, int n, int32_t v) {
@@ -154,7 +265,7 @@ __global__ void k_nd_factor(NdTables tab, const NdNode* __restrict__ nodes, int6
                             int max_s, const int64_t* __restrict__ slice_ptr, const int32_t* __restrict__ col,
                             const uint8_t* __restrict__ pad, const double* __restrict__ val,
                             const double* __restrict__ bg, const double* __restrict__ bs, T* front, const T* below,
-                            T* aux, T* fac, int* __restrict__ status) {
+                            T* aux, T* fac, NdReport rep) {
     using A = NdArith<T>;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     T* fcol = reinterpret_cast<T*>(smem_raw);
@@ -221,8 +332,12 @@ __global__ void k_nd_factor(NdTables tab, const NdNode* __restrict__ nodes, int6
         S = X;
     }
     __syncthreads();
-    if (!nd_invert(W, s, ld, perm, fcol, frow)) {
-        if (tid == 0) atomicExch(status, 1);
+    if (const int bad = nd_invert(W, s, ld, perm, fcol, frow)) {
+        if (tid == 0) atomicExch(&rep.status[bad == 2 ? 0 : 1], 1);
+        if (bad == 1 && b > 0) {                       // exactly singular: all of it moves up
+            for (int i = tid; i < s; i += nt)
+                rep.moves[atomicAdd(&rep.status[2], 1)] = make_int2((int)(node0 + blockIdx.x), rs[i]);
+        }
         return;
     }
     // One Newton step, W += W (I - S W): Gauss-Jordan leaves an error of
@@ -257,8 +372,11 @@ __global__ void k_nd_factor(NdTables tab, const NdNode* __restrict__ nodes, int6
     __syncthreads();
     nd_gemm<T>(s, b, s, S, n, Y, n, [&](int i, int j, T a) { Rs[(int64_t)i * n + j] = A::add(Fb[(int64_t)i * n + j], A::neg(a)); });
     __syncthreads();
+    double hm = 0;
     nd_gemm<T>(s, b, s, W, ld, Rs, n, [&](int i, int j, T a) {
         const T h = A::neg(A::add(Y[(int64_t)i * n + j], a));
+        const double v = A::size(h);
+        if (!(v <= hm)) hm = v;
         fac[nd_at(sf, N.row_f + s + j, i)] = h;
         fac[nd_at(sb, N.row_b + i, j)] = h;
     });
@@ -271,15 +389,29 @@ __global__ void k_nd_factor(NdTables tab, const NdNode* __restrict__ nodes, int6
         for (int k = 0; k < s; ++k) a = A::fma_(F[(int64_t)(s + i) * n + k], h[(k >> 2) * 128 + (k & 3)], a);
         *d = a;
     }
+    __shared__ double s_red[32];
+    hm = nd_block_max(hm, s_red);
+    if (hm <= ND_GROWTH) return;
+    if (!isfinite(hm)) {
+        if (tid == 0) atomicExch(&rep.status[0], 1);
+        return;
+    }
+    for (int t = tid; t < s * n; t += nt) {            // [W | H] over the scratch, which is free
+        const int i = t / n, j = t - i * n;
+        Y[t] = j < s ? W[(int64_t)i * ld + j] : A::neg(fac[nd_at(sb, N.row_b + i, j - s)]);
+    }
+    __syncthreads();
+    nd_pick<T>(Y, s, b, n, fcol, perm, rs, (int)(node0 + blockIdx.x), rep);
 }
 
-NdTables nd_tables(const thm_mesh* m) {
-    const auto& D = m->ndd;
+NdTables nd_tables(const thm_sys* s, bool cplx) {
+    const auto& own = cplx ? s->ownc : s->own;
+    const NdDev& D = own ? own->d : s->m->ndd;
     NdTables T{};
     T.parts = D.parts.p; T.levs = D.levs.p; T.slt = D.slt.p;
     T.rowd = D.rowd.p; T.rowm = D.rowm.p; T.ymap = D.ymap.p; T.rmap = D.rmap.p;
-    T.idx = D.idx.p; T.perm = D.perm.p; T.welem = D.welem.p; T.subs = m->d_subs.p;
-    T.mw = m->nd.mw;
+    T.idx = D.idx.p; T.perm = D.perm.p; T.welem = D.welem.p; T.subs = s->m->d_subs.p;
+    T.mw = s->m->nd.mw;
     return T;
 }
 
@@ -287,43 +419,137 @@ void require_nd(const thm_mesh* m) {
     THM_REQUIRE(m->nd_ok, "subdomain too large for the shared-memory block solve");
 }
 
+// dst = base, `add` behind it, and room for `more` entries
+template <class X>
+static void append(DArr<X>& dst, const DArr<X>& base, const std::vector<X>& add, cudaStream_t st, size_t more = 0) {
+    DArr<X> a;
+    a.alloc(base.n + add.size() + more);
+    if (base.n) THM_CUDA(cudaMemcpyAsync(a.p, base.p, base.n * sizeof(X), cudaMemcpyDeviceToDevice, st));
+    if (!add.empty()) THM_CUDA(cudaMemcpyAsync(a.p + base.n, add.data(), add.size() * sizeof(X), cudaMemcpyHostToDevice, st));
+    THM_CUDA(cudaStreamSynchronize(st));
+    std::swap(dst.p, a.p);
+    std::swap(dst.n, a.n);
+}
+
+// Builds the trees of the subdomains of `found` again with these unknowns of
+// nodes of H in the parents, and puts their tables behind the present ones
+// (own: null while these are the mesh's).  False, and nothing changed: they
+// outgrow the solve kernel.
+static bool move_up(const thm_sys* s, const NdHost& H, const std::vector<int2>& found, std::unique_ptr<NdOwn>& own, NdHost& out) {
+    const thm_mesh* m = s->m;
+    cudaStream_t st = s->st;
+    const int C = m->nd.C;
+    auto moves = own ? own->moves : std::vector<std::vector<NdMove>>(m->n_sub);
+    std::vector<int> list;
+    for (const int2& f : found) {
+        const NdRef& r = H.node_ref[f.x];
+        auto& v = moves[r.sub];
+        auto it = std::lower_bound(v.begin(), v.end(), f.y, [](const NdMove& a, int row) { return a.row < row; });
+        if (it != v.end() && it->row == f.y) it->node = r.parent;
+        else v.insert(it, NdMove{f.y, r.parent});
+        list.push_back(r.sub);
+    }
+    std::sort(list.begin(), list.end());
+    list.erase(std::unique(list.begin(), list.end()), list.end());
+    int p = 0;
+    while ((1 << p) < C) ++p;
+    if (!build_tables(m, out, list, p, &moves)) return false;
+    const NdDev& B = own ? own->d : m->ndd;
+    const int64_t fac0 = own ? own->fac_elems : m->nd.fac_elems;
+    if (!place_tables(out, NdPlace{B.levs.n, B.slt.n, B.rowd.n, B.ymap.n, B.rmap.n, B.idx.n, B.perm.n, (size_t)fac0})) return false;
+    std::unique_ptr<NdOwn> o(new NdOwn());
+    append(o->d.levs, B.levs, out.levs, st);
+    append(o->d.slt, B.slt, out.slt, st);
+    append(o->d.rowd, B.rowd, out.rowd, st);
+    append(o->d.rowm, B.rowm, out.rowm, st);
+    append(o->d.ymap, B.ymap, out.ymap, st);
+    append(o->d.rmap, B.rmap, out.rmap, st);
+    append(o->d.idx, B.idx, out.idx, st);
+    append(o->d.perm, B.perm, out.perm, st);
+    o->parts = own ? own->parts : m->nd.parts;
+    o->welem = own ? own->welem : m->nd.welem;
+    for (size_t i = 0; i < list.size(); ++i) {
+        for (int k = 0; k < C; ++k) o->parts[(size_t)list[i] * C + k] = out.parts[i * C + k];
+        o->welem[list[i]] = out.welem[i];
+    }
+    o->d.parts.upload(o->parts, st);
+    o->d.welem.upload(o->welem, st);
+    o->d.nodes.upload(out.nodes, st);
+    o->d.rows.upload(out.rows, st);
+    o->d.cmap.upload(out.cmap, st);
+    o->d.childs.upload(out.childs, st);
+    o->z = s->nd_sizes(&own == &s->ownc);
+    o->z.nlev = std::max(o->z.nlev, out.z.nlev);
+    o->z.nslt = std::max(o->z.nslt, out.z.nslt);
+    o->z.nvec = std::max(o->z.nvec, out.z.nvec);
+    o->z.ny = std::max(o->z.ny, out.z.ny);
+    for (int k = 0; k < 2; ++k) o->z.nu[k] = std::max(o->z.nu[k], out.z.nu[k]);
+    o->fac_elems = fac0 + out.fac_elems;
+    o->moves.swap(moves);
+    own.swap(o);
+    return true;
+}
+
 template <class T>
 static void factor(thm_sys* s, DArr<T>& fac, const char* what) {
+    constexpr bool cplx = NdCplx<T>::value;
     const thm_mesh* m = s->m;
-    const NdHost& H = m->nd;
     cudaStream_t st = s->st;
     require_nd(m);
-    fac.alloc(H.fac_elems);
+    std::unique_ptr<NdOwn>& own = cplx ? s->ownc : s->own;
+    own.reset();
+    fac.alloc(m->nd.fac_elems);
     fac.zero(st);
-    int64_t most[2] = {0, 0};
-    const int nd = (int)H.depth_front.size();
-    for (int d = 0; d < nd; ++d) most[d & 1] = std::max(most[d & 1], H.depth_front[d]);
     DArr<T> front[2], aux;
-    front[0].alloc(most[0]);
-    front[1].alloc(most[1]);
-    aux.alloc(3 * std::max(most[0], most[1]));
     DArr<int> status;
-    status.alloc(1);
-    status.zero(st);
+    status.alloc(3);
+    DArr<int2> moves;
+    moves.alloc(m->n_loc);
+    THM_CUDA(cudaFuncSetAttribute(k_nd_factor<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, 225 * 1024));
     const size_t cap = 200 * 1024;
-    THM_CUDA(cudaFuncSetAttribute(k_nd_factor<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, 226 * 1024));
-    for (int d = 0; d < nd; ++d) {
-        const int64_t n0 = H.depth_node[d], cnt = H.depth_node[d + 1] - n0;
-        const int ms = std::max(1, H.depth_s[d]), mn = H.depth_n[d];
-        // blocks up to smem_s in shared memory; the others of the depth in place
-        const int smem_s = (size_t)ms * ms * sizeof(T) <= cap ? ms : 0;
-        const size_t smem = (size_t)2 * ms * sizeof(T) + (size_t)smem_s * smem_s * sizeof(T) + (size_t)ms * sizeof(int);
-        int threads = 32;
-        while (threads < 512 && threads * 16 < mn * mn) threads *= 2;
-        THM_LAUNCH(THM_K_SETUP, st, k_nd_factor<T><<<(unsigned)cnt, threads, smem, st>>>(
-            nd_tables(m), m->ndd.nodes.p, n0, m->ndd.rows.p, m->ndd.cmap.p, m->ndd.childs.p, H.C, smem_s, ms,
-            m->d_slice_ptr.p, m->d_sell_col.p, m->d_sell_pad.p, s->val64.p, s->bg64.p, s->bs64.p, front[d & 1].p,
-            front[(d + 1) & 1].p, aux.p, fac.p, status.p));
-        THM_CUDA(cudaGetLastError());
+    NdHost again;                                      // the subdomains that are factorised again
+    for (bool first = true;; first = false) {
+        const NdHost& H = first ? m->nd : again;
+        const NdDev& D = first ? m->ndd : own->d;
+        int64_t most[2] = {0, 0};
+        const int nd = (int)H.depth_front.size();
+        for (int d = 0; d < nd; ++d) most[d & 1] = std::max(most[d & 1], H.depth_front[d]);
+        for (int k = 0; k < 2; ++k)
+            if ((int64_t)front[k].n < most[k]) front[k].alloc(most[k]);
+        if ((int64_t)aux.n < 3 * std::max(most[0], most[1])) aux.alloc(3 * std::max(most[0], most[1]));
+        status.zero(st);
+        for (int d = 0; d < nd; ++d) {
+            const int64_t n0 = H.depth_node[d], cnt = H.depth_node[d + 1] - n0;
+            const int ms = std::max(1, H.depth_s[d]), mn = H.depth_n[d];
+            // blocks up to smem_s in shared memory; the others of the depth in place
+            const int smem_s = (size_t)ms * ms * sizeof(T) <= cap ? ms : 0;
+            const size_t smem = (size_t)2 * ms * sizeof(T) + (size_t)smem_s * smem_s * sizeof(T) + (size_t)ms * sizeof(int);
+            int threads = 32;
+            while (threads < 512 && threads * 16 < mn * mn) threads *= 2;
+            THM_LAUNCH(THM_K_SETUP, st, k_nd_factor<T><<<(unsigned)cnt, threads, smem, st>>>(
+                nd_tables(s, cplx), D.nodes.p, n0, D.rows.p, D.cmap.p, D.childs.p, H.C, smem_s, ms,
+                m->d_slice_ptr.p, m->d_sell_col.p, m->d_sell_pad.p, s->val64.p, s->bg64.p, s->bs64.p, front[d & 1].p,
+                front[(d + 1) & 1].p, aux.p, fac.p, NdReport{status.p, moves.p}));
+            THM_CUDA(cudaGetLastError());
+        }
+        std::vector<int> hs;
+        status.download(hs, st);
+        if (hs[0] != 0 || (hs[1] != 0 && hs[2] == 0)) fail(THM_ESINGULAR, what);
+        if (hs[2] == 0) break;
+        std::vector<int2> found(hs[2]);
+        THM_CUDA(cudaMemcpyAsync(found.data(), moves.p, found.size() * sizeof(int2), cudaMemcpyDeviceToHost, st));
+        THM_CUDA(cudaStreamSynchronize(st));
+        std::sort(found.begin(), found.end(), [](const int2& a, const int2& b) { return a.x != b.x ? a.x < b.x : a.y < b.y; });
+        NdHost next;
+        if (!move_up(s, H, found, own, next)) {        // trees too large for the solve kernel: the factors as they are
+            if (hs[1] != 0) fail(THM_ESINGULAR, what);
+            break;
+        }
+        std::swap(again, next);
+        const size_t n0 = fac.n;
+        append(fac, fac, std::vector<T>(), st, again.fac_elems);
+        THM_CUDA(cudaMemsetAsync(fac.p + n0, 0, (fac.n - n0) * sizeof(T), st));
     }
-    std::vector<int> hs;
-    status.download(hs, st);
-    if (hs[0] != 0) fail(THM_ESINGULAR, what);
 }
 
 __global__ void k_to_float2(int64_t n, const double2* __restrict__ a, float2* __restrict__ b) {

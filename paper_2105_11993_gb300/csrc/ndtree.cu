@@ -93,8 +93,9 @@ void bisect(const thm_mesh* m, std::vector<int32_t>& cs, int leaf, std::vector<B
     cs.swap(out);
 }
 
-// The tree of subdomain s for C = 2^p CTAs.
-void build_tree(const thm_mesh* m, int s, std::vector<int32_t> cs, int p, std::vector<int32_t>& cell_bin, SubTree& T) {
+// The tree of subdomain s for C = 2^p CTAs, with the unknowns of `moves` in the nodes it names.
+void build_tree(const thm_mesh* m, int s, std::vector<int32_t> cs, int p, const std::vector<NdMove>* moves,
+                std::vector<int32_t>& cell_bin, SubTree& T) {
     const auto& S = m->subs[s];
     std::vector<Bin> bins;
     bisect(m, cs, leaf_cells(m), bins);
@@ -155,6 +156,13 @@ void build_tree(const thm_mesh* m, int s, std::vector<int32_t> cs, int p, std::v
             T.nodes.push_back(N);
             T.nodes[host].ch.push_back(cell_node[i]);
         }
+    if (moves && !moves->empty()) {
+        std::vector<int32_t> to(S.n, -1);
+        for (const NdMove& v : *moves) to[v.row - S.off] = v.node;
+        for (auto& N : T.nodes)
+            N.s.erase(std::remove_if(N.s.begin(), N.s.end(), [&](int32_t r) { return to[r - S.off] >= 0; }), N.s.end());
+        for (const NdMove& v : *moves) T.nodes[v.node].s.push_back(v.row);
+    }
     // depths and ancestor unknowns, children before parents (a parent's number is lower than its children's)
     T.maxdepth = 0;
     std::vector<std::vector<int32_t>> own(T.nodes.size());
@@ -162,9 +170,9 @@ void build_tree(const thm_mesh* m, int s, std::vector<int32_t> cs, int p, std::v
         T.nodes[q].depth = T.nodes[T.nodes[q].parent].depth + 1;
         T.maxdepth = std::max(T.maxdepth, T.nodes[q].depth);
     }
-    const int dpc = m->dpc, nedge = m->order == 2 ? 8 : dpc;
+    const int dpc = m->dpc;                            // (what a node eliminates itself is sorted out below)
     for (size_t i = 0; i < cs.size(); ++i)
-        for (int k = 0; k < nedge; ++k) {
+        for (int k = 0; k < dpc; ++k) {
             const int32_t r = m->cell_loc[(int64_t)cs[i] * dpc + k];
             if (r >= 0) own[m->order == 2 ? cell_node[i] : bins[cell_bin[cs[i]]].node].push_back(r);
         }
@@ -200,11 +208,21 @@ int pad4(int v) { return (v + 3) / 4 * 4; }
 
 }  // namespace
 
-// Tables for C = 2^p CTAs per subdomain.  False: an index outgrows its 16 bits.
-bool build_tables(thm_mesh* m, const std::vector<std::vector<int32_t>>& cells, int p) {
-    const int ns = m->n_sub, C = 1 << p, mw = m->maxc / 2;
-    auto& H = m->nd;
+// Shared memory of a solve CTA in FP64 (the larger of the two precisions),
+// with everything but the vector itself moved out if need be.
+static size_t smallest_smem(const NdSizes& z) { return nd_layout<double2>(z, 0, 1, 1).total; }
+
+bool build_tables(const thm_mesh* m, NdHost& H, const std::vector<int>& list, int p,
+                  const std::vector<std::vector<NdMove>>* moves) {
+    const int ns = (int)list.size(), C = 1 << p, mw = m->maxc / 2;
     H = NdHost();
+    std::vector<std::vector<int32_t>> cells(ns);
+    {
+        std::vector<int32_t> at(m->n_sub, -1);
+        for (int i = 0; i < ns; ++i) at[list[i]] = i;
+        for (int64_t c = 0; c < m->n_cell; ++c)
+            if (at[m->cell_sub[c]] >= 0) cells[at[m->cell_sub[c]]].push_back((int32_t)c);
+    }
     H.C = C;
     H.mw = mw;
     std::vector<SubTree> trees(ns);
@@ -214,7 +232,8 @@ bool build_tables(thm_mesh* m, const std::vector<std::vector<int32_t>>& cells, i
         std::vector<std::thread> th;
         for (int t = 0; t < nt; ++t)
             th.emplace_back([&, t]() {
-                for (int s = t; s < ns; s += nt) build_tree(m, s, cells[s], p, cell_bin, trees[s]);
+                for (int i = t; i < ns; i += nt)
+                    build_tree(m, list[i], cells[i], p, moves ? &(*moves)[list[i]] : nullptr, cell_bin, trees[i]);
             });
         for (auto& t : th) t.join();
     }
@@ -232,6 +251,7 @@ bool build_tables(thm_mesh* m, const std::vector<std::vector<int32_t>>& cells, i
         for (auto& e : by[d]) {
             Node& N = trees[e.first].nodes[e.second];
             N.id = id++;
+            H.node_ref.push_back({list[e.first], e.second, N.parent});
             const int64_t n = (int64_t)(N.s.size() + N.b.size());
             front += n * n;
             ms = std::max(ms, (int)N.s.size());
@@ -251,7 +271,7 @@ bool build_tables(thm_mesh* m, const std::vector<std::vector<int32_t>>& cells, i
     std::vector<int32_t> place;                            // front index of a local row of the subdomain
     for (int s = 0; s < ns; ++s) {
         SubTree& T = trees[s];
-        const auto& S = m->subs[s];
+        const auto& S = m->subs[list[s]];
         place.assign(S.n, -1);
         for (auto& N : T.nodes) H.welem[s] += (int64_t)N.s.size() * (N.s.size() + 2 * N.b.size());
         const Node& root = T.nodes[0];
@@ -441,7 +461,7 @@ bool build_tables(thm_mesh* m, const std::vector<std::vector<int32_t>>& cells, i
             NdNode& D = nodes[N.id];
             D.s = (int32_t)N.s.size();
             D.b = (int32_t)N.b.size();
-            D.sub = s;
+            D.sub = list[s];
             D.slt_f = N.slt_f;
             D.slt_b = N.slt_b;
             D.row_f = N.row_f;
@@ -466,7 +486,7 @@ bool build_tables(thm_mesh* m, const std::vector<std::vector<int32_t>>& cells, i
     }
     for (int i = 0; i < 64; ++i) H.idx.push_back(0);
     H.fac_elems = fo * 128 + 128;
-    if (!fits) return false;
+    if (!fits || smallest_smem(H.z) > ND_SMEM_MAX) return false;
     H.nodes.swap(nodes);
     H.rows.swap(rows);
     H.cmap.swap(cmap);
@@ -474,14 +494,33 @@ bool build_tables(thm_mesh* m, const std::vector<std::vector<int32_t>>& cells, i
     return true;
 }
 
-// Shared memory of a solve CTA in FP64 (the larger of the two precisions),
-// with everything but the vector itself moved out if need be.
-static size_t smallest_smem(const NdSizes& z) { return nd_layout<double2>(z, 0, 1, 1).total; }
+bool place_tables(NdHost& H, const NdPlace& at) {
+    const size_t most = INT32_MAX, mw = H.mw;
+    if (at.levs + H.levs.size() > most || at.slt + H.slt.size() > most || at.rowd + H.rowd.size() > most ||
+        at.idx + H.idx.size() > most || (at.fac + H.fac_elems) / 128 > most)
+        return false;
+    THM_REQUIRE(at.slt % 2 == 0 && at.idx % 4 == 0 && at.fac % 128 == 0, "internal: tables out of alignment");
+    for (NdPart& P : H.parts) {
+        P.lev0 += (int32_t)at.levs;
+        P.slt0 += (int32_t)at.slt;
+        P.rmap0 += (int32_t)(at.rmap / (2 * mw));
+        P.perm0 += (int64_t)at.perm;
+    }
+    for (NdLev& L : H.levs) {
+        L.rowf += (int32_t)at.rowd;
+        L.rowb += (int32_t)at.rowd;
+        L.ymap += (int32_t)(at.ymap / mw);
+        L.idx += (int32_t)at.idx;
+    }
+    for (int2& v : H.slt) v.x += (int)(at.fac / 128);
+    for (NdNode& N : H.nodes) { N.slt_f += (int32_t)at.slt; N.slt_b += (int32_t)at.slt; }
+    return true;
+}
 
 void build_nd(thm_mesh* m) {
     const int ns = m->n_sub;
-    std::vector<std::vector<int32_t>> cells(ns);
-    for (int64_t c = 0; c < m->n_cell; ++c) cells[m->cell_sub[c]].push_back((int32_t)c);
+    std::vector<int> all(ns);
+    std::iota(all.begin(), all.end(), 0);
     int dev = 0, sms = 0;
     THM_CUDA(cudaGetDevice(&dev));
     THM_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
@@ -490,7 +529,7 @@ void build_nd(thm_mesh* m) {
     int p = 0;
     while (p < 3 && (int64_t)ns * (2 << p) <= 2 * (int64_t)sms && m->n_loc / ns >= (int64_t)(64 << (p + 1))) ++p;
     for (;; ++p) {
-        m->nd_ok = build_tables(m, cells, p) && smallest_smem(m->nd.z) <= ND_SMEM_MAX;
+        m->nd_ok = build_tables(m, m->nd, all, p, nullptr);
         if (m->nd_ok || p == 3) break;
     }
     if (!m->nd_ok) return;                                 // reported by the first apply, as a size limit of the kernel

@@ -550,7 +550,7 @@ template <class V, class FW>
 static bool nd_memory(const thm_sys* s, bool glob, size_t more, size_t keep, NdMem* out, size_t* keep_off, size_t* smem) {
     const thm_mesh* m = s->m;
     require_nd(m);
-    const NdSizes& z = m->nd.z;
+    const NdSizes& z = s->nd_sizes(NdCplx<FW>::value);
     if (!s->bt_work.p) {
         s->bt_work.alloc(4);
         s->bt_work.zero(s->st);
@@ -623,7 +623,7 @@ static void nd_apply(const thm_sys* s, const FW* fac, const V* x, V* y) {
                 "subdomain too large for the shared-memory block solve");
     // the work counter follows the Eq. 7 (real-factor) applies only
     unsigned long long* work = NdCplx<FW>::value ? nullptr : s->bt_work.p + (sizeof(FW) == 4 ? 2 : 0);
-    nd_launch(s, THM_K_PINV, glob ? k_nd_solve<true, V, FW> : k_nd_solve<false, V, FW>, smem, nd_tables(s->m), s->m->nd.z, mm, reinterpret_cast<V*>(s->nd_glob.p),
+    nd_launch(s, THM_K_PINV, glob ? k_nd_solve<true, V, FW> : k_nd_solve<false, V, FW>, smem, nd_tables(s, NdCplx<FW>::value), s->nd_sizes(NdCplx<FW>::value), mm, reinterpret_cast<V*>(s->nd_glob.p),
               fac, nd_wait_ns(), nd_stall(), s->dev_err.p, work, x, y);
 }
 
@@ -688,7 +688,7 @@ static void subsolve(thm_sys* s, const SolveCfg& c, SubWork<V>& k, const FW* fac
     a.kw64 = kwork(s);
     a.kw = a.kw64 + (f32 ? 4 : 0);
     a.bt = NdCplx<FW>::value ? nullptr : s->bt_work.p + (f32 ? 2 : 0);
-    nd_launch(s, THM_K_SUBSOLVE, glob ? k_subsolve<true, V, FW, F> : k_subsolve<false, V, FW, F>, smem, nd_tables(m), m->nd.z, mm, reinterpret_cast<V*>(s->nd_glob.p),
+    nd_launch(s, THM_K_SUBSOLVE, glob ? k_subsolve<true, V, FW, F> : k_subsolve<false, V, FW, F>, smem, nd_tables(s, NdCplx<FW>::value), s->nd_sizes(NdCplx<FW>::value), mm, reinterpret_cast<V*>(s->nd_glob.p),
               fac, a, (int)keep_off, nd_wait_ns(), nd_stall(), s->dev_err.p);
 }
 
