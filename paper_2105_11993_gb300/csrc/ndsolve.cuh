@@ -220,6 +220,21 @@ __host__ __device__ inline NdLayout nd_layout(const NdSizes& z, int slt_smem, in
     return L;
 }
 
+// The workspace of a CTA whose u buffers and staged y are in global memory, in
+// vector entries: u of the even depths at 0.  Every part starts at a multiple
+// of 4 entries, since the staged y is read 16 bytes at a time (nd_y4).
+struct NdGlob {
+    int64_t u1, y, stride;
+};
+__host__ __device__ inline NdGlob nd_glob_layout(const NdSizes& z) {
+    auto r4 = [](int64_t v) { return (v + 3) / 4 * 4; };
+    NdGlob g;
+    g.u1 = r4(z.nu[0]);
+    g.y = g.u1 + r4(z.nu[1]);
+    g.stride = g.y + r4(z.ny);
+    return g;
+}
+
 // Launch options that the host decides from the sizes (nd_memory).
 struct NdMem {
     int slt_smem, u_glob, y_glob, prefetch;
@@ -260,16 +275,17 @@ __device__ __forceinline__ void nd_enter(NdCta<V>& c, const NdTables& T, const N
     c.ysc = reinterpret_cast<V*>(smem + lay.ysc);
     c.u_even = reinterpret_cast<V*>(smem + lay.u0);        // u of the even depths
     c.u_odd = reinterpret_cast<V*>(smem + lay.u1);
+    const NdGlob gw = nd_glob_layout(z);
     if constexpr (GLOB) {
         V* gl = glob + ((int64_t)sub * C + rank) * mm.glob_stride;
         if (!mm.slt_smem) c.slt = T.slt + c.P.slt0;
-        if (mm.y_glob) c.ysc = gl + z.nu[0] + z.nu[1];
+        if (mm.y_glob) c.ysc = gl + gw.y;
         if (mm.u_glob) {
             c.u_even = gl;
-            c.u_odd = gl + z.nu[0];
+            c.u_odd = gl + gw.u1;
         }
     }
-    c.glob = glob + (int64_t)sub * C * mm.glob_stride + z.nu[0];
+    c.glob = glob + (int64_t)sub * C * mm.glob_stride + gw.u1;
     c.glob_stride = mm.glob_stride;
     c.rank = rank;
     c.C = C;

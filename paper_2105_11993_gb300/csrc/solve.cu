@@ -573,7 +573,7 @@ static bool nd_memory(const thm_sys* s, bool glob, size_t more, size_t keep, NdM
         if (need() > ND_SMEM_MAX) mm.y_glob = 1;
     }
     if ((!glob && !mm.slt_smem) || need() > ND_SMEM_MAX) return false;
-    mm.glob_stride = (mm.u_glob || mm.y_glob) ? (int64_t)z.nu[0] + z.nu[1] + z.ny : 0;
+    mm.glob_stride = (mm.u_glob || mm.y_glob) ? nd_glob_layout(z).stride : 0;
     const size_t entries = (size_t)(mm.glob_stride * m->n_sub * m->nd.C);
     if (s->nd_glob.n < entries) s->nd_glob.alloc(entries);
     *out = mm;
