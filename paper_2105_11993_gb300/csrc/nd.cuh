@@ -26,6 +26,7 @@ constexpr int ND_NW = ND_NT / 32;
 constexpr uint32_t ND_NONE = 0xffffu;       // no child entry in a map half-word
 constexpr uint32_t ND_NOROW = 0xffffffffu;  // padding row of a slice
 constexpr size_t ND_SMEM_MAX = 226 * 1024; // dynamic; the kernels keep less than 1 KB of static shared memory
+constexpr int ND_RESTART = 120;             // default restart length of the subdomain solves
 constexpr uint32_t ND_U = 0x8000u;          // destination of a row: an entry of u (else of the vector)
 
 // Tree node, as the factorisation sees it (nodes are sorted by depth, deepest first).

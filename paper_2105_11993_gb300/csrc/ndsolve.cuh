@@ -241,6 +241,55 @@ struct NdMem {
     int64_t glob_stride;
 };
 
+// Work items that a dot-product pass is cut into while there are few basis
+// vectors: three per warp, so that the last round is not nearly empty.
+constexpr int SUB_ITEMS = 3 * ND_NW;
+// Shared memory of a subdomain solve that outlives a step: rotations and g of the cycle (givens_core)
+// and the previous step's [b; d].
+__host__ __device__ inline size_t sub_keep_bytes(int m) { return (size_t)m * 40 + (size_t)(m + 1) * 48 + 48; }
+
+// Bytes of the Krylov phases' shared memory (they reuse the apply's): u and w
+// of the CTA's rows, the totals and the Hessenberg column, the coefficients,
+// the warps' sums.
+template <class V>
+__host__ __device__ inline size_t sub_krylov_bytes(int rows, int m, int k_glob) {
+    const size_t red = (size_t)(m / 4 + 2 + SUB_ITEMS) * 16 * sizeof(typename VT<V>::R);
+    return (k_glob ? 0 : 2 * (size_t)rows * sizeof(V)) + (size_t)(2 * m + 2) * 16 + (size_t)(m + 1) * 16 +
+           (size_t)(2 * m + 2) * sizeof(V) + (red + 15) / 16 * 16;
+}
+// rows of a CTA: the subdomain's local rows in C equal parts of whole warps
+// of the SELL slices, or of 8 where that would leave CTAs without rows
+__host__ __device__ inline int sub_rows(int64_t n, int C) {
+    const int64_t r = (n + C - 1) / C, g = r >= 512 ? 32 : 8;
+    return (int)((r + g - 1) / g * g);
+}
+
+// The shared memory of a solve kernel with vectors V: one function for the
+// build of the trees, which picks the CTAs per subdomain by it, and for the
+// launches.  more: bytes that other phases need over the apply's vectors;
+// keep: bytes beside everything.  glob: the u buffers, then the staged y, then
+// the slice table may move to global memory, in this order, until it fits.
+// Returns the bytes, or 0 if it does not fit.
+template <class V>
+inline size_t nd_fit(const NdSizes& z, bool glob, size_t more, size_t keep, NdMem* mm) {
+    mm->slt_smem = (size_t)z.nslt * sizeof(int2) <= 16 * 1024 ? 1 : 0;
+    mm->u_glob = mm->y_glob = 0;
+    auto need = [&]() {
+        const NdLayout L = nd_layout<V>(z, mm->slt_smem, mm->u_glob, mm->y_glob);
+        const size_t all = L.total > L.vec + more ? L.total : L.vec + more;
+        return (all + 15) / 16 * 16 + keep;
+    };
+    if (glob) {
+        if (need() > ND_SMEM_MAX) mm->u_glob = 1;
+        if (need() > ND_SMEM_MAX) mm->y_glob = 1;
+        if (need() > ND_SMEM_MAX) mm->slt_smem = 0;
+    } else if (!mm->slt_smem) {
+        return 0;
+    }
+    mm->glob_stride = (mm->u_glob || mm->y_glob) ? nd_glob_layout(z).stride : 0;
+    return need() <= ND_SMEM_MAX ? need() : 0;
+}
+
 // Where a CTA's pieces are: built once per launch, used by every apply in it.
 template <class V>
 struct NdCta {

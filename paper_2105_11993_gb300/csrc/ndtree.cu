@@ -208,9 +208,18 @@ int pad4(int v) { return (v + 3) / 4 * 4; }
 
 }  // namespace
 
-// Shared memory of a solve CTA in FP64 (the larger of the two precisions),
-// with everything but the vector itself moved out if need be.
-static size_t smallest_smem(const NdSizes& z) { return nd_layout<double2>(z, 0, 1, 1).total; }
+// Whether an apply, resp. a subdomain solve with m steps per cycle, fits shared
+// memory in FP64 (the larger of the two precisions).
+static bool apply_fits(const NdSizes& z) {
+    NdMem mm{};
+    return nd_fit<double2>(z, true, 0, 0, &mm) > 0;
+}
+static bool solve_fits(const thm_mesh* mesh, const NdSizes& z, int C, int m) {
+    NdMem mm{};
+    int64_t n = 0;
+    for (const auto& S : mesh->subs) n = std::max(n, S.n);
+    return nd_fit<double2>(z, true, sub_krylov_bytes<double2>(sub_rows(n, C), m, 1), sub_keep_bytes(m), &mm) > 0;
+}
 
 bool build_tables(const thm_mesh* m, NdHost& H, const std::vector<int>& list, int p,
                   const std::vector<std::vector<NdMove>>* moves) {
@@ -486,7 +495,7 @@ bool build_tables(const thm_mesh* m, NdHost& H, const std::vector<int>& list, in
     }
     for (int i = 0; i < 64; ++i) H.idx.push_back(0);
     H.fac_elems = fo * 128 + 128;
-    if (!fits || smallest_smem(H.z) > ND_SMEM_MAX) return false;
+    if (!fits || !apply_fits(H.z)) return false;
     H.nodes.swap(nodes);
     H.rows.swap(rows);
     H.cmap.swap(cmap);
@@ -528,10 +537,16 @@ void build_nd(thm_mesh* m) {
     // many that a CTA has less than a warp pass of unknowns
     int p = 0;
     while (p < 3 && (int64_t)ns * (2 << p) <= 2 * (int64_t)sms && m->n_loc / ns >= (int64_t)(64 << (p + 1))) ++p;
+    // ... and more where a CTA's shared memory is too small for a solve of the
+    // default restart length (40x40 order-2 cells: 246 KB with one CTA, 131 KB
+    // with two, of 226)
+    int applies = -1;                                      // an apply fits, at least
     for (;; ++p) {
         m->nd_ok = build_tables(m, m->nd, all, p, nullptr);
-        if (m->nd_ok || p == 3) break;
+        if (m->nd_ok) applies = p;
+        if (p == 3 || (m->nd_ok && solve_fits(m, m->nd.z, 1 << p, ND_RESTART))) break;
     }
+    if (!m->nd_ok && applies >= 0) m->nd_ok = build_tables(m, m->nd, all, applies, nullptr);
     if (!m->nd_ok) return;                                 // reported by the first apply, as a size limit of the kernel
     auto& H = m->nd;
     auto& D = m->ndd;

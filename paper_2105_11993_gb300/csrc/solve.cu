@@ -492,7 +492,7 @@ SolveCfg make_cfg(const thm_solve_opts* o) {
     c.fp32 = o && o->mode == THM_MODE_MIXED;
     THM_REQUIRE(!o || o->mode == THM_MODE_FP64 || o->mode == THM_MODE_MIXED, "unknown mode");
     c.rtol = (o && o->rtol > 0) ? o->rtol : 1e-8;
-    c.m_in = (o && o->inner_restart > 0) ? o->inner_restart : 120;
+    c.m_in = (o && o->inner_restart > 0) ? o->inner_restart : ND_RESTART;
     c.m_out = (o && o->outer_restart > 0) ? o->outer_restart : 600;
     c.inner_maxit = (o && o->inner_maxit > 0) ? o->inner_maxit : 2000;
     c.outer_maxit = (o && o->outer_maxit > 0) ? o->outer_maxit : 2000;
@@ -541,11 +541,8 @@ static void apply_T(const thm_sys* s, const F* val, const F* bg, const F* bs, in
 
 // The block preconditioner of every subdomain: one cluster of nd.C CTAs each.
 // Two CTAs to an SM where their vectors fit (each hides the other's barriers
-// and L2 latency); vectors that outgrow shared memory leave the u buffers,
-// then the staged y, in a workspace of the system.
-// more: bytes that other phases of the kernel need in place of the vectors;
-// keep: bytes beside everything.  False: it does not fit (glob: with vectors
-// moved to the global workspace as need be).
+// and L2 latency); what outgrows shared memory (nd_fit) is in a workspace of
+// the system.  False: it does not fit.
 template <class V, class FW>
 static bool nd_memory(const thm_sys* s, bool glob, size_t more, size_t keep, NdMem* out, size_t* keep_off, size_t* smem) {
     const thm_mesh* m = s->m;
@@ -556,7 +553,6 @@ static bool nd_memory(const thm_sys* s, bool glob, size_t more, size_t keep, NdM
         s->bt_work.zero(s->st);
     }
     NdMem mm{};
-    mm.slt_smem = (size_t)z.nslt * sizeof(int2) <= 16 * 1024 ? 1 : 0;
     // L2 prefetch of the factor two levels ahead of its use where all factors
     // together are more than a small part of L2 (129 MB), which the bases of
     // the solves share: FP32 sweeps with 80 to 140 MB of factors 18.1 -> 17.0 ms
@@ -564,20 +560,11 @@ static bool nd_memory(const thm_sys* s, bool glob, size_t more, size_t keep, NdM
     // factors of a few MB are in L2 anyway, and asking costs 1% (4 squares of
     // 24^2, order 2: 641 -> 648 ms a solve).
     mm.prefetch = m->nd.fac_elems * (int64_t)sizeof(FW) >= (int64_t)16 << 20;
-    auto need = [&]() {
-        const NdLayout L = nd_layout<V>(z, mm.slt_smem, mm.u_glob, mm.y_glob);
-        return (std::max(L.total, L.vec + more) + 15) / 16 * 16 + keep;
-    };
-    if (glob) {
-        if (need() > ND_SMEM_MAX) mm.u_glob = 1;
-        if (need() > ND_SMEM_MAX) mm.y_glob = 1;
-    }
-    if ((!glob && !mm.slt_smem) || need() > ND_SMEM_MAX) return false;
-    mm.glob_stride = (mm.u_glob || mm.y_glob) ? nd_glob_layout(z).stride : 0;
+    *smem = nd_fit<V>(z, glob, more, keep, &mm);
+    if (*smem == 0) return false;
     const size_t entries = (size_t)(mm.glob_stride * m->n_sub * m->nd.C);
     if (s->nd_glob.n < entries) s->nd_glob.alloc(entries);
     *out = mm;
-    *smem = need();
     *keep_off = *smem - keep;
     return true;
 }
@@ -652,15 +639,16 @@ static void subsolve(thm_sys* s, const SolveCfg& c, SubWork<V>& k, const FW* fac
     NdMem mm{};
     // glob: u and w of the rows stay in global memory, like the apply's vectors
     // as need be.  A restart length whose scalars outgrow shared memory (about
-    // 1,000) is cut to what fits: such a cycle restarts there.
+    // 1,000; less where the vectors fill it) is cut to what fits: such a cycle
+    // restarts there.
     int mr = k.m;
     bool glob = false;
     while (true) {
         const size_t keep = sub_keep_bytes(mr);
         glob = !m->col16 || !nd_memory<V, FW>(s, false, sub_krylov_bytes<V>(rows, mr, 0), keep, &mm, &keep_off, &smem);
         if (!glob || nd_memory<V, FW>(s, true, sub_krylov_bytes<V>(rows, mr, 1), keep, &mm, &keep_off, &smem)) break;
-        THM_REQUIRE(mr > 128, "subdomain too large for the shared-memory block solve");
-        mr -= 64;
+        THM_REQUIRE(mr > 8, "subdomain too large for the shared-memory block solve");
+        mr -= 8;
     }
     SubArgs<V, F> a{};
     const bool f32 = sizeof(F) == 4;

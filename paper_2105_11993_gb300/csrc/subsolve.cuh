@@ -83,29 +83,6 @@ struct SubArgs {
     unsigned long long *kw, *kw64, *bt;     // work counters: SpMV rows, dot and update bytes; FP64 SpMV rows; applies
 };
 
-// Work items that a dot-product pass is cut into while there are few basis
-// vectors: three per warp, so that the last round is not nearly empty.
-constexpr int SUB_ITEMS = 3 * ND_NW;
-// Shared memory that outlives a step: rotations and g of the cycle (givens_core)
-// and the previous step's [b; d].
-__host__ __device__ inline size_t sub_keep_bytes(int m) { return (size_t)m * 40 + (size_t)(m + 1) * 48 + 48; }
-
-// Bytes of the Krylov phases' shared memory (they reuse the apply's): u and w
-// of the CTA's rows, the totals and the Hessenberg column, the coefficients,
-// the warps' sums.
-template <class V>
-__host__ __device__ inline size_t sub_krylov_bytes(int rows, int m, int k_glob) {
-    const size_t red = (size_t)(m / 4 + 2 + SUB_ITEMS) * 16 * sizeof(typename VT<V>::R);
-    return (k_glob ? 0 : 2 * (size_t)rows * sizeof(V)) + (size_t)(2 * m + 2) * 16 + (size_t)(m + 1) * 16 +
-           (size_t)(2 * m + 2) * sizeof(V) + (red + 15) / 16 * 16;
-}
-// rows of a CTA: the subdomain's local rows in C equal parts of whole warps
-// of the SELL slices, or of 8 where that would leave CTAs without rows
-__host__ __device__ inline int sub_rows(int64_t n, int C) {
-    const int64_t r = (n + C - 1) / C, g = r >= 512 ? 32 : 8;
-    return (int)((r + g - 1) / g * g);
-}
-
 // A sum with the rounding of its partial sums compensated (Kahan): FP32 sums
 // over a CTA's rows stay as accurate as sums over 8 rows.  FP64 sums plainly.
 template <class R> struct RowSum;
