@@ -832,7 +832,7 @@ static void check_device_error(thm_sys* s) {
     THM_CUDA(cudaStreamSynchronize(s->st));
     if (h) {
         THM_CUDA(cudaMemsetAsync(s->dev_err.p, 0, sizeof(int), s->st));
-        fail(THM_ETIMEOUT, "a bounded wait for a TMA copy in the block-preconditioner apply gave up");
+        fail(THM_ETIMEOUT, "a bounded wait for the table copies of a solve kernel gave up");
     }
 }
 
@@ -961,6 +961,7 @@ int sweep_diag(thm_sys* s, const thm_solve_opts* opts, int with_sources, const d
     RunStats rs;
     sweep(s, c, with_sources ? s->f_loc.p : nullptr, g_in, g_out, uloc, rs, with_sources ? s->uD.p : nullptr);
     collect(s, rs);
+    check_device_error(s);
     if (stats) {
         memset(stats, 0, sizeof(*stats));
         stats->sweeps = rs.sweeps;
