@@ -303,6 +303,22 @@ struct NdCta {
     bool ok;                  // the tables came
 };
 
+// One thread waits for the table copies, for at most wait_ns; then it gives up
+// (the CTA skips the work and keeps the barriers).  Copies under way write the
+// CTA's shared memory, so it does not leave before they are through, or as
+// long again.  (Out of line: the solve kernels have no registers to spare.)
+static __device__ __noinline__ void nd_wait(uint64_t* bar, unsigned long long wait_ns, int stall, int* s_abort, int* err) {
+    for (int round = 0; round < 2; ++round) {
+        const unsigned long long t0 = nd_now_ns();
+        do {
+            if (mbar_try(bar, 0)) return;
+        } while (nd_now_ns() - t0 <= wait_ns);
+        *s_abort = 1;
+        atomicExch(err, 1);
+        if (stall) return;                     // (none was sent)
+    }
+}
+
 // Start of a solve CTA: its level and slice tables come by TMA (stall:
 // failure-detection test, the copies never come).  GLOB: some of the tables
 // and vectors are in global memory; else all are in shared memory, which the
@@ -353,15 +369,7 @@ __device__ __forceinline__ void nd_enter(NdCta<V>& c, const NdTables& T, const N
             tma_load_1d(lev, T.levs + c.P.lev0, lb, bar);
             if (sb) tma_load_1d(smem + lay.slt, T.slt + c.P.slt0, sb, bar);
         }
-        if (!mbar_try(bar, 0)) {
-            const unsigned long long t0 = nd_now_ns();
-            while (!mbar_try(bar, 0))
-                if (nd_now_ns() - t0 > wait_ns) {          // bounded: give up, skip the work, keep the barriers
-                    *s_abort = 1;
-                    atomicExch(err, 1);
-                    break;
-                }
-        }
+        if (!mbar_try(bar, 0)) nd_wait(bar, wait_ns, stall, s_abort, err);
     }
     __syncthreads();
     c.ok = *s_abort == 0;
