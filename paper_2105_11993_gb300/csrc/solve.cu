@@ -266,13 +266,15 @@ struct Krylov {
             for (auto& e : ring_ev) THM_CUDA(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
         }
         // the kernels are shared by every instance: only ever raise their limit
+        // (coefficients and products of a step: 51 KB at the longest restart)
         const size_t dots_smem = 2 * (size_t)(m + 1) * sizeof(double2);
-        THM_REQUIRE((size_t)(m + 1) * KW * sizeof(double2) <= 200 * 1024, "restart length too large");
+        THM_REQUIRE(m < 1600, "restart length too large");
         static size_t dots_attr = 0;
         if (dots_smem > dots_attr) {
             THM_CUDA(cudaFuncSetAttribute(k_chunk_dots, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dots_smem));
             THM_CUDA(cudaFuncSetAttribute(k_update_givens, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dots_smem));
             THM_CUDA(cudaFuncSetAttribute(k_update_dots, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dots_smem));
+            THM_CUDA(cudaFuncSetAttribute(k_backsolve, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dots_smem));
             dots_attr = dots_smem;
         }
         THM_CUDA(cudaDeviceSynchronize());
