@@ -218,21 +218,13 @@ struct Krylov {
     double2* gmon = nullptr;
     int* h_pinned = nullptr;
     std::vector<int> h_kused;
-    // asynchronous convergence monitor: per Arnoldi step the monitor record
-    // lands in a pinned ring (one copy); the host reads it a few steps behind
-    // the GPU instead of blocking every step
-    static constexpr int RING = 4;
-    double2* h_ring = nullptr;       // [RING][2] copies of the monitor record
+    double2* h_mon = nullptr;        // [2] the record of the latest step, pinned
     double h_beta0 = 0;              // ||r_0|| of segment 0 at the first cycle
-    double last_rel = 1.0;           // latest residual estimate of segment 0 seen by the host, relative
-    bool fresh = false;              // wait for each step's record before the next step (the operator uses last_rel)
-    cudaEvent_t ring_ev[RING] = {};
+    double last_rel = 1.0;           // latest residual estimate of segment 0, relative
 
     ~Krylov() {
         if (h_pinned) cudaFreeHost(h_pinned);
-        if (h_ring) cudaFreeHost(h_ring);
-        for (auto& e : ring_ev)
-            if (e) cudaEventDestroy(e);
+        if (h_mon) cudaFreeHost(h_mon);
     }
 
     void init(int64_t n_, int nseg_, int m_, const std::vector<Chunk>& chunks) {
@@ -261,10 +253,7 @@ struct Krylov {
         flag = nact + 2;
         gmon = mon.p + 1;
         if (!h_pinned) THM_CUDA(cudaMallocHost(&h_pinned, 2 * sizeof(int)));
-        if (!h_ring) {
-            THM_CUDA(cudaMallocHost(&h_ring, 2 * RING * sizeof(double2)));
-            for (auto& e : ring_ev) THM_CUDA(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
-        }
+        if (!h_mon) THM_CUDA(cudaMallocHost(&h_mon, 2 * sizeof(double2)));
         // the kernels are shared by every instance: only ever raise their limit
         // (coefficients and products of a step: 51 KB at the longest restart)
         const size_t dots_smem = 2 * (size_t)(m + 1) * sizeof(double2);
@@ -317,32 +306,20 @@ struct Krylov {
             if (read_nact(st) == 0) break;
             if (total >= maxit) { ks.status = THM_ENOCONV; break; }
             THM_LAUNCH(THM_K_KRYLOV, st, k_chunk_scale<V><<<nch, 256, 0, st>>>(d_chunks.p, r.p, beta.p, basis.p, nullptr));
-            int j = 0, checked = 0;
-            // the monitor record of step jj is in the ring; true when the host
-            // has seen every segment stop or a breakdown (reads run a few
-            // steps behind the GPU and block only when the ring is full)
-            auto monitor = [&](int jj) -> bool {
-                const int slot = jj % RING;
-                THM_CUDA(cudaMemcpyAsync(h_ring + 2 * slot, mon.p, 2 * sizeof(double2), cudaMemcpyDeviceToHost, st));
-                THM_CUDA(cudaEventRecord(ring_ev[slot], st));
-                while (checked <= jj) {
-                    const int rs_ = checked % RING;
-                    cudaError_t q = (fresh || jj - checked >= RING - 1) ? cudaEventSynchronize(ring_ev[rs_])
-                                                                        : cudaEventQuery(ring_ev[rs_]);
-                    if (q == cudaErrorNotReady) break;
-                    THM_CUDA(q);
-                    const int* rec = reinterpret_cast<const int*>(h_ring + 2 * rs_);
-                    if (rec[2]) { ks.status = THM_EBREAKDOWN; return true; }
-                    if (nseg == 1 && h_beta0 > 0) {
-                        const double2 g1 = h_ring[2 * rs_ + 1];
-                        last_rel = std::hypot(g1.x, g1.y) / h_beta0;
-                    }
-                    if (rec[0] == 0) return true;
-                    ++checked;
-                }
-                return false;
+            // Waits for the record of the latest step; true when every segment has
+            // stopped, or on a breakdown.  A step goes out only after this: one
+            // beyond the last would run a whole sweep, on a basis vector that was
+            // not written, to be thrown away (with the host three steps ahead 3 of
+            // some 85 sweeps of a solve; the wait costs about 10 us a step).
+            auto stopped = [&]() -> bool {
+                THM_CUDA(cudaMemcpyAsync(h_mon, mon.p, 2 * sizeof(double2), cudaMemcpyDeviceToHost, st));
+                THM_CUDA(cudaStreamSynchronize(st));
+                const int* rec = reinterpret_cast<const int*>(h_mon);
+                if (rec[2]) { ks.status = THM_EBREAKDOWN; return true; }
+                if (nseg == 1 && h_beta0 > 0) last_rel = std::hypot(h_mon[1].x, h_mon[1].y) / h_beta0;
+                return rec[0] == 0;
             };
-            for (; j < m && total < maxit; ++j) {
+            for (int j = 0; j < m && total < maxit; ++j) {
                 V* vj = basis.p + (int64_t)j * n;
                 A(vj, w.p);
                 const int nk = j + 1;
@@ -362,13 +339,8 @@ struct Krylov {
                                                                                       active.p, ga, kw(1)));
                 THM_LAUNCH(THM_K_KRYLOV, st, k_chunk_scale<V><<<nch, 256, 0, st>>>(d_chunks.p, w.p, beta.p, basis.p + (int64_t)(j + 1) * n, active.p));
                 ++total;
-                // monitor: one copy of the step's record into the ring
-                if (monitor(j)) break;
+                if (stopped()) break;
             }
-            // drain the monitor: any later step may still report breakdown
-            THM_CUDA(cudaStreamSynchronize(st));
-            for (; checked < j && ks.status != THM_EBREAKDOWN; ++checked)
-                if (reinterpret_cast<const int*>(h_ring + 2 * (checked % RING))[2]) ks.status = THM_EBREAKDOWN;
             THM_CUDA(cudaGetLastError());
             // x += V y
             THM_LAUNCH(THM_K_KRYLOV, st, k_backsolve<<<nseg, 32, 2 * (size_t)m * sizeof(double2), st>>>(nseg, m, Rm.p, gv.p,
@@ -769,7 +741,6 @@ static void ddm_solve(thm_sys* s, const SolveCfg& c, const double2* src, double2
         sweep(s, cr, nullptr, v, w->gtmp.p, w->ytmp.p, rs);
         THM_LAUNCH(THM_K_KRYLOV, st, k_sub<double2><<<nblk(m->n_if), 256, 0, st>>>(m->n_if, v, w->gtmp.p, out));   // (I - A) v
     };
-    w->outer.fresh = c.relax != 0;
     static const bool verbose = getenv("THM_VERBOSE") != nullptr;
     std::function<void(const double2*, double2*)> Av = A;
     if (verbose) {
