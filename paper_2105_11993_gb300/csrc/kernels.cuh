@@ -157,14 +157,17 @@ __global__ void __launch_bounds__(KT) k_chunk_norm2(const Chunk* __restrict__ ch
 __global__ void k_seg_reduce_real(int nseg, const int32_t* __restrict__ seg_ch, const double* __restrict__ part,
                                   double* __restrict__ out);
 
-// scale: x[e] = (beta[seg] > 0) ? r[e] / beta[seg] : 0
+// scale: x[e] = (beta[seg] > 0) ? r[e] / beta[seg] : 0, and 0 in segments that are not active (act, or null)
 template <class V>
 __global__ void k_chunk_scale(const Chunk* __restrict__ chunks, const V* __restrict__ r,
                               const double* __restrict__ beta, V* __restrict__ x, const int* __restrict__ act) {
     using R = typename VT<V>::R;
     __shared__ R s_inv;
     const Chunk c = chunks[blockIdx.x];
-    if (act && !act[c.seg]) return;
+    if (act && !act[c.seg]) {                  // the operator runs over all segments
+        for (int64_t e = c.begin + threadIdx.x; e < c.end; e += blockDim.x) x[e] = mk<V>(0, 0);
+        return;
+    }
     if (threadIdx.x == 0) {                    // one FP64 division per block, not per thread
         const double b = beta[c.seg];
         s_inv = b > 0 ? (R)(1.0 / b) : (R)0;
