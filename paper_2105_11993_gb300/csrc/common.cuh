@@ -304,6 +304,7 @@ void require_nd(const thm_mesh* m);
 bool build_tables(const thm_mesh* m, NdHost& H, const std::vector<int>& list, int p,
                   const std::vector<std::vector<NdMove>>* moves);
 bool place_tables(NdHost& H, const NdPlace& at);
+NdSizes larger(NdSizes a, const NdSizes& b);
 NdTables nd_tables(const thm_sys* s, bool cplx);
 void assemble(thm_sys* s);
 void ensure_factor(thm_sys* s, bool fp32);

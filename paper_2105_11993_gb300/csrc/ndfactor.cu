@@ -426,7 +426,7 @@ static void append(DArr<X>& dst, const DArr<X>& base, const std::vector<X>& add,
     a.alloc(base.n + add.size() + more);
     if (base.n) THM_CUDA(cudaMemcpyAsync(a.p, base.p, base.n * sizeof(X), cudaMemcpyDeviceToDevice, st));
     if (!add.empty()) THM_CUDA(cudaMemcpyAsync(a.p + base.n, add.data(), add.size() * sizeof(X), cudaMemcpyHostToDevice, st));
-    THM_CUDA(cudaStreamSynchronize(st));
+    if (&dst == &base) THM_CUDA(cudaStreamSynchronize(st));      // its array goes now
     std::swap(dst.p, a.p);
     std::swap(dst.n, a.n);
 }
@@ -478,14 +478,10 @@ static bool move_up(const thm_sys* s, const NdHost& H, const std::vector<int2>& 
     o->d.rows.upload(out.rows, st);
     o->d.cmap.upload(out.cmap, st);
     o->d.childs.upload(out.childs, st);
-    o->z = s->nd_sizes(&own == &s->ownc);
-    o->z.nlev = std::max(o->z.nlev, out.z.nlev);
-    o->z.nslt = std::max(o->z.nslt, out.z.nslt);
-    o->z.nvec = std::max(o->z.nvec, out.z.nvec);
-    o->z.ny = std::max(o->z.ny, out.z.ny);
-    for (int k = 0; k < 2; ++k) o->z.nu[k] = std::max(o->z.nu[k], out.z.nu[k]);
+    o->z = larger(s->nd_sizes(&own == &s->ownc), out.z);
     o->fac_elems = fac0 + out.fac_elems;
     o->moves.swap(moves);
+    THM_CUDA(cudaStreamSynchronize(st));               // the copies are done with both
     own.swap(o);
     return true;
 }

@@ -1,8 +1,13 @@
 // Host build of the nested-dissection trees and their device tables (nd.cuh).
 #include <algorithm>
+#include <atomic>
 #include <cmath>
 #include <cstdlib>
+#include <exception>
+#include <functional>
+#include <mutex>
 #include <numeric>
+#include <system_error>
 #include <thread>
 
 #include "common.cuh"
@@ -33,6 +38,7 @@ struct Node {
     int vpos = 0, upos = 0;        // in the CTA's vector / the level's u buffer
     int row_f = 0, row_b = 0, slt_f = 0, slt_b = 0;
     int64_t id = 0;                // global node number
+    int64_t front = 0;             // its front's place in the depth's workspace
     double cost = 0;               // values under the node
 };
 
@@ -206,7 +212,302 @@ void build_tree(const thm_mesh* m, int s, std::vector<int32_t> cs, int p, const 
 
 int pad4(int v) { return (v + 3) / 4 * 4; }
 
+// Tables of one subdomain, positions within its own arrays; `nodes` in the tree's order, rows, cmap and
+// childs (node numbers) likewise.  False: an index outgrows its 16 bits.
+bool emit_tables(const thm_mesh* m, int sub, SubTree& T, int C, NdHost& H) {
+    const int mw = m->maxc / 2;
+    const auto& S = m->subs[sub];
+    H.C = C;
+    H.mw = mw;
+    H.welem.assign(1, 0);
+    H.nodes.resize(T.nodes.size());
+    int64_t fo = 0;                                    // factor offset, in 128 entries
+    bool fits = true;
+    std::vector<int32_t> place(S.n, -1);               // front index of a local row of the subdomain
+    size_t ss = 0, sb = 0;                             // all s, all b
+    for (auto& N : T.nodes) {
+        H.welem[0] += (int64_t)N.s.size() * (N.s.size() + 2 * N.b.size());
+        ss += N.s.size();
+        sb += N.b.size();
+    }
+    const size_t nrow = 2 * ss + sb + (size_t)64 * C * (T.maxdepth + 2);
+    H.rowd.reserve(nrow);
+    H.rowm.reserve(nrow * mw);
+    H.ymap.reserve((ss + 4 * T.nodes.size()) * mw);
+    H.idx.reserve(sb + 4 * T.nodes.size() + (size_t)C * (T.maxdepth + 2) * 256);
+    H.perm.reserve(ss + 4 * T.nodes.size() + (size_t)C * (T.nodes[0].s.size() + 8));
+    H.rows.reserve(ss + sb);
+    H.cmap.reserve(sb);
+    H.childs.reserve(T.nodes.size());
+    const Node& root = T.nodes[0];
+    const int sr = (int)root.s.size(), srp = pad4(sr);
+    std::vector<std::vector<uint32_t>> rmap(sr);
+    std::vector<int32_t> vrow(S.n, -1);                // vector entry of a local row in the CTA at hand
+    const int share = (sr + C - 1) / C;
+    for (int rk = 0; rk < C; ++rk) {
+        NdPart P{};
+        P.lev0 = (int32_t)H.levs.size();
+        P.slt0 = (int32_t)H.slt.size();
+        P.perm0 = (int64_t)H.perm.size();
+        P.sroot = sr;
+        P.rr0 = std::min(sr, rk * share);
+        P.nrr = std::min(sr, (rk + 1) * share) - P.rr0;
+        std::vector<std::vector<int>> lv(T.maxdepth + 1);
+        for (size_t q = 1; q < T.nodes.size(); ++q)
+            if (T.nodes[q].rank == rk) lv[T.nodes[q].depth].push_back((int)q);
+        int deepest = 0;
+        for (int d = 1; d <= T.maxdepth; ++d)
+            if (!lv[d].empty()) deepest = d;
+        P.nlev = deepest;
+        // vector: root, a zero entry, the levels deepest first
+        for (int i = 0; i < srp + 4; ++i) H.perm.push_back(i < sr ? root.s[i] : -1);
+        for (int i = 0; i < sr; ++i) vrow[root.s[i] - S.off] = i;
+        int vo = srp + 4;
+        const int zero = srp;
+        for (int d = deepest; d >= 1; --d) {
+            std::stable_sort(lv[d].begin(), lv[d].end(), [&](int a, int b) { return T.nodes[a].s.size() > T.nodes[b].s.size(); });
+            for (int q : lv[d]) {
+                Node& N = T.nodes[q];
+                N.vpos = vo;
+                for (size_t i = 0; i < N.s.size(); ++i) { vrow[N.s[i] - S.off] = vo + (int)i; H.perm.push_back(N.s[i]); }
+                vo += pad4((int)N.s.size());
+                while ((int64_t)H.perm.size() - P.perm0 < vo) H.perm.push_back(-1);
+            }
+        }
+        P.nvec = vo;
+        H.z.nvec = std::max(H.z.nvec, vo);
+        fits = fits && vo < (int)ND_U;
+        auto new_slice = [&](int nq) {
+            H.slt.push_back(make_int2((int)fo, nq));
+            fo += nq;
+            fits = fits && fo < (int64_t)INT32_MAX;
+        };
+        // slices over rows whose column quads are nqs; returns the number of slices
+        auto slices = [&](const std::vector<int>& nqs) {
+            int n = 0;
+            for (size_t i = 0; i < nqs.size(); i += 32, ++n)
+                new_slice(*std::max_element(nqs.begin() + i, nqs.begin() + std::min(nqs.size(), i + 32)));
+            return n;
+        };
+        auto share_cols = [&](int nsl, const std::vector<int>& nqs) {
+            if (nsl == 0 || nsl * 2 > ND_NW) return 1;
+            const int mq = *std::max_element(nqs.begin(), nqs.end());
+            return std::max(1, std::min(ND_NW / nsl, mq / 2));
+        };
+        auto pad_rows = [&](size_t words) {
+            while (H.rowd.size() % 32) {
+                H.rowd.push_back(ND_NOROW);
+                for (size_t w = 0; w < words; ++w) H.rowm.push_back(0xffffffffu);
+            }
+        };
+        // ---- up
+        for (int d = deepest; d >= 1; --d) {
+            NdLev L{};
+            L.depth = d;
+            int uo = 0;
+            for (int q : lv[d]) { T.nodes[q].upos = uo; uo += (int)T.nodes[q].b.size(); }
+            H.z.nu[d & 1] = std::max(H.z.nu[d & 1], uo);
+            fits = fits && uo < (int)ND_U;
+            L.v0 = lv[d].empty() ? vo : T.nodes[lv[d][0]].vpos;
+            int nv = 0;
+            for (int q : lv[d]) nv += pad4((int)T.nodes[q].s.size());
+            L.nv = nv;
+            L.ymap = (int32_t)(H.ymap.size() / mw);
+            L.rowf = (int32_t)H.rowd.size();
+            L.sltf = (int32_t)H.slt.size() - P.slt0;
+            std::vector<int> nqs;
+            for (int q : lv[d]) {
+                Node& N = T.nodes[q];
+                const int sn = (int)N.s.size(), bn = (int)N.b.size();
+                std::vector<uint32_t> map((size_t)(pad4(sn) + bn) * 2 * mw, ND_NONE);   // s part padded, then b
+                std::vector<int> cnt(pad4(sn) + bn, 0);
+                for (int i = 0; i < sn; ++i) place[N.s[i] - S.off] = i;
+                for (int i = 0; i < bn; ++i) place[N.b[i] - S.off] = pad4(sn) + i;
+                for (int c : N.ch) {
+                    const Node& K = T.nodes[c];
+                    for (size_t i = 0; i < K.b.size(); ++i) {
+                        const int at = place[K.b[i] - S.off];
+                        if (cnt[at] >= 2 * mw) fail(THM_EINVAL, "internal: too many subtrees share an unknown");
+                        map[(size_t)at * 2 * mw + cnt[at]++] = (uint32_t)(K.upos + i);
+                    }
+                }
+                auto words = [&](int at, std::vector<uint32_t>& to) {
+                    for (int w = 0; w < mw; ++w)
+                        to.push_back((map[(size_t)at * 2 * mw + 2 * w] & 0xffffu) | map[(size_t)at * 2 * mw + 2 * w + 1] << 16);
+                };
+                for (int i = 0; i < pad4(sn); ++i) words(i, H.ymap);
+                N.row_f = (int)H.rowd.size() - L.rowf;
+                N.slt_f = P.slt0 + L.sltf;
+                for (int i = 0; i < sn + bn; ++i) {
+                    const uint32_t dst = i < sn ? (uint32_t)(N.vpos + i) : (ND_U | (uint32_t)(N.upos + i - sn));
+                    H.rowd.push_back((uint32_t)(N.vpos - L.v0) | dst << 16);
+                    words(i < sn ? i : pad4(sn) + i - sn, H.rowm);
+                    nqs.push_back(pad4(sn) / 4);
+                }
+            }
+            pad_rows(mw);
+            L.nsf = slices(nqs);
+            L.ksf = share_cols(L.nsf, nqs);
+            int mq = 0;
+            for (int v : nqs) mq = std::max(mq, v);
+            H.z.ny = std::max(H.z.ny, nv + 4 * mq);
+            H.levs.push_back(L);
+        }
+        {   // the root's rows of this CTA
+            NdLev L{};
+            L.nv = sr;
+            L.rowf = (int32_t)H.rowd.size();
+            L.sltf = (int32_t)H.slt.size() - P.slt0;
+            std::vector<int> nqs(P.nrr, srp / 4);
+            for (int i = 0; i < P.nrr; ++i) {
+                H.rowd.push_back((uint32_t)(P.rr0 + i) << 16);
+                for (int w = 0; w < mw; ++w) H.rowm.push_back(0xffffffffu);
+            }
+            pad_rows(mw);
+            L.nsf = slices(nqs);
+            L.ksf = share_cols(L.nsf, nqs);
+            H.z.ny = std::max(H.z.ny, srp);
+            H.levs.push_back(L);
+            for (int c : root.ch)
+                if (T.nodes[c].rank == rk)
+                    for (size_t i = 0; i < T.nodes[c].b.size(); ++i) {
+                        const int at = vrow[T.nodes[c].b[i] - S.off];
+                        rmap[at].push_back((uint32_t)rk << 16 | (uint32_t)(T.nodes[c].upos + i));
+                    }
+        }
+        // ---- down, nearest the root first (the order the solve streams them in)
+        for (int d = 1; d <= deepest; ++d) {
+            NdLev& L = H.levs[P.lev0 + deepest - d];
+            std::vector<int> order = lv[d];
+            std::stable_sort(order.begin(), order.end(), [&](int a, int b) { return T.nodes[a].b.size() > T.nodes[b].b.size(); });
+            while (H.idx.size() % 4) H.idx.push_back((uint16_t)zero);
+            L.idx = (int32_t)H.idx.size();
+            L.rowb = (int32_t)H.rowd.size();
+            L.sltb = (int32_t)H.slt.size() - P.slt0;
+            std::vector<int> nqs;
+            for (int q : order) {
+                Node& N = T.nodes[q];
+                N.row_b = (int)H.rowd.size() - L.rowb;
+                N.slt_b = P.slt0 + L.sltb;
+                if (N.b.empty()) continue;
+                const size_t i0 = (H.idx.size() - (size_t)L.idx) / 4;
+                fits = fits && i0 < 0xffffu;
+                for (int32_t r : N.b) H.idx.push_back((uint16_t)vrow[r - S.off]);
+                while (H.idx.size() % 4) H.idx.push_back((uint16_t)zero);
+                for (size_t i = 0; i < N.s.size(); ++i) {
+                    H.rowd.push_back((uint32_t)i0 | (uint32_t)(N.vpos + i) << 16);
+                    for (int w = 0; w < mw; ++w) H.rowm.push_back(0xffffffffu);
+                    nqs.push_back(pad4((int)N.b.size()) / 4);
+                }
+            }
+            pad_rows(mw);
+            L.nsb = slices(nqs);
+            L.ksb = share_cols(L.nsb, nqs);
+            int mq = 0;
+            for (int v : nqs) mq = std::max(mq, v);
+            for (int i = 0; i < 4 * mq; ++i) H.idx.push_back((uint16_t)zero);   // narrower rows read on to their slice's width
+        }
+        P.nslt = (int32_t)H.slt.size() - P.slt0;
+        while (H.slt.size() % 2) H.slt.push_back(make_int2(0, 0));
+        H.z.nlev = std::max(H.z.nlev, P.nlev);
+        H.z.nslt = std::max(H.z.nslt, (P.nslt + 1) / 2 * 2);
+        H.parts.push_back(P);
+    }
+    // root: children's entries per unknown
+    const int32_t rm0 = (int32_t)(H.rmap.size() / (2 * mw));
+    for (int i = 0; i < sr; ++i) {
+        THM_REQUIRE((int)rmap[i].size() <= 2 * mw, "internal: too many subtrees share a root unknown");
+        for (int c = 0; c < 2 * mw; ++c) H.rmap.push_back(c < (int)rmap[i].size() ? rmap[i][c] : 0xffffffffu);
+    }
+    for (int rk = 0; rk < C; ++rk) H.parts[rk].rmap0 = rm0;
+    // the factorisation's view
+    for (size_t q = 0; q < T.nodes.size(); ++q) {
+        Node& N = T.nodes[q];
+        NdNode& D = H.nodes[q];
+        D.s = (int32_t)N.s.size();
+        D.b = (int32_t)N.b.size();
+        D.sub = sub;
+        D.slt_f = N.slt_f;
+        D.slt_b = N.slt_b;
+        D.row_f = N.row_f;
+        D.row_b = N.row_b;
+        D.root_rows = q == 0 ? std::max(1, share) : 0;
+        D.rows0 = (int64_t)H.rows.size();
+        H.rows.insert(H.rows.end(), N.s.begin(), N.s.end());
+        H.rows.insert(H.rows.end(), N.b.begin(), N.b.end());
+        D.front = N.front;
+        D.child0 = (int32_t)H.childs.size();
+        D.nchild = (int32_t)N.ch.size();
+        for (size_t i = 0; i < N.s.size(); ++i) place[N.s[i] - S.off] = (int32_t)i;
+        for (size_t i = 0; i < N.b.size(); ++i) place[N.b[i] - S.off] = (int32_t)(N.s.size() + i);
+        for (int c : N.ch) {
+            H.childs.push_back((int32_t)T.nodes[c].id);
+            H.nodes[c].cmap0 = (int64_t)H.cmap.size();
+            for (int32_t r : T.nodes[c].b) H.cmap.push_back(place[r - S.off]);
+        }
+    }
+    H.fac_elems = fo * 128;
+    return fits;
+}
+
+// fn(i) for i < n on several threads; the first exception comes back here.
+void parallel(int n, const std::function<void(int)>& fn) {
+    const int nt = std::max(1, std::min<int>({16, n, (int)std::thread::hardware_concurrency()}));
+    std::atomic<int> next{0};
+    std::mutex mu;
+    std::exception_ptr err;
+    auto work = [&]() {
+        try {
+            for (int i; (i = next++) < n;) fn(i);
+        } catch (...) {
+            std::lock_guard<std::mutex> g(mu);
+            if (!err) err = std::current_exception();
+        }
+    };
+    std::vector<std::thread> th;
+    th.reserve(nt);
+    try {
+        for (int t = 1; t < nt; ++t) th.emplace_back(work);
+    } catch (const std::system_error&) {               // no more threads: those there are do it
+    }
+    work();
+    for (auto& t : th) t.join();
+    if (err) std::rethrow_exception(err);
+}
+
 }  // namespace
+
+bool place_tables(NdHost& H, const NdPlace& at) {
+    const size_t most = INT32_MAX, mw = H.mw;
+    if (at.levs + H.levs.size() > most || at.slt + H.slt.size() > most || at.rowd + H.rowd.size() > most ||
+        at.idx + H.idx.size() > most || (at.fac + H.fac_elems) / 128 > most)
+        return false;
+    THM_REQUIRE(at.slt % 2 == 0 && at.idx % 4 == 0 && at.fac % 128 == 0, "internal: tables out of alignment");
+    for (NdPart& P : H.parts) {
+        P.lev0 += (int32_t)at.levs;
+        P.slt0 += (int32_t)at.slt;
+        P.rmap0 += (int32_t)(at.rmap / (2 * mw));
+        P.perm0 += (int64_t)at.perm;
+    }
+    for (NdLev& L : H.levs) {
+        L.rowf += (int32_t)at.rowd;
+        L.rowb += (int32_t)at.rowd;
+        L.ymap += (int32_t)(at.ymap / mw);
+        L.idx += (int32_t)at.idx;
+    }
+    for (int2& v : H.slt) v.x += (int)(at.fac / 128);
+    for (NdNode& N : H.nodes) { N.slt_f += (int32_t)at.slt; N.slt_b += (int32_t)at.slt; }
+    return true;
+}
+
+NdSizes larger(NdSizes a, const NdSizes& b) {
+    a.nlev = std::max(a.nlev, b.nlev);
+    a.nslt = std::max(a.nslt, b.nslt);
+    a.nvec = std::max(a.nvec, b.nvec);
+    a.ny = std::max(a.ny, b.ny);
+    for (int k = 0; k < 2; ++k) a.nu[k] = std::max(a.nu[k], b.nu[k]);
+    return a;
+}
 
 // Whether an apply, resp. a subdomain solve with m steps per cycle, fits shared
 // memory in FP64 (the larger of the two precisions).
@@ -235,17 +536,10 @@ bool build_tables(const thm_mesh* m, NdHost& H, const std::vector<int>& list, in
     H.C = C;
     H.mw = mw;
     std::vector<SubTree> trees(ns);
-    {
-        std::vector<int32_t> cell_bin(m->n_cell, -1);     // cells belong to one subdomain each: no sharing
-        const int nt = std::max(1, std::min<int>(8, std::min<int>(ns, (int)std::thread::hardware_concurrency())));
-        std::vector<std::thread> th;
-        for (int t = 0; t < nt; ++t)
-            th.emplace_back([&, t]() {
-                for (int i = t; i < ns; i += nt)
-                    build_tree(m, list[i], cells[i], p, moves ? &(*moves)[list[i]] : nullptr, cell_bin, trees[i]);
-            });
-        for (auto& t : th) t.join();
-    }
+    std::vector<int32_t> cell_bin(m->n_cell, -1);         // cells belong to one subdomain each: no sharing
+    parallel(ns, [&](int i) {
+        build_tree(m, list[i], std::move(cells[i]), p, moves ? &(*moves)[list[i]] : nullptr, cell_bin, trees[i]);
+    });
     // node numbers: by depth, deepest first
     int maxd = 0;
     for (const auto& T : trees) maxd = std::max(maxd, T.maxdepth);
@@ -262,6 +556,7 @@ bool build_tables(const thm_mesh* m, NdHost& H, const std::vector<int>& list, in
             N.id = id++;
             H.node_ref.push_back({list[e.first], e.second, N.parent});
             const int64_t n = (int64_t)(N.s.size() + N.b.size());
+            N.front = front;
             front += n * n;
             ms = std::max(ms, (int)N.s.size());
             mn = std::max(mn, (int)n);
@@ -271,259 +566,62 @@ bool build_tables(const thm_mesh* m, NdHost& H, const std::vector<int>& list, in
         H.depth_s.push_back(ms);
         H.depth_n.push_back(mn);
     }
-    std::vector<NdNode> nodes(id);
-    std::vector<int32_t> rows, cmap, childs;
-    std::vector<int64_t> fsum(maxd + 1, 0);
-    int64_t fo = 0;                                        // factor offset, in 128 entries
-    H.welem.assign(ns, 0);
+    // the subdomains' tables, then one behind the other
+    std::vector<NdHost> part(ns);
+    std::vector<char> ok(ns, 0);
+    parallel(ns, [&](int i) { ok[i] = emit_tables(m, list[i], trees[i], C, part[i]); });
+    std::vector<NdPlace> at(ns + 1);
+    std::vector<size_t> rows0(ns + 1, 0), cmap0(ns + 1, 0), child0(ns + 1, 0);
     bool fits = true;
-    std::vector<int32_t> place;                            // front index of a local row of the subdomain
-    for (int s = 0; s < ns; ++s) {
-        SubTree& T = trees[s];
-        const auto& S = m->subs[list[s]];
-        place.assign(S.n, -1);
-        for (auto& N : T.nodes) H.welem[s] += (int64_t)N.s.size() * (N.s.size() + 2 * N.b.size());
-        const Node& root = T.nodes[0];
-        const int sr = (int)root.s.size(), srp = pad4(sr);
-        std::vector<std::vector<uint32_t>> rmap(sr);
-        std::vector<int32_t> vrow(S.n, -1);                // vector entry of a local row in the CTA at hand
-        const int share = (sr + C - 1) / C;
-        for (int rk = 0; rk < C; ++rk) {
-            NdPart P{};
-            P.lev0 = (int32_t)H.levs.size();
-            P.slt0 = (int32_t)H.slt.size();
-            P.perm0 = (int64_t)H.perm.size();
-            P.sroot = sr;
-            P.rr0 = std::min(sr, rk * share);
-            P.nrr = std::min(sr, (rk + 1) * share) - P.rr0;
-            std::vector<std::vector<int>> lv(T.maxdepth + 1);
-            for (size_t q = 1; q < T.nodes.size(); ++q)
-                if (T.nodes[q].rank == rk) lv[T.nodes[q].depth].push_back((int)q);
-            int deepest = 0;
-            for (int d = 1; d <= T.maxdepth; ++d)
-                if (!lv[d].empty()) deepest = d;
-            P.nlev = deepest;
-            // vector: root, a zero entry, the levels deepest first
-            for (int i = 0; i < srp + 4; ++i) H.perm.push_back(i < sr ? root.s[i] : -1);
-            for (int i = 0; i < sr; ++i) vrow[root.s[i] - S.off] = i;
-            int vo = srp + 4;
-            const int zero = srp;
-            for (int d = deepest; d >= 1; --d) {
-                std::stable_sort(lv[d].begin(), lv[d].end(), [&](int a, int b) { return T.nodes[a].s.size() > T.nodes[b].s.size(); });
-                for (int q : lv[d]) {
-                    Node& N = T.nodes[q];
-                    N.vpos = vo;
-                    for (size_t i = 0; i < N.s.size(); ++i) { vrow[N.s[i] - S.off] = vo + (int)i; H.perm.push_back(N.s[i]); }
-                    vo += pad4((int)N.s.size());
-                    while ((int64_t)H.perm.size() - P.perm0 < vo) H.perm.push_back(-1);
-                }
-            }
-            P.nvec = vo;
-            H.z.nvec = std::max(H.z.nvec, vo);
-            fits = fits && vo < (int)ND_U;
-            auto new_slice = [&](int nq) {
-                H.slt.push_back(make_int2((int)fo, nq));
-                fo += nq;
-                fits = fits && fo < (int64_t)INT32_MAX;
-            };
-            // slices over rows whose column quads are nqs; returns the number of slices
-            auto slices = [&](const std::vector<int>& nqs) {
-                int n = 0;
-                for (size_t i = 0; i < nqs.size(); i += 32, ++n)
-                    new_slice(*std::max_element(nqs.begin() + i, nqs.begin() + std::min(nqs.size(), i + 32)));
-                return n;
-            };
-            auto share_cols = [&](int nsl, const std::vector<int>& nqs) {
-                if (nsl == 0 || nsl * 2 > ND_NW) return 1;
-                const int mq = *std::max_element(nqs.begin(), nqs.end());
-                return std::max(1, std::min(ND_NW / nsl, mq / 2));
-            };
-            auto pad_rows = [&](size_t words) {
-                while (H.rowd.size() % 32) {
-                    H.rowd.push_back(ND_NOROW);
-                    for (size_t w = 0; w < words; ++w) H.rowm.push_back(0xffffffffu);
-                }
-            };
-            // ---- up
-            for (int d = deepest; d >= 1; --d) {
-                NdLev L{};
-                L.depth = d;
-                int uo = 0;
-                for (int q : lv[d]) { T.nodes[q].upos = uo; uo += (int)T.nodes[q].b.size(); }
-                H.z.nu[d & 1] = std::max(H.z.nu[d & 1], uo);
-                fits = fits && uo < (int)ND_U;
-                L.v0 = lv[d].empty() ? vo : T.nodes[lv[d][0]].vpos;
-                int nv = 0;
-                for (int q : lv[d]) nv += pad4((int)T.nodes[q].s.size());
-                L.nv = nv;
-                L.ymap = (int32_t)(H.ymap.size() / mw);
-                L.rowf = (int32_t)H.rowd.size();
-                L.sltf = (int32_t)H.slt.size() - P.slt0;
-                std::vector<int> nqs;
-                for (int q : lv[d]) {
-                    Node& N = T.nodes[q];
-                    const int sn = (int)N.s.size(), bn = (int)N.b.size();
-                    std::vector<uint32_t> map((size_t)(pad4(sn) + bn) * 2 * mw, ND_NONE);   // s part padded, then b
-                    std::vector<int> cnt(pad4(sn) + bn, 0);
-                    for (int i = 0; i < sn; ++i) place[N.s[i] - S.off] = i;
-                    for (int i = 0; i < bn; ++i) place[N.b[i] - S.off] = pad4(sn) + i;
-                    for (int c : N.ch) {
-                        const Node& K = T.nodes[c];
-                        for (size_t i = 0; i < K.b.size(); ++i) {
-                            const int at = place[K.b[i] - S.off];
-                            if (cnt[at] >= 2 * mw) fail(THM_EINVAL, "internal: too many subtrees share an unknown");
-                            map[(size_t)at * 2 * mw + cnt[at]++] = (uint32_t)(K.upos + i);
-                        }
-                    }
-                    auto words = [&](int at, std::vector<uint32_t>& to) {
-                        for (int w = 0; w < mw; ++w)
-                            to.push_back((map[(size_t)at * 2 * mw + 2 * w] & 0xffffu) | map[(size_t)at * 2 * mw + 2 * w + 1] << 16);
-                    };
-                    for (int i = 0; i < pad4(sn); ++i) words(i, H.ymap);
-                    N.row_f = (int)H.rowd.size() - L.rowf;
-                    N.slt_f = P.slt0 + L.sltf;
-                    for (int i = 0; i < sn + bn; ++i) {
-                        const uint32_t dst = i < sn ? (uint32_t)(N.vpos + i) : (ND_U | (uint32_t)(N.upos + i - sn));
-                        H.rowd.push_back((uint32_t)(N.vpos - L.v0) | dst << 16);
-                        words(i < sn ? i : pad4(sn) + i - sn, H.rowm);
-                        nqs.push_back(pad4(sn) / 4);
-                    }
-                }
-                pad_rows(mw);
-                L.nsf = slices(nqs);
-                L.ksf = share_cols(L.nsf, nqs);
-                int mq = 0;
-                for (int v : nqs) mq = std::max(mq, v);
-                H.z.ny = std::max(H.z.ny, nv + 4 * mq);
-                H.levs.push_back(L);
-            }
-            {   // the root's rows of this CTA
-                NdLev L{};
-                L.nv = sr;
-                L.rowf = (int32_t)H.rowd.size();
-                L.sltf = (int32_t)H.slt.size() - P.slt0;
-                std::vector<int> nqs(P.nrr, srp / 4);
-                for (int i = 0; i < P.nrr; ++i) {
-                    H.rowd.push_back((uint32_t)(P.rr0 + i) << 16);
-                    for (int w = 0; w < mw; ++w) H.rowm.push_back(0xffffffffu);
-                }
-                pad_rows(mw);
-                L.nsf = slices(nqs);
-                L.ksf = share_cols(L.nsf, nqs);
-                H.z.ny = std::max(H.z.ny, srp);
-                H.levs.push_back(L);
-                for (int c : root.ch)
-                    if (T.nodes[c].rank == rk)
-                        for (size_t i = 0; i < T.nodes[c].b.size(); ++i) {
-                            const int at = vrow[T.nodes[c].b[i] - S.off];
-                            rmap[at].push_back((uint32_t)rk << 16 | (uint32_t)(T.nodes[c].upos + i));
-                        }
-            }
-            // ---- down, nearest the root first (the order the solve streams them in)
-            for (int d = 1; d <= deepest; ++d) {
-                NdLev& L = H.levs[P.lev0 + deepest - d];
-                std::vector<int> order = lv[d];
-                std::stable_sort(order.begin(), order.end(), [&](int a, int b) { return T.nodes[a].b.size() > T.nodes[b].b.size(); });
-                while (H.idx.size() % 4) H.idx.push_back((uint16_t)zero);
-                L.idx = (int32_t)H.idx.size();
-                L.rowb = (int32_t)H.rowd.size();
-                L.sltb = (int32_t)H.slt.size() - P.slt0;
-                std::vector<int> nqs;
-                for (int q : order) {
-                    Node& N = T.nodes[q];
-                    N.row_b = (int)H.rowd.size() - L.rowb;
-                    N.slt_b = P.slt0 + L.sltb;
-                    if (N.b.empty()) continue;
-                    const size_t i0 = (H.idx.size() - (size_t)L.idx) / 4;
-                    fits = fits && i0 < 0xffffu;
-                    for (int32_t r : N.b) H.idx.push_back((uint16_t)vrow[r - S.off]);
-                    while (H.idx.size() % 4) H.idx.push_back((uint16_t)zero);
-                    for (size_t i = 0; i < N.s.size(); ++i) {
-                        H.rowd.push_back((uint32_t)i0 | (uint32_t)(N.vpos + i) << 16);
-                        for (int w = 0; w < mw; ++w) H.rowm.push_back(0xffffffffu);
-                        nqs.push_back(pad4((int)N.b.size()) / 4);
-                    }
-                }
-                pad_rows(mw);
-                L.nsb = slices(nqs);
-                L.ksb = share_cols(L.nsb, nqs);
-                int mq = 0;
-                for (int v : nqs) mq = std::max(mq, v);
-                for (int i = 0; i < 4 * mq; ++i) H.idx.push_back((uint16_t)zero);   // narrower rows read on to their slice's width
-            }
-            P.nslt = (int32_t)H.slt.size() - P.slt0;
-            while (H.slt.size() % 2) H.slt.push_back(make_int2(0, 0));
-            H.z.nlev = std::max(H.z.nlev, P.nlev);
-            H.z.nslt = std::max(H.z.nslt, (P.nslt + 1) / 2 * 2);
-            H.parts.push_back(P);
-        }
-        // root: children's entries per unknown
-        const int32_t rm0 = (int32_t)(H.rmap.size() / (2 * mw));
-        for (int i = 0; i < sr; ++i) {
-            THM_REQUIRE((int)rmap[i].size() <= 2 * mw, "internal: too many subtrees share a root unknown");
-            for (int c = 0; c < 2 * mw; ++c) H.rmap.push_back(c < (int)rmap[i].size() ? rmap[i][c] : 0xffffffffu);
-        }
-        for (int rk = 0; rk < C; ++rk) H.parts[(size_t)s * C + rk].rmap0 = rm0;
-        // the factorisation's view
-        for (size_t q = 0; q < T.nodes.size(); ++q) {
-            Node& N = T.nodes[q];
-            NdNode& D = nodes[N.id];
-            D.s = (int32_t)N.s.size();
-            D.b = (int32_t)N.b.size();
-            D.sub = list[s];
-            D.slt_f = N.slt_f;
-            D.slt_b = N.slt_b;
-            D.row_f = N.row_f;
-            D.row_b = N.row_b;
-            D.root_rows = q == 0 ? std::max(1, share) : 0;
-            D.rows0 = (int64_t)rows.size();
-            rows.insert(rows.end(), N.s.begin(), N.s.end());
-            rows.insert(rows.end(), N.b.begin(), N.b.end());
-            const int64_t n = (int64_t)(N.s.size() + N.b.size());
-            D.front = fsum[N.depth];
-            fsum[N.depth] += n * n;
-            D.child0 = (int32_t)childs.size();
-            D.nchild = (int32_t)N.ch.size();
-            for (size_t i = 0; i < N.s.size(); ++i) place[N.s[i] - S.off] = (int32_t)i;
-            for (size_t i = 0; i < N.b.size(); ++i) place[N.b[i] - S.off] = (int32_t)(N.s.size() + i);
-            for (int c : N.ch) {
-                childs.push_back((int32_t)T.nodes[c].id);
-                nodes[T.nodes[c].id].cmap0 = (int64_t)cmap.size();
-                for (int32_t r : T.nodes[c].b) cmap.push_back(place[r - S.off]);
-            }
-        }
+    NdPlace end{};
+    for (int i = 0; i < ns; ++i) {
+        const NdHost& P = part[i];
+        at[i] = end;
+        end = NdPlace{end.levs + P.levs.size(), end.slt + P.slt.size(), end.rowd + P.rowd.size(), end.ymap + P.ymap.size(),
+                      end.rmap + P.rmap.size(), end.idx + P.idx.size(), end.perm + P.perm.size(), end.fac + P.fac_elems};
+        rows0[i + 1] = rows0[i] + P.rows.size();
+        cmap0[i + 1] = cmap0[i] + P.cmap.size();
+        child0[i + 1] = child0[i] + P.childs.size();
+        H.z = larger(H.z, P.z);
+        fits = fits && ok[i];
     }
-    for (int i = 0; i < 64; ++i) H.idx.push_back(0);
-    H.fac_elems = fo * 128 + 128;
-    if (!fits || !apply_fits(H.z)) return false;
-    H.nodes.swap(nodes);
-    H.rows.swap(rows);
-    H.cmap.swap(cmap);
-    H.childs.swap(childs);
-    return true;
-}
-
-bool place_tables(NdHost& H, const NdPlace& at) {
-    const size_t most = INT32_MAX, mw = H.mw;
-    if (at.levs + H.levs.size() > most || at.slt + H.slt.size() > most || at.rowd + H.rowd.size() > most ||
-        at.idx + H.idx.size() > most || (at.fac + H.fac_elems) / 128 > most)
-        return false;
-    THM_REQUIRE(at.slt % 2 == 0 && at.idx % 4 == 0 && at.fac % 128 == 0, "internal: tables out of alignment");
-    for (NdPart& P : H.parts) {
-        P.lev0 += (int32_t)at.levs;
-        P.slt0 += (int32_t)at.slt;
-        P.rmap0 += (int32_t)(at.rmap / (2 * mw));
-        P.perm0 += (int64_t)at.perm;
-    }
-    for (NdLev& L : H.levs) {
-        L.rowf += (int32_t)at.rowd;
-        L.rowb += (int32_t)at.rowd;
-        L.ymap += (int32_t)(at.ymap / mw);
-        L.idx += (int32_t)at.idx;
-    }
-    for (int2& v : H.slt) v.x += (int)(at.fac / 128);
-    for (NdNode& N : H.nodes) { N.slt_f += (int32_t)at.slt; N.slt_b += (int32_t)at.slt; }
-    return true;
+    if (!fits || child0[ns] > INT32_MAX || !apply_fits(H.z)) return false;
+    H.parts.resize((size_t)ns * C);
+    H.welem.resize(ns);
+    H.levs.resize(end.levs); H.slt.resize(end.slt);
+    H.rowd.resize(end.rowd); H.rowm.resize(end.rowd * mw);
+    H.ymap.resize(end.ymap); H.rmap.resize(end.rmap); H.perm.resize(end.perm);
+    H.idx.assign(end.idx + 64, 0);                     // (a lane reads whole quads)
+    H.nodes.resize(id);
+    H.rows.resize(rows0[ns]); H.cmap.resize(cmap0[ns]); H.childs.resize(child0[ns]);
+    H.fac_elems = (int64_t)end.fac + 128;
+    parallel(ns, [&](int i) {
+        NdHost& P = part[i];
+        ok[i] = place_tables(P, at[i]);
+        std::copy(P.parts.begin(), P.parts.end(), H.parts.begin() + (size_t)i * C);
+        H.welem[i] = P.welem[0];
+        std::copy(P.levs.begin(), P.levs.end(), H.levs.begin() + at[i].levs);
+        std::copy(P.slt.begin(), P.slt.end(), H.slt.begin() + at[i].slt);
+        std::copy(P.rowd.begin(), P.rowd.end(), H.rowd.begin() + at[i].rowd);
+        std::copy(P.rowm.begin(), P.rowm.end(), H.rowm.begin() + at[i].rowd * mw);
+        std::copy(P.ymap.begin(), P.ymap.end(), H.ymap.begin() + at[i].ymap);
+        std::copy(P.rmap.begin(), P.rmap.end(), H.rmap.begin() + at[i].rmap);
+        std::copy(P.idx.begin(), P.idx.end(), H.idx.begin() + at[i].idx);
+        std::copy(P.perm.begin(), P.perm.end(), H.perm.begin() + at[i].perm);
+        std::copy(P.rows.begin(), P.rows.end(), H.rows.begin() + rows0[i]);
+        std::copy(P.cmap.begin(), P.cmap.end(), H.cmap.begin() + cmap0[i]);
+        std::copy(P.childs.begin(), P.childs.end(), H.childs.begin() + child0[i]);
+        for (size_t q = 0; q < P.nodes.size(); ++q) {
+            NdNode N = P.nodes[q];
+            N.rows0 += (int64_t)rows0[i];
+            N.cmap0 += (int64_t)cmap0[i];
+            N.child0 += (int32_t)child0[i];
+            H.nodes[trees[i].nodes[q].id] = N;
+        }
+        P = NdHost();
+    });
+    for (char o : ok) fits = fits && o;
+    return fits;
 }
 
 void build_nd(thm_mesh* m) {
