@@ -158,11 +158,13 @@ __device__ __forceinline__ double nd_block_max(double v, double* red) {
 // Entries of H above this move unknowns to the parent.
 constexpr double ND_GROWTH = 100;
 
-// What a factorisation reports: status[0] a non-finite pivot, [1] a zero pivot,
-// [2] the number of moves {node, local row} (at most one per local row).
+// What a factorisation reports: status[0] a non-finite pivot, [1] the number of
+// entries of moves: {node, local row} (at most one per local row) for an
+// unknown that moves up, {node, -1} for a node with a zero pivot.
 struct NdReport {
     int* status;
     int2* moves;
+    __device__ void add(int node, int row) const { moves[atomicAdd(&status[1], 1)] = make_int2(node, row); }
 };
 
 // The unknowns of a node that must not be eliminated there.  G = [W | H], s x
@@ -202,7 +204,7 @@ __device__ __noinline__ void nd_pick(T* G, int s, int b, int ld, T* col, int* go
             if (s_idx[w] >= 0 && (d < 0 || s_val[w] > best || (s_val[w] == best && s_idx[w] < d))) { best = s_val[w]; d = s_idx[w]; }
         if (d < 0 || !(best > 0)) {            // (not reached from finite entries but for a zero diagonal) all of them go
             for (int i = tid; i < s; i += nt)
-                if (!gone[i]) rep.moves[atomicAdd(&rep.status[2], 1)] = make_int2(node, rows[i]);
+                if (!gone[i]) rep.add(node, rows[i]);
             return;
         }
         const T id = A::inv(G[(int64_t)d * ld + d]);
@@ -210,7 +212,7 @@ __device__ __noinline__ void nd_pick(T* G, int s, int b, int ld, T* col, int* go
         __syncthreads();
         if (tid == 0) {
             gone[d] = 1;
-            rep.moves[atomicAdd(&rep.status[2], 1)] = make_int2(node, rows[d]);
+            rep.add(node, rows[d]);
         }
         __syncthreads();
         double hm = 0;
@@ -333,11 +335,11 @@ __global__ void k_nd_factor(NdTables tab, const NdNode* __restrict__ nodes, int6
     }
     __syncthreads();
     if (const int bad = nd_invert(W, s, ld, perm, fcol, frow)) {
-        if (tid == 0) atomicExch(&rep.status[bad == 2 ? 0 : 1], 1);
-        if (bad == 1 && b > 0) {                       // exactly singular: all of it moves up
-            for (int i = tid; i < s; i += nt)
-                rep.moves[atomicAdd(&rep.status[2], 1)] = make_int2((int)(node0 + blockIdx.x), rs[i]);
-        }
+        const int node = (int)(node0 + blockIdx.x);
+        if (tid == 0 && bad == 2) atomicExch(&rep.status[0], 1);
+        if (tid == 0 && bad == 1) rep.add(node, -1);
+        if (bad == 1 && b > 0)                         // exactly singular: all of it moves up
+            for (int i = tid; i < s; i += nt) rep.add(node, rs[i]);
         return;
     }
     // One Newton step, W += W (I - S W): Gauss-Jordan leaves an error of
@@ -431,18 +433,32 @@ static void append(DArr<X>& dst, const DArr<X>& base, const std::vector<X>& add,
     std::swap(dst.n, a.n);
 }
 
+// A subdomain whose moves make its factor this many times larger keeps the one
+// it has: moves are for a few unknowns of a few nodes (1.0005 times the values
+// at most on the inputs above, 1.06 on uniform media), and coefficients or
+// cells that show large H everywhere would fill the tree up to one dense block.
+constexpr double ND_FILL = 2;
+constexpr int ND_PASSES = 12;               // (2 or 3 are the rule)
+
 // Builds the trees of the subdomains of `found` again with these unknowns of
 // nodes of H in the parents, and puts their tables behind the present ones
-// (own: null while these are the mesh's).  False, and nothing changed: they
-// outgrow the solve kernel.
-static bool move_up(const thm_sys* s, const NdHost& H, const std::vector<int2>& found, std::unique_ptr<NdOwn>& own, NdHost& out) {
+// (own: null while these are the mesh's).  False, and no tables changed: there
+// is nothing left to move, or the tables outgrow the solve kernel.
+// kept [n_sub]: subdomains that are left as they are, more of which are found
+// here; singular: a zero pivot is in one of these.
+static bool move_up(const thm_sys* s, const NdHost& H, const std::vector<int2>& found, std::vector<char>& kept, bool& singular,
+                    std::unique_ptr<NdOwn>& own, NdHost& out) {
     const thm_mesh* m = s->m;
     cudaStream_t st = s->st;
     const int C = m->nd.C;
-    auto moves = own ? own->moves : std::vector<std::vector<NdMove>>(m->n_sub);
+    const auto before = own ? own->moves : std::vector<std::vector<NdMove>>(m->n_sub);
+    auto moves = before;
+    std::vector<char> zero(m->n_sub, 0);
     std::vector<int> list;
     for (const int2& f : found) {
         const NdRef& r = H.node_ref[f.x];
+        if (f.y < 0) zero[r.sub] = 1;
+        if (f.y < 0 || kept[r.sub]) continue;
         auto& v = moves[r.sub];
         auto it = std::lower_bound(v.begin(), v.end(), f.y, [](const NdMove& a, int row) { return a.row < row; });
         if (it != v.end() && it->row == f.y) it->node = r.parent;
@@ -453,10 +469,31 @@ static bool move_up(const thm_sys* s, const NdHost& H, const std::vector<int2>& 
     list.erase(std::unique(list.begin(), list.end()), list.end());
     int p = 0;
     while ((1 << p) < C) ++p;
-    if (!build_tables(m, out, list, p, &moves)) return false;
+    while (true) {
+        const bool ok = !list.empty() && build_tables(m, out, list, p, &moves);
+        // those that stay within ND_FILL, or (tables too large) all but the one with the most moves
+        auto most = std::max_element(list.begin(), list.end(), [&](int a, int b) { return moves[a].size() < moves[b].size(); });
+        std::vector<int> fit;
+        for (size_t i = 0; i < list.size(); ++i)
+            if (ok ? out.welem[i] <= ND_FILL * m->nd.welem[list[i]] : list[i] != *most) fit.push_back(list[i]);
+        if (ok && fit.size() == list.size()) break;
+        for (int q : list)
+            if (!std::binary_search(fit.begin(), fit.end(), q)) {
+                kept[q] = 1;
+                moves[q] = before[q];
+            }
+        list.swap(fit);
+        if (list.empty()) break;
+    }
+    for (int q = 0; q < m->n_sub; ++q)
+        singular = singular || (zero[q] && !std::binary_search(list.begin(), list.end(), q));
+    if (list.empty()) return false;
     const NdDev& B = own ? own->d : m->ndd;
     const int64_t fac0 = own ? own->fac_elems : m->nd.fac_elems;
-    if (!place_tables(out, NdPlace{B.levs.n, B.slt.n, B.rowd.n, B.ymap.n, B.rmap.n, B.idx.n, B.perm.n, (size_t)fac0})) return false;
+    if (!place_tables(out, NdPlace{B.levs.n, B.slt.n, B.rowd.n, B.ymap.n, B.rmap.n, B.idx.n, B.perm.n, (size_t)fac0})) {
+        singular = std::any_of(zero.begin(), zero.end(), [](char z) { return z != 0; });
+        return false;
+    }
     std::unique_ptr<NdOwn> o(new NdOwn());
     append(o->d.levs, B.levs, out.levs, st);
     append(o->d.slt, B.slt, out.slt, st);
@@ -498,13 +535,15 @@ static void factor(thm_sys* s, DArr<T>& fac, const char* what) {
     fac.zero(st);
     DArr<T> front[2], aux;
     DArr<int> status;
-    status.alloc(3);
+    status.alloc(2);
     DArr<int2> moves;
-    moves.alloc(m->n_loc);
+    moves.alloc(m->n_loc + m->nd.nodes.size());
+    std::vector<char> kept(m->n_sub, 0);
     THM_CUDA(cudaFuncSetAttribute(k_nd_factor<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, 225 * 1024));
     const size_t cap = 200 * 1024;
     NdHost again;                                      // the subdomains that are factorised again
-    for (bool first = true;; first = false) {
+    for (int passes = 0;; ++passes) {
+        const bool first = passes == 0;
         const NdHost& H = first ? m->nd : again;
         const NdDev& D = first ? m->ndd : own->d;
         int64_t most[2] = {0, 0};
@@ -530,17 +569,18 @@ static void factor(thm_sys* s, DArr<T>& fac, const char* what) {
         }
         std::vector<int> hs;
         status.download(hs, st);
-        if (hs[0] != 0 || (hs[1] != 0 && hs[2] == 0)) fail(THM_ESINGULAR, what);
-        if (hs[2] == 0) break;
-        std::vector<int2> found(hs[2]);
+        if (hs[0] != 0) fail(THM_ESINGULAR, what);
+        if (hs[1] == 0) break;
+        std::vector<int2> found(hs[1]);
         THM_CUDA(cudaMemcpyAsync(found.data(), moves.p, found.size() * sizeof(int2), cudaMemcpyDeviceToHost, st));
         THM_CUDA(cudaStreamSynchronize(st));
         std::sort(found.begin(), found.end(), [](const int2& a, const int2& b) { return a.x != b.x ? a.x < b.x : a.y < b.y; });
         NdHost next;
-        if (!move_up(s, H, found, own, next)) {        // trees too large for the solve kernel: the factors as they are
-            if (hs[1] != 0) fail(THM_ESINGULAR, what);
-            break;
-        }
+        if (passes == ND_PASSES) kept.assign(m->n_sub, 1);
+        bool singular = false;
+        const bool moved = move_up(s, H, found, kept, singular, own, next);
+        if (singular) fail(THM_ESINGULAR, what);
+        if (!moved) break;
         std::swap(again, next);
         const size_t n0 = fac.n;
         append(fac, fac, std::vector<T>(), st, again.fac_elems);
