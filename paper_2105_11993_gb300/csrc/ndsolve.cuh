@@ -268,10 +268,10 @@ __host__ __device__ inline int sub_rows(int64_t n, int C) {
 // build of the trees, which picks the CTAs per subdomain by it, and for the
 // launches.  more: bytes that other phases need over the apply's vectors;
 // keep: bytes beside everything.  glob: the u buffers, then the staged y, then
-// the slice table may move to global memory, in this order, until it fits.
-// Returns the bytes, or 0 if it does not fit.
+// the slice table may move to global memory, in this order, until it fits
+// (force, for tests: all of them do).  Returns the bytes, or 0 if it does not fit.
 template <class V>
-inline size_t nd_fit(const NdSizes& z, bool glob, size_t more, size_t keep, NdMem* mm) {
+inline size_t nd_fit(const NdSizes& z, bool glob, size_t more, size_t keep, NdMem* mm, bool force = false) {
     mm->slt_smem = (size_t)z.nslt * sizeof(int2) <= 16 * 1024 ? 1 : 0;
     mm->u_glob = mm->y_glob = 0;
     auto need = [&]() {
@@ -280,10 +280,10 @@ inline size_t nd_fit(const NdSizes& z, bool glob, size_t more, size_t keep, NdMe
         return (all + 15) / 16 * 16 + keep;
     };
     if (glob) {
-        if (need() > ND_SMEM_MAX) mm->u_glob = 1;
-        if (need() > ND_SMEM_MAX) mm->y_glob = 1;
-        if (need() > ND_SMEM_MAX) mm->slt_smem = 0;
-    } else if (!mm->slt_smem) {
+        if (force || need() > ND_SMEM_MAX) mm->u_glob = 1;
+        if (force || need() > ND_SMEM_MAX) mm->y_glob = 1;
+        if (force || need() > ND_SMEM_MAX) mm->slt_smem = 0;
+    } else if (force || !mm->slt_smem) {
         return 0;
     }
     mm->glob_stride = (mm->u_glob || mm->y_glob) ? nd_glob_layout(z).stride : 0;

@@ -534,7 +534,9 @@ static bool nd_memory(const thm_sys* s, bool glob, size_t more, size_t keep, NdM
     // factors of a few MB are in L2 anyway, and asking costs 1% (4 squares of
     // 24^2, order 2: 641 -> 648 ms a solve).
     mm.prefetch = m->nd.fac_elems * (int64_t)sizeof(FW) >= (int64_t)16 << 20;
-    *smem = nd_fit<V>(z, glob, more, keep, &mm);
+    // THM_BT_CPL_GLOBAL=1 runs everything from global memory that can be there
+    const char* force = getenv("THM_BT_CPL_GLOBAL");
+    *smem = nd_fit<V>(z, glob, more, keep, &mm, force && atoi(force) != 0);
     if (*smem == 0) return false;
     const size_t entries = (size_t)(mm.glob_stride * m->n_sub * m->nd.C);
     if (s->nd_glob.n < entries) s->nd_glob.alloc(entries);
