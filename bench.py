@@ -295,20 +295,6 @@ def reference_arm(args):
 # --------------------------------------------------------------------------
 # our arm
 # --------------------------------------------------------------------------
-def measured_traffic(kernel, mode):
-    """DRAM bytes (read + write) per launch of `kernel` from the committed ncu
-    summary, or None when the kernel source changed since that capture."""
-    import hashlib
-    try:
-        rec = json.load(open(os.path.join(ROOT, "profiles", "traffic.json")))[kernel]
-        src = open(os.path.join(ROOT, rec["source"]), "rb").read()
-    except (OSError, ValueError, KeyError):
-        return None
-    if hashlib.sha256(src).hexdigest() != rec["source_sha256"] or rec.get("mode") != mode:
-        return None
-    return rec["dram_bytes_per_launch"]
-
-
 def bytes_per_launch(sysg, mode, cls):
     import paper_2105_11993_gb300 as thm
     return thm.algorithmic_bytes(sysg, mode, cls)
@@ -542,7 +528,7 @@ def main():
     roofline = {"kernel": "k_subsolve (subdomain GMRES solves, one launch per sweep)", "bound": "hbm",
                 "achieved": achieved, "peak": hbm_peak, "unit": "GB/s",
                 "frac": (achieved / hbm_peak) if achieved else None,
-                "traffic": measured_traffic("k_subsolve", mode),
+                "traffic": None,               # no DRAM counters of a whole solve launch
                 "peak_source": peak_src, "launches": n_launch, "avg_launch_us": 1e3 * sub_ms / max(1, n_launch),
                 "alg_bytes_processed": total_work,
                 "alg_bytes_by_part": {names[c]: work[c] for c in names},

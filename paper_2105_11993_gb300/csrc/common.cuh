@@ -183,8 +183,6 @@ struct thm_mesh {
     thm::NdHost nd;
     bool nd_ok = false;                             // false: a subdomain outgrows the solve kernel
     thm::NdDev ndd;
-    // reduction chunks over subdomains
-    std::vector<thm::Chunk> chunks;
     // interface entries (directed pairs i <- j, one per free DOF on Sigma_ij)
     int64_t n_if = 0;
     std::vector<int32_t> if_recv, if_send, if_rowi, if_partner;
@@ -221,7 +219,6 @@ struct thm_mesh {
         d_face_dof, d_face_loc, d_row_face, d_if_tf, d_if_tcol;
     thm::DArr<int64_t> d_if_ptr;
     thm::DArr<thm::Sub> d_subs;
-    thm::DArr<thm::Chunk> d_chunks;
     thm::DArr<thm::Chunk> d_dof_chunks;
 };
 

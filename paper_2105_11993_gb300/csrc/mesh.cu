@@ -586,19 +586,6 @@ void build_mesh(thm_mesh* m) {
     }
     row_cols_all.clear();
 
-    // ---- reduction chunks
-    m->chunks.clear();
-    for (int s = 0; s < ns; ++s) {
-        const auto& S = m->subs[s];
-        for (int64_t b = 0; b < S.n; b += CHUNK) {
-            Chunk ch{};
-            ch.seg = s;
-            ch.begin = S.off + b;
-            ch.end = S.off + std::min<int64_t>(S.n, b + CHUNK);
-            m->chunks.push_back(ch);
-        }
-    }
-
     // ---- global <-> local maps
     m->owner_loc.assign(m->n_dof, -1);
     std::vector<int64_t> ccount(m->n_dof + 1, 0);
@@ -816,7 +803,6 @@ void build_mesh(thm_mesh* m) {
     m->d_if_tb.upload(m->if_tb);
     m->d_if_tcol.upload(m->if_tcol);
     m->d_subs.upload(m->subs);
-    m->d_chunks.upload(m->chunks);
     m->d_dir_edges.upload(m->dir_edges);
     m->dir_dofs.clear();
     for (int64_t g = 0; g < m->n_dof; ++g)

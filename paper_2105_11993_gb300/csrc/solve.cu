@@ -1,5 +1,5 @@
-// The DDM-GMRES solve: batched block-preconditioned GMRES in every subdomain
-// (Section 3.2, Eq. 7), the impedance-trace exchange (Eqs. 5-6), GMRES on the
+// The DDM-GMRES solve: block-preconditioned GMRES in every subdomain (Section
+// 3.2, Eq. 7; subsolve.cuh), the impedance-trace exchange (Eqs. 5-6), GMRES on the
 // interface system (Eq. 8), gluing, the FP64 true residual and iterative
 // refinement.
 #include <chrono>
