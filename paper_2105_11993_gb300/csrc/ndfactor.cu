@@ -65,45 +65,68 @@ template <> struct NdArith<double2> {
     static __device__ __forceinline__ double2 add(double2 a, double2 b) { return make_double2(a.x + b.x, a.y + b.y); }
 };
 
+// Pivot of column k: the row of the largest |col[i * ld]|, k <= i < m (lowest
+// index on ties), for the whole block; -1: it is zero, -2: not finite.
+template <class T>
+__device__ int nd_pivot(const T* col, int k, int m, int64_t ld) {
+    using A = NdArith<T>;
+    __shared__ double s_best[32];
+    __shared__ int s_at[32];
+    __shared__ int s_piv;
+    const int nt = blockDim.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    double best = -1;
+    int bi = -1;
+    for (int i = k + tid; i < m; i += nt) {
+        const double v = A::mag(col[(int64_t)i * ld]);
+        if (v > best || !(v == v)) { best = v; bi = i; }
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        const double ov = __shfl_xor_sync(0xffffffffu, best, o);
+        const int oi = __shfl_xor_sync(0xffffffffu, bi, o);
+        if (oi >= 0 && (bi < 0 || ov > best || (ov == best && oi < bi) || !(ov == ov))) { best = ov; bi = oi; }
+    }
+    if (lane == 0) { s_best[warp] = best; s_at[warp] = bi; }
+    __syncthreads();
+    if (tid == 0) {
+        for (int w = 1; w < (nt >> 5); ++w)
+            if (s_at[w] >= 0 && (bi < 0 || s_best[w] > best || (s_best[w] == best && s_at[w] < bi) || !(s_best[w] == s_best[w]))) {
+                best = s_best[w];
+                bi = s_at[w];
+            }
+        s_piv = (best > 0 && isfinite(best)) ? bi : best == 0 ? -1 : -2;
+    }
+    __syncthreads();
+    return s_piv;
+}
+
+// Undoes the row interchanges of an inversion as column interchanges, last first.
+template <class T>
+__device__ void nd_unswap(T* W, int m, int ld, const int* perm) {
+    for (int i = threadIdx.x; i < m; i += blockDim.x)
+        for (int k = m - 1; k >= 0; --k) {
+            const int p = perm[k];
+            if (p != k) {
+                const T a = W[(int64_t)i * ld + k];
+                W[(int64_t)i * ld + k] = W[(int64_t)i * ld + p];
+                W[(int64_t)i * ld + p] = a;
+            }
+        }
+    __syncthreads();
+}
+
 // In-place inverse of the m x m block W (row stride ld) by Gauss-Jordan with
 // partial pivoting, one CTA.  fcol, frow: m entries of shared memory each.
 // 0, or on a zero pivot 1, on a non-finite one 2.
 template <class T>
 __device__ int nd_invert(T* W, int m, int ld, int* perm, T* fcol, T* frow) {
     using A = NdArith<T>;
-    __shared__ double s_best[32];
-    __shared__ int s_at[32];
-    __shared__ int s_piv;
-    const int nt = blockDim.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int nt = blockDim.x, tid = threadIdx.x;
     const int di = nt / m, dj = nt % m, i0 = tid / m, j0 = tid % m;   // this thread's walk over the block
     for (int k = 0; k < m; ++k) {
-        // pivot: largest |W[i][k]|, i >= k (lowest index on ties)
-        double best = -1;
-        int bi = -1;
-        for (int i = k + tid; i < m; i += nt) {
-            const double v = A::mag(W[(int64_t)i * ld + k]);
-            if (v > best || !(v == v)) { best = v; bi = i; }
-        }
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-            const double ov = __shfl_xor_sync(0xffffffffu, best, o);
-            const int oi = __shfl_xor_sync(0xffffffffu, bi, o);
-            if (oi >= 0 && (bi < 0 || ov > best || (ov == best && oi < bi) || !(ov == ov))) { best = ov; bi = oi; }
-        }
-        if (lane == 0) { s_best[warp] = best; s_at[warp] = bi; }
-        __syncthreads();
-        if (tid == 0) {
-            for (int w = 1; w < (nt >> 5); ++w)
-                if (s_at[w] >= 0 && (bi < 0 || s_best[w] > best || (s_best[w] == best && s_at[w] < bi) || !(s_best[w] == s_best[w]))) {
-                    best = s_best[w];
-                    bi = s_at[w];
-                }
-            perm[k] = bi;
-            s_piv = (best > 0 && isfinite(best)) ? bi : best == 0 ? -1 : -2;
-        }
-        __syncthreads();
-        const int p = s_piv;
+        const int p = nd_pivot(W + k, k, m, ld);
         if (p < 0) return -p;
+        if (tid == 0) perm[k] = p;
         // row k of the result (the pivot row over the pivot) and column k, staged
         const T ip = A::inv(W[(int64_t)p * ld + k]);
         for (int j = tid; j < m; j += nt) {
@@ -125,17 +148,89 @@ __device__ int nd_invert(T* W, int m, int ld, int* perm, T* fcol, T* frow) {
         }
         __syncthreads();
     }
-    // undo the row interchanges as column interchanges, last first
-    for (int i = tid; i < m; i += nt)
-        for (int k = m - 1; k >= 0; --k) {
-            const int p = perm[k];
-            if (p != k) {
-                const T a = W[(int64_t)i * ld + k];
-                W[(int64_t)i * ld + k] = W[(int64_t)i * ld + p];
-                W[(int64_t)i * ld + p] = a;
-            }
+    nd_unswap(W, m, ld, perm);
+    return 0;
+}
+
+// The same for blocks that outgrow shared memory, NB columns at a time: the
+// panel of all m rows is eliminated in shared memory (columns contiguous), and
+// then the other columns take its NB steps at once,
+//     W_j = (W_j without the pivot rows) + X (pivot rows of W_j), X the panel,
+// so W goes through L2 m / NB times instead of m times.  What bounds it then is
+// the CTA's FP64 units (m^3 multiply-adds at 2 per clock).
+template <class T, int NB>
+__device__ __noinline__ int nd_invert_panels(T* W, int m, int ld, int* perm, T* X) {
+    using A = NdArith<T>;
+    __shared__ T s_row[NB];
+    const int nt = blockDim.x, tid = threadIdx.x;
+    // a column per thread, its rows shared out where there are fewer columns than threads
+    const int cw = min(nt, (m + 31) / 32 * 32), ng = nt / cw, grp = tid / cw, tc = tid - grp * cw;
+    for (int k0 = 0; k0 < m; k0 += NB) {
+        const int nb = min(NB, m - k0);
+        for (int t = tid; t < m * nb; t += nt) {
+            const int i = t / nb, q = t - i * nb;
+            X[q * m + i] = W[(int64_t)i * ld + k0 + q];
         }
-    __syncthreads();
+        __syncthreads();
+        for (int q = 0; q < nb; ++q) {
+            const int k = k0 + q, p = nd_pivot(X + q * m, k, m, 1);
+            if (p < 0) return -p;
+            if (tid == 0) perm[k] = p;
+            const T ip = A::inv(X[q * m + p]);
+            if (tid < nb) s_row[tid] = tid == q ? ip : A::mul(X[tid * m + p], ip);
+            __syncthreads();
+            if (p != k && tid < nb) X[tid * m + p] = X[tid * m + k];
+            __syncthreads();
+            for (int i = tid; i < m; i += nt) {
+                const T f = A::neg(X[q * m + i]);
+                for (int c = 0; c < nb; ++c)
+                    X[c * m + i] = i == k ? s_row[c] : A::fma_(f, s_row[c], c == q ? A::zero() : X[c * m + i]);
+            }
+            __syncthreads();
+        }
+        for (int c0 = 0; c0 < m; c0 += cw) {
+            const int j = c0 + tc;
+            const bool on = grp < ng && j < m && (j < k0 || j >= k0 + nb);
+            if (on && grp == 0)
+                for (int q = 0; q < nb; ++q) {
+                    const int p = perm[k0 + q];
+                    if (p == k0 + q) continue;
+                    const T a = W[(int64_t)(k0 + q) * ld + j];
+                    W[(int64_t)(k0 + q) * ld + j] = W[(int64_t)p * ld + j];
+                    W[(int64_t)p * ld + j] = a;
+                }
+            __syncthreads();
+            T t[NB];
+#pragma unroll
+            for (int q = 0; q < NB; ++q) t[q] = on && q < nb ? W[(int64_t)(k0 + q) * ld + j] : A::zero();
+            __syncthreads();
+            constexpr int U = 4;                       // rows in flight
+            if (on)
+                for (int i0 = grp * U; i0 < m; i0 += ng * U) {
+                    T v[U];
+#pragma unroll
+                    for (int u = 0; u < U; ++u) {
+                        const int i = i0 + u;
+                        v[u] = i < m && (i < k0 || i >= k0 + nb) ? W[(int64_t)i * ld + j] : A::zero();
+                    }
+#pragma unroll
+                    for (int q = 0; q < NB; ++q)
+#pragma unroll
+                        for (int u = 0; u < U; ++u)
+                            if (q < nb) v[u] = A::fma_(X[q * m + min(i0 + u, m - 1)], t[q], v[u]);
+#pragma unroll
+                    for (int u = 0; u < U; ++u)
+                        if (i0 + u < m) W[(int64_t)(i0 + u) * ld + j] = v[u];
+                }
+        }
+        __syncthreads();
+        for (int t = tid; t < m * nb; t += nt) {
+            const int i = t / nb, q = t - i * nb;
+            W[(int64_t)i * ld + k0 + q] = X[q * m + i];
+        }
+        __syncthreads();
+    }
+    nd_unswap(W, m, ld, perm);
     return 0;
 }
 
@@ -245,25 +340,63 @@ __device__ __forceinline__ int64_t nd_at(const int2* slt, int row, int col) {
     return (int64_t)slt[row >> 5].x * 128 + (col >> 2) * 128 + (row & 31) * 4 + (col & 3);
 }
 
-// out(i, j, sum_k A[i][k] B[k][j]) for an m x n product, one CTA
-template <class T, class Out>
-__device__ __forceinline__ void nd_gemm(int m, int n, int kk, const T* A, int lda, const T* B, int ldb, Out out) {
+// out(i, j, init(i, j) + sum_k A[i][k] col(j)[at(k)]) for an m x n product, one
+// CTA, the sums in the order of k.  Large products take 8 rows at a time per thread:
+// one element of B serves 8 multiply-adds, and those of A are the same for a
+// warp.  (One at a time every multiply-add waits for two loads: with the whole
+// product from L2, and the inverse a column at a time, the factorisation of 8
+// subdomains of 16^3 cells, whose roots have some 1,500 unknowns, took 7.1 s
+// instead of 3.1, of 64 such 2.6 s instead of 1.1.)
+template <class T, bool BIG, class Init, class Col, class At, class Out>
+__device__ __forceinline__ void nd_product(int m, int n, int kk, const T* A, int lda, Init init, Col col, At at, Out out) {
     using Ar = NdArith<T>;
+    constexpr int RB = 8;
+    if (BIG && m * n >= 2 * RB * (int)blockDim.x) {
+        const int mb = (m + RB - 1) / RB;
+        for (int t = threadIdx.x; t < mb * n; t += blockDim.x) {
+            const int ib = t / n, j = t - ib * n, i0 = ib * RB;
+            const T* bj = col(j);
+            const T* a[RB];
+            T c[RB];
+#pragma unroll
+            for (int r = 0; r < RB; ++r) {
+                a[r] = A + (int64_t)min(i0 + r, m - 1) * lda;
+                c[r] = init(min(i0 + r, m - 1), j);
+            }
+            for (int k = 0; k < kk; ++k) {
+                const T b = bj[at(k)];
+#pragma unroll
+                for (int r = 0; r < RB; ++r) c[r] = Ar::fma_(a[r][k], b, c[r]);
+            }
+#pragma unroll
+            for (int r = 0; r < RB; ++r)
+                if (i0 + r < m) out(i0 + r, j, c[r]);
+        }
+        return;
+    }
     for (int t = threadIdx.x; t < m * n; t += blockDim.x) {
         const int i = t / n, j = t - i * n;
-        const T* a = A + (int64_t)i * lda;
-        const T* b = B + j;
-        T c = Ar::zero();
-        for (int k = 0; k < kk; ++k) c = Ar::fma_(a[k], b[(int64_t)k * ldb], c);
+        const T *a = A + (int64_t)i * lda, *bj = col(j);
+        T c = init(i, j);
+        for (int k = 0; k < kk; ++k) c = Ar::fma_(a[k], bj[at(k)], c);
         out(i, j, c);
     }
 }
 
-// One CTA per node of a depth.  smem_s: blocks of at most that many unknowns
-// are inverted in shared memory, larger ones in place in the front.
-template <class T>
-__global__ void k_nd_factor(NdTables tab, const NdNode* __restrict__ nodes, int64_t node0, const int32_t* __restrict__ rows,
-                            const int32_t* __restrict__ cmap, const int32_t* __restrict__ childs, int C, int smem_s,
+template <class T, bool BIG, class Out>
+__device__ __forceinline__ void nd_gemm(int m, int n, int kk, const T* A, int lda, const T* B, int ldb, Out out) {
+    nd_product<T, BIG>(m, n, kk, A, lda, [](int, int) { return NdArith<T>::zero(); },
+                       [&](int j) { return B + j; }, [&](int k) { return (int64_t)k * ldb; }, out);
+}
+
+// One CTA per node of a depth.  BIG: blocks of the depth outgrow shared memory
+// (more than 160 unknowns, 113 complex); they are inverted in place in the
+// front, `panel` columns at a time (0: one), and products take 8 rows at a time.
+// (A kernel of its own: its registers would halve the CTAs per SM of the many
+// small nodes.)
+template <class T, bool BIG>
+__global__ void __launch_bounds__(512) k_nd_factor(NdTables tab, const NdNode* __restrict__ nodes, int64_t node0, const int32_t* __restrict__ rows,
+                            const int32_t* __restrict__ cmap, const int32_t* __restrict__ childs, int C, int panel,
                             int max_s, const int64_t* __restrict__ slice_ptr, const int32_t* __restrict__ col,
                             const uint8_t* __restrict__ pad, const double* __restrict__ val,
                             const double* __restrict__ bg, const double* __restrict__ bs, T* front, const T* below,
@@ -273,7 +406,7 @@ __global__ void k_nd_factor(NdTables tab, const NdNode* __restrict__ nodes, int6
     T* fcol = reinterpret_cast<T*>(smem_raw);
     T* frow = fcol + max_s;
     T* blk = frow + max_s;
-    int* perm = reinterpret_cast<int*>(blk + (smem_s > 0 ? (size_t)smem_s * smem_s : 0));
+    int* perm = reinterpret_cast<int*>(blk + (size_t)max_s * (BIG ? panel : max_s));
     const NdNode N = nodes[node0 + blockIdx.x];
     const int s = N.s, b = N.b, n = s + b, tid = threadIdx.x, nt = blockDim.x;
     const int32_t* rs = rows + N.rows0;
@@ -325,7 +458,7 @@ __global__ void k_nd_factor(NdTables tab, const NdNode* __restrict__ nodes, int6
     T* W = F;
     const T* S = F;
     int ld = n;
-    if (s <= smem_s) {
+    if (!BIG) {
         W = blk;
         ld = s;
         for (int t = tid; t < s * s; t += nt) W[t] = F[(int64_t)(t / s) * n + t % s];
@@ -334,7 +467,14 @@ __global__ void k_nd_factor(NdTables tab, const NdNode* __restrict__ nodes, int6
         S = X;
     }
     __syncthreads();
-    if (const int bad = nd_invert(W, s, ld, perm, fcol, frow)) {
+    int bad;
+    if constexpr (BIG)
+        bad = panel == 16  ? nd_invert_panels<T, 16>(W, s, ld, perm, blk)
+              : panel == 8 ? nd_invert_panels<T, 8>(W, s, ld, perm, blk)
+                           : nd_invert(W, s, ld, perm, fcol, frow);
+    else
+        bad = nd_invert(W, s, ld, perm, fcol, frow);
+    if (bad) {
         const int node = (int)(node0 + blockIdx.x);
         if (tid == 0 && bad == 2) atomicExch(&rep.status[0], 1);
         if (tid == 0 && bad == 1) rep.add(node, -1);
@@ -346,9 +486,9 @@ __global__ void k_nd_factor(NdTables tab, const NdNode* __restrict__ nodes, int6
     // u cond(S)^2 or so in W, and the Schur complements of the parents inherit
     // it (measured on 32x32 order-1 cells at omega = 4: the solve's error is
     // 6e-13 without this and the one of H below, 1.4e-14 with them).
-    nd_gemm<T>(s, s, s, S, n, W, ld, [&](int i, int j, T a) { Rs[(int64_t)i * n + j] = A::add(i == j ? A::one() : A::zero(), A::neg(a)); });
+    nd_gemm<T, BIG>(s, s, s, S, n, W, ld, [&](int i, int j, T a) { Rs[(int64_t)i * n + j] = A::add(i == j ? A::one() : A::zero(), A::neg(a)); });
     __syncthreads();
-    nd_gemm<T>(s, s, s, W, ld, Rs, n, [&](int i, int j, T a) { Y[(int64_t)i * n + j] = A::add(W[(int64_t)i * ld + j], a); });
+    nd_gemm<T, BIG>(s, s, s, W, ld, Rs, n, [&](int i, int j, T a) { Y[(int64_t)i * n + j] = A::add(W[(int64_t)i * ld + j], a); });
     __syncthreads();
     for (int t = tid; t < s * s; t += nt) W[(int64_t)(t / s) * ld + t % s] = Y[(int64_t)(t / s) * n + t % s];
     __syncthreads();
@@ -370,12 +510,12 @@ __global__ void k_nd_factor(NdTables tab, const NdNode* __restrict__ nodes, int6
     const int2* sb = tab.slt + N.slt_b;
     // H = W F_sb with a residual correction H += W (F_sb - S H)
     const T* Fb = F + s;
-    nd_gemm<T>(s, b, s, W, ld, Fb, n, [&](int i, int j, T a) { Y[(int64_t)i * n + j] = a; });
+    nd_gemm<T, BIG>(s, b, s, W, ld, Fb, n, [&](int i, int j, T a) { Y[(int64_t)i * n + j] = a; });
     __syncthreads();
-    nd_gemm<T>(s, b, s, S, n, Y, n, [&](int i, int j, T a) { Rs[(int64_t)i * n + j] = A::add(Fb[(int64_t)i * n + j], A::neg(a)); });
+    nd_gemm<T, BIG>(s, b, s, S, n, Y, n, [&](int i, int j, T a) { Rs[(int64_t)i * n + j] = A::add(Fb[(int64_t)i * n + j], A::neg(a)); });
     __syncthreads();
     double hm = 0;
-    nd_gemm<T>(s, b, s, W, ld, Rs, n, [&](int i, int j, T a) {
+    nd_gemm<T, BIG>(s, b, s, W, ld, Rs, n, [&](int i, int j, T a) {
         const T h = A::neg(A::add(Y[(int64_t)i * n + j], a));
         const double v = A::size(h);
         if (!(v <= hm)) hm = v;
@@ -383,14 +523,10 @@ __global__ void k_nd_factor(NdTables tab, const NdNode* __restrict__ nodes, int6
         fac[nd_at(sb, N.row_b + i, j)] = h;
     });
     __syncthreads();
-    for (int t = tid; t < b * b; t += nt) {
-        const int i = t / b, j = t - i * b;
-        T* d = F + (int64_t)(s + i) * n + s + j;
-        T a = *d;
-        const T* h = fac + nd_at(sf, N.row_f + s + j, 0);
-        for (int k = 0; k < s; ++k) a = A::fma_(F[(int64_t)(s + i) * n + k], h[(k >> 2) * 128 + (k & 3)], a);
-        *d = a;
-    }
+    T* U = F + (int64_t)s * n + s;
+    nd_product<T, BIG>(b, b, s, F + (int64_t)s * n, n, [&](int i, int j) { return U[(int64_t)i * n + j]; },
+                       [&](int j) { return fac + nd_at(sf, N.row_f + s + j, 0); }, [](int k) { return (k >> 2) * 128 + (k & 3); },
+                       [&](int i, int j, T a) { U[(int64_t)i * n + j] = a; });
     __shared__ double s_red[32];
     hm = nd_block_max(hm, s_red);
     if (hm <= ND_GROWTH) return;
@@ -438,6 +574,7 @@ static void append(DArr<X>& dst, const DArr<X>& base, const std::vector<X>& add,
 // at most on the inputs above, 1.06 on uniform media), and coefficients or
 // cells that show large H everywhere would fill the tree up to one dense block.
 constexpr double ND_FILL = 2;
+constexpr size_t ND_FACTOR_SMEM = 225 * 1024;      // dynamic, beside 1 KB or so of static shared memory
 constexpr int ND_PASSES = 12;               // (2 or 3 are the rule)
 
 // Builds the trees of the subdomains of `found` again with these unknowns of
@@ -539,8 +676,8 @@ static void factor(thm_sys* s, DArr<T>& fac, const char* what) {
     DArr<int2> moves;
     moves.alloc(m->n_loc + m->nd.nodes.size());
     std::vector<char> kept(m->n_sub, 0);
-    THM_CUDA(cudaFuncSetAttribute(k_nd_factor<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, 225 * 1024));
-    const size_t cap = 200 * 1024;
+    THM_CUDA(cudaFuncSetAttribute(k_nd_factor<T, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ND_FACTOR_SMEM));
+    THM_CUDA(cudaFuncSetAttribute(k_nd_factor<T, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ND_FACTOR_SMEM));
     NdHost again;                                      // the subdomains that are factorised again
     for (int passes = 0;; ++passes) {
         const bool first = passes == 0;
@@ -556,13 +693,17 @@ static void factor(thm_sys* s, DArr<T>& fac, const char* what) {
         for (int d = 0; d < nd; ++d) {
             const int64_t n0 = H.depth_node[d], cnt = H.depth_node[d + 1] - n0;
             const int ms = std::max(1, H.depth_s[d]), mn = H.depth_n[d];
-            // blocks up to smem_s in shared memory; the others of the depth in place
-            const int smem_s = (size_t)ms * ms * sizeof(T) <= cap ? ms : 0;
-            const size_t smem = (size_t)2 * ms * sizeof(T) + (size_t)smem_s * smem_s * sizeof(T) + (size_t)ms * sizeof(int);
+            const bool big = (size_t)ms * ms * sizeof(T) > 200 * 1024;
+            const size_t rest = (size_t)2 * ms * sizeof(T) + (size_t)ms * sizeof(int);
+            int panel = 0;
+            for (int w : {16, 8})                  // (8: more than 1,556 unknowns, 789 complex; 0: more than 2,742, 1,404)
+                if (big && panel == 0 && rest + (size_t)ms * w * sizeof(T) <= ND_FACTOR_SMEM) panel = w;
+            const size_t smem = rest + (size_t)ms * (big ? panel : ms) * sizeof(T);
             int threads = 32;
             while (threads < 512 && threads * 16 < mn * mn) threads *= 2;
-            THM_LAUNCH(THM_K_SETUP, st, k_nd_factor<T><<<(unsigned)cnt, threads, smem, st>>>(
-                nd_tables(s, cplx), D.nodes.p, n0, D.rows.p, D.cmap.p, D.childs.p, H.C, smem_s, ms,
+            const auto kernel = big ? k_nd_factor<T, true> : k_nd_factor<T, false>;
+            THM_LAUNCH(THM_K_SETUP, st, kernel<<<(unsigned)cnt, threads, smem, st>>>(
+                nd_tables(s, cplx), D.nodes.p, n0, D.rows.p, D.cmap.p, D.childs.p, H.C, panel, ms,
                 m->d_slice_ptr.p, m->d_sell_col.p, m->d_sell_pad.p, s->val64.p, s->bg64.p, s->bs64.p, front[d & 1].p,
                 front[(d + 1) & 1].p, aux.p, fac.p, NdReport{status.p, moves.p}));
             THM_CUDA(cudaGetLastError());
