@@ -380,6 +380,7 @@ template <class FW>
 __device__ __forceinline__ void nd_prefetch(const FW* fac, const int2* slt, int s0, int n) {
     if (n <= 0) return;
     const int64_t a = slt[s0].x, b = (int64_t)slt[s0 + n - 1].x + slt[s0 + n - 1].y;
+    if (a == b) return;                        // rows of nodes without unknowns of their own
     asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;\n" ::"l"(fac + a * 128),
                  "r"((unsigned)((b - a) * 128 * sizeof(FW)))
                  : "memory");
