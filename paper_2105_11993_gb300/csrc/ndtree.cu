@@ -450,9 +450,9 @@ bool emit_tables(const thm_mesh* m, int sub, SubTree& T, int C, NdHost& H) {
     return fits;
 }
 
-// fn(i) for i < n on several threads; the first exception comes back here.
-void parallel(int n, const std::function<void(int)>& fn) {
-    const int nt = std::max(1, std::min<int>({16, n, (int)std::thread::hardware_concurrency()}));
+// fn(i) for i < n on at most `most` threads; the first exception comes back here.
+void parallel(int n, int most, const std::function<void(int)>& fn) {
+    const int nt = std::max(1, std::min<int>({most, n, (int)std::thread::hardware_concurrency()}));
     std::atomic<int> next{0};
     std::mutex mu;
     std::exception_ptr err;
@@ -535,9 +535,13 @@ bool build_tables(const thm_mesh* m, NdHost& H, const std::vector<int>& list, in
     }
     H.C = C;
     H.mw = mw;
+    // a thread costs as much as some hundred cells take
+    size_t nc = 0;
+    for (const auto& c : cells) nc += c.size();
+    const int nt = (int)std::min<size_t>(16, 1 + nc / 512);
     std::vector<SubTree> trees(ns);
     std::vector<int32_t> cell_bin(m->n_cell, -1);         // cells belong to one subdomain each: no sharing
-    parallel(ns, [&](int i) {
+    parallel(ns, nt, [&](int i) {
         build_tree(m, list[i], std::move(cells[i]), p, moves ? &(*moves)[list[i]] : nullptr, cell_bin, trees[i]);
     });
     // node numbers: by depth, deepest first
@@ -569,7 +573,7 @@ bool build_tables(const thm_mesh* m, NdHost& H, const std::vector<int>& list, in
     // the subdomains' tables, then one behind the other
     std::vector<NdHost> part(ns);
     std::vector<char> ok(ns, 0);
-    parallel(ns, [&](int i) { ok[i] = emit_tables(m, list[i], trees[i], C, part[i]); });
+    parallel(ns, nt, [&](int i) { ok[i] = emit_tables(m, list[i], trees[i], C, part[i]); });
     std::vector<NdPlace> at(ns + 1);
     std::vector<size_t> rows0(ns + 1, 0), cmap0(ns + 1, 0), child0(ns + 1, 0);
     bool fits = true;
@@ -595,7 +599,7 @@ bool build_tables(const thm_mesh* m, NdHost& H, const std::vector<int>& list, in
     H.nodes.resize(id);
     H.rows.resize(rows0[ns]); H.cmap.resize(cmap0[ns]); H.childs.resize(child0[ns]);
     H.fac_elems = (int64_t)end.fac + 128;
-    parallel(ns, [&](int i) {
+    parallel(ns, nt, [&](int i) {
         NdHost& P = part[i];
         ok[i] = place_tables(P, at[i]);
         std::copy(P.parts.begin(), P.parts.end(), H.parts.begin() + (size_t)i * C);
