@@ -380,7 +380,8 @@ int thm_dirichlet_values(thm_sys* s, double* u_d);
  *               the subdomains' elimination trees of s^2 + 2 s b (s unknowns
  *               eliminated at the node, b unknowns of its ancestors that it
  *               couples to: the inverse block once, the coupling block on the
- *               way up and on the way down), x read + y written
+ *               way up and on the way down; of the mesh's trees, which a factorisation
+ *               may grow a little by moving unknowns up), x read + y written
  * Other classes: THM_EINVAL. */
 int thm_alg_bytes(const thm_sys* s, int mode, int cls, double* bytes);
 
@@ -432,7 +433,9 @@ int thm_residual_noalloc(const thm_sys* s, const double* u, double* out);
 /* Bytes of the stored preconditioner factors (the dense blocks of every node of
  * the subdomains' elimination trees, in slices of 32 rows padded to the widest
  * of their rows) for precond THM_PRECOND_* in mode THM_MODE_*: real values for
- * Eq. 7, complex ones for the full 2x2 block operator.  From the sizes alone (nothing is factorised by this call). */
+ * Eq. 7, complex ones for the full 2x2 block operator.  From the sizes of the
+ * mesh's trees alone (nothing is factorised by this call; a factorisation that
+ * moves unknowns up stores the blocks of those subdomains a second time). */
 int thm_factor_bytes(const thm_sys* s, int precond, int mode, double* bytes);
 
 /* Kernel launches issued by this library since the process started. */

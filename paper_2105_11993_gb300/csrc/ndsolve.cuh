@@ -13,7 +13,8 @@
 // 32x32-cell order-2 subdomain 0.38M values are multiplied instead of 1.2M
 // (dense level blocks of 130 rows) in 7 dependent steps each way and the root
 // instead of 33.  Measured against that level-by-level elimination (64 such
-// subdomains, FP64): 529 us to 210 us per apply, factorisation 28 ms to 8 ms.
+// subdomains, FP64): 529 us to 210 us per apply, factorisation 28 ms to 7 ms
+// (18 ms in the mean with what ndfactor.cu does near resonances).
 //
 // One cluster of C CTAs per subdomain: the top of the tree is one root node
 // with at least C subtrees under it, each CTA runs its subtrees alone with
