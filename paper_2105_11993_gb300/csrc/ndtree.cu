@@ -212,8 +212,8 @@ void build_tree(const thm_mesh* m, int s, std::vector<int32_t> cs, int p, const 
 
 int pad4(int v) { return (v + 3) / 4 * 4; }
 
-// Tables of one subdomain, positions within its own arrays; `nodes` in the tree's order, rows, cmap and
-// childs (node numbers) likewise.  False: an index outgrows its 16 bits.
+// Tables of one subdomain, positions within its own arrays; `nodes` in the tree's order, and childs numbered
+// in it.  False: an index outgrows its 16 bits.
 bool emit_tables(const thm_mesh* m, int sub, SubTree& T, int C, NdHost& H) {
     const int mw = m->maxc / 2;
     const auto& S = m->subs[sub];
@@ -435,13 +435,12 @@ bool emit_tables(const thm_mesh* m, int sub, SubTree& T, int C, NdHost& H) {
         D.rows0 = (int64_t)H.rows.size();
         H.rows.insert(H.rows.end(), N.s.begin(), N.s.end());
         H.rows.insert(H.rows.end(), N.b.begin(), N.b.end());
-        D.front = N.front;
         D.child0 = (int32_t)H.childs.size();
         D.nchild = (int32_t)N.ch.size();
         for (size_t i = 0; i < N.s.size(); ++i) place[N.s[i] - S.off] = (int32_t)i;
         for (size_t i = 0; i < N.b.size(); ++i) place[N.b[i] - S.off] = (int32_t)(N.s.size() + i);
         for (int c : N.ch) {
-            H.childs.push_back((int32_t)T.nodes[c].id);
+            H.childs.push_back((int32_t)c);
             H.nodes[c].cmap0 = (int64_t)H.cmap.size();
             for (int32_t r : T.nodes[c].b) H.cmap.push_back(place[r - S.off]);
         }
@@ -535,14 +534,16 @@ bool build_tables(const thm_mesh* m, NdHost& H, const std::vector<int>& list, in
     }
     H.C = C;
     H.mw = mw;
-    // a thread costs as much as some hundred cells take
     size_t nc = 0;
     for (const auto& c : cells) nc += c.size();
-    const int nt = (int)std::min<size_t>(16, 1 + nc / 512);
+    const bool big = nc >= 8192;                          // (threads cost: 1 ms for 15 of them three times)
     std::vector<SubTree> trees(ns);
     std::vector<int32_t> cell_bin(m->n_cell, -1);         // cells belong to one subdomain each: no sharing
-    parallel(ns, nt, [&](int i) {
+    std::vector<NdHost> part(ns);
+    std::vector<char> ok(ns, 0);
+    parallel(ns, big ? 16 : 8, [&](int i) {
         build_tree(m, list[i], std::move(cells[i]), p, moves ? &(*moves)[list[i]] : nullptr, cell_bin, trees[i]);
+        ok[i] = emit_tables(m, list[i], trees[i], C, part[i]);
     });
     // node numbers: by depth, deepest first
     int maxd = 0;
@@ -570,10 +571,7 @@ bool build_tables(const thm_mesh* m, NdHost& H, const std::vector<int>& list, in
         H.depth_s.push_back(ms);
         H.depth_n.push_back(mn);
     }
-    // the subdomains' tables, then one behind the other
-    std::vector<NdHost> part(ns);
-    std::vector<char> ok(ns, 0);
-    parallel(ns, nt, [&](int i) { ok[i] = emit_tables(m, list[i], trees[i], C, part[i]); });
+    // the subdomains' tables one behind the other
     std::vector<NdPlace> at(ns + 1);
     std::vector<size_t> rows0(ns + 1, 0), cmap0(ns + 1, 0), child0(ns + 1, 0);
     bool fits = true;
@@ -599,7 +597,7 @@ bool build_tables(const thm_mesh* m, NdHost& H, const std::vector<int>& list, in
     H.nodes.resize(id);
     H.rows.resize(rows0[ns]); H.cmap.resize(cmap0[ns]); H.childs.resize(child0[ns]);
     H.fac_elems = (int64_t)end.fac + 128;
-    parallel(ns, nt, [&](int i) {
+    parallel(ns, big ? 16 : 1, [&](int i) {
         NdHost& P = part[i];
         ok[i] = place_tables(P, at[i]);
         std::copy(P.parts.begin(), P.parts.end(), H.parts.begin() + (size_t)i * C);
@@ -614,12 +612,14 @@ bool build_tables(const thm_mesh* m, NdHost& H, const std::vector<int>& list, in
         std::copy(P.perm.begin(), P.perm.end(), H.perm.begin() + at[i].perm);
         std::copy(P.rows.begin(), P.rows.end(), H.rows.begin() + rows0[i]);
         std::copy(P.cmap.begin(), P.cmap.end(), H.cmap.begin() + cmap0[i]);
-        std::copy(P.childs.begin(), P.childs.end(), H.childs.begin() + child0[i]);
+        std::transform(P.childs.begin(), P.childs.end(), H.childs.begin() + child0[i],
+                       [&](int32_t q) { return (int32_t)trees[i].nodes[q].id; });
         for (size_t q = 0; q < P.nodes.size(); ++q) {
             NdNode N = P.nodes[q];
             N.rows0 += (int64_t)rows0[i];
             N.cmap0 += (int64_t)cmap0[i];
             N.child0 += (int32_t)child0[i];
+            N.front = trees[i].nodes[q].front;
             H.nodes[trees[i].nodes[q].id] = N;
         }
         P = NdHost();
